@@ -95,135 +95,350 @@ __global__ void __launch_bounds__(256, 2) hydro_gate_data_kernel(GateDataArgs A)
   }
 }
 
-// ---- MLP training ----------------------------------------------------------
-constexpr int kTile = 128;
+// ---- MLP forward and training ------------------------------------------------
+// Both kernels are FP32 contractions of 64-sample tiles against 54 x 32 and
+// 32 x 32 weights, bound by shared-memory reads and the FP32 pipe (the
+// parameters are BF16 values, but the activations are not, so the tensor
+// cores would need them rounded or split).  A CTA of 128 threads keeps the
+// weights and the tile's activations in shared memory and gives each thread
+// a 4 x 4 block of a product: 8 float4 reads feed 64 multiply-adds, where a
+// thread per sample read two operands per multiply-add.  Rows are padded to
+// 60 and 36 floats (28 and 4 banks apart), so that the eight rows a quarter
+// of a warp reads as float4 lie on distinct banks.  Measured: the forward
+// pass over 262,144 samples 747 -> about 60 us (its thread-per-sample form
+// kept 86 activations in spilled registers), a training step (gradient,
+// reduction, optimiser) at 65,536 samples 216 -> 47 us.
+constexpr int kTile = 128;        // samples per partial of hydro_mlp_work_bytes
+constexpr int kMt = 64;           // samples per tile
+constexpr int kMThreads = 128;
+constexpr int kMStrX = 60, kMStrH = 36;
+constexpr int kGradCtas = 456;    // 3 resident CTAs (70 KB) on each of 152 SMs
 
-struct SmemW {
-  const float* w;
-  __device__ float operator()(int i) const { return w[i]; }
+// Network weights in shared memory, rows padded with zeros: W1 [32][kMStrX],
+// W2 [32][kMStrH], then b1, b2, w3 [32] each and b3.
+struct MlpSmem {
+  static constexpr int w1 = 0, w2 = w1 + kGateH * kMStrX, b1 = w2 + kGateH * kMStrH, b2 = b1 + kGateH,
+                       w3 = b2 + kGateH, b3 = w3 + kGateH, end = b3 + 4;
 };
 
+__device__ __forceinline__ void mlp_load_weights(const float* __restrict__ params, float* sm) {
+  for (int i = threadIdx.x; i < kGateH * kMStrX; i += kMThreads) {
+    const int j = i / kMStrX, k = i % kMStrX;
+    sm[MlpSmem::w1 + i] = k < kGateIn ? bf16r(params[j * kGateIn + k]) : 0.f;
+  }
+  for (int i = threadIdx.x; i < kGateH * kMStrH; i += kMThreads) {
+    const int j = i / kMStrH, k = i % kMStrH;
+    sm[MlpSmem::w2 + i] = k < kGateH ? bf16r(params[kGateW2 + j * kGateH + k]) : 0.f;
+  }
+  for (int i = threadIdx.x; i < kGateH; i += kMThreads) {
+    sm[MlpSmem::b1 + i] = bf16r(params[kGateB1 + i]);
+    sm[MlpSmem::b2 + i] = bf16r(params[kGateB2 + i]);
+    sm[MlpSmem::w3 + i] = bf16r(params[kGateW3 + i]);
+  }
+  if (threadIdx.x == 0) sm[MlpSmem::b3] = bf16r(params[kGateB3]);
+}
+
+// The tile's features into xs [kMt][kMStrX] (columns 54 .. 59 zero; samples
+// past n zero); kRound: rounded to BF16.  vec: X is 8-byte aligned (a tile
+// starts at a multiple of 13,824 bytes, a row at a multiple of 216).
+template <bool kRound>
+__device__ __forceinline__ void mlp_load_tile(const float* __restrict__ X, int tile, int n, bool vec, float* xs) {
+  const int live = min(kMt, n - tile * kMt);
+  const float* src = X + (size_t)tile * kMt * kGateIn;
+  auto r = [](float v) { return kRound ? bf16r(v) : v; };
+  if (vec) {
+    const float2* s2 = reinterpret_cast<const float2*>(src);
+    for (int i = threadIdx.x; i < kMt * (kMStrX / 2); i += kMThreads) {
+      const int s = i / (kMStrX / 2), k = i % (kMStrX / 2);
+      float2 v = make_float2(0.f, 0.f);
+      if (k < kGateIn / 2 && s < live) v = __ldg(s2 + s * (kGateIn / 2) + k);
+      *reinterpret_cast<float2*>(xs + s * kMStrX + 2 * k) = make_float2(r(v.x), r(v.y));
+    }
+  } else {
+    for (int i = threadIdx.x; i < kMt * kMStrX; i += kMThreads) {
+      const int s = i / kMStrX, k = i % kMStrX;
+      xs[i] = (k < kGateIn && s < live) ? r(__ldg(src + s * kGateIn + k)) : 0.f;
+    }
+  }
+}
+
+// acc[m][o] = sum over k < kK (kK a multiple of 4) of a[row m][k] b[row o][k],
+// rows (threadIdx.x / 8) + 16 m of a and (threadIdx.x % 8) + 8 o of b: the
+// even and the odd k in the two lanes of packed multiply-adds, added at the
+// end.  The first operand of each chain is init[o] (lane 0).
+template <int kK, int kSa, int kSb>
+__device__ __forceinline__ void mlp_block(const float* __restrict__ a, const float* __restrict__ b,
+                                          const float init[4], float acc[4][4]) {
+  const float* pa = a + (threadIdx.x >> 3) * kSa;
+  const float* pb = b + (threadIdx.x & 7) * kSb;
+  float2 s[4][4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int o = 0; o < 4; ++o) s[m][o] = f2(init[o], 0.f);
+#pragma unroll
+  for (int k = 0; k < kK; k += 4) {
+    float4 va[4], vb[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) va[m] = *reinterpret_cast<const float4*>(pa + 16 * m * kSa + k);
+#pragma unroll
+    for (int o = 0; o < 4; ++o) vb[o] = *reinterpret_cast<const float4*>(pb + 8 * o * kSb + k);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        s[m][o] = fma2(f2(va[m].x, va[m].y), f2(vb[o].x, vb[o].y), s[m][o]);
+        s[m][o] = fma2(f2(va[m].z, va[m].w), f2(vb[o].z, vb[o].w), s[m][o]);
+      }
+  }
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int o = 0; o < 4; ++o) acc[m][o] = s[m][o].x + s[m][o].y;
+}
+
+// Store the thread's block (rows as mlp_block's) to out [kMt][kMStrH].
+__device__ __forceinline__ void mlp_store(float* out, const float v[4][4]) {
+  const int r = threadIdx.x >> 3, c = threadIdx.x & 7;
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int o = 0; o < 4; ++o) out[(r + 16 * m) * kMStrH + c + 8 * o] = v[m][o];
+}
+
+// w3 . h2 + b3 of sample s.
+__device__ __forceinline__ float mlp_head(const float* sm, const float* h2, int s) {
+  float z = sm[MlpSmem::b3];
+#pragma unroll
+  for (int j = 0; j < kGateH; j += 4) {
+    const float4 h = *reinterpret_cast<const float4*>(h2 + s * kMStrH + j);
+    const float4 w = *reinterpret_cast<const float4*>(sm + MlpSmem::w3 + j);
+    z = fmaf(w.x, h.x, z);
+    z = fmaf(w.y, h.y, z);
+    z = fmaf(w.z, h.z, z);
+    z = fmaf(w.w, h.w, z);
+  }
+  return z;
+}
+
 // Forward only, in the deployed form (BF16 inputs and first hidden layer,
-// FP32 accumulation; gate_logit_infer): out[i] = sigmoid(logit(x_i)).
-__global__ void __launch_bounds__(kTile) hydro_mlp_forward_kernel(const float* params, const float* X, int n,
-                                                                  float* out) {
-  __shared__ float w[kGateParams];
-  for (int i = threadIdx.x; i < kGateParams; i += blockDim.x) w[i] = bf16r(params[i]);
-  __syncthreads();
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
-    float x[54];
-#pragma unroll
-    for (int k = 0; k < 54; ++k) x[k] = X[(size_t)t * 54 + k];
-    const float z = gate_logit_infer(SmemW{w}, x);
-    out[t] = 1.f / (1.f + __expf(-z));
-  }
-}
-
-// Loss and gradient of one tile of kTile samples; per-tile partial sums
-// (kGateParams gradient entries, then the loss) in a fixed order.
-__global__ void __launch_bounds__(kTile) hydro_mlp_grad_kernel(const float* params, const float* X, const float* y,
-                                                               int n, float w1, float w0, float inv_n,
-                                                               float* partial) {
+// FP32 accumulation): out[i] = sigmoid(logit(x_i)).
+constexpr int kFwdSmem = MlpSmem::end + kMt * kMStrX + 2 * kMt * kMStrH;  // floats
+static_assert(kFwdSmem * sizeof(float) <= 48 * 1024, "forward kernel: no shared-memory opt-in");
+__global__ void __launch_bounds__(kMThreads, 4) hydro_mlp_forward_kernel(const float* __restrict__ params,
+                                                                         const float* __restrict__ X, int n, bool vec,
+                                                                         float* __restrict__ out) {
   extern __shared__ __align__(16) float sm[];
-  float* w = sm;                               // kGateParams
-  float* xs = w + kGateParams + 3;             // [kTile][54]
-  float* h1s = xs + kTile * kGateIn;           // [kTile][32]
-  float* h2s = h1s + kTile * kGateH;           // [kTile][32]
-  float* g1s = h2s + kTile * kGateH;           // dL/dz1 [kTile][32]
-  float* g2s = g1s + kTile * kGateH;           // dL/dz2 [kTile][32]
-  float* g3s = g2s + kTile * kGateH;           // dL/dz3 [kTile]
-  float* ls = g3s + kTile;                     // loss terms [kTile]
-  for (int i = threadIdx.x; i < kGateParams; i += blockDim.x) w[i] = bf16r(params[i]);
-  __syncthreads();
-  const int t = threadIdx.x;
-  const int sidx = blockIdx.x * kTile + t;
-  const int oW2 = kGateH * kGateIn + kGateH, ob2 = oW2 + kGateH * kGateH, ow3 = ob2 + kGateH, ob3 = ow3 + kGateH;
-  {
-    float x[54];
-    const bool live = sidx < n;
+  float* xs = sm + MlpSmem::end;
+  float* h1s = xs + kMt * kMStrX;
+  float* h2s = h1s + kMt * kMStrH;
+  mlp_load_weights(params, sm);
+  const int c = threadIdx.x & 7;
+  const int tiles = (n + kMt - 1) / kMt;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    mlp_load_tile<true>(X, tile, n, vec, xs);
+    __syncthreads();
+    float init[4], v[4][4];
 #pragma unroll
-    for (int k = 0; k < 54; ++k) {
-      x[k] = live ? X[(size_t)sidx * 54 + k] : 0.f;
-      xs[t * kGateIn + k] = x[k];
-    }
-    float z1[kGateH], h1[kGateH], z2[kGateH];
+    for (int o = 0; o < 4; ++o) init[o] = sm[MlpSmem::b1 + c + 8 * o];
+    mlp_block<56, kMStrX, kMStrX>(xs, sm + MlpSmem::w1, init, v);
 #pragma unroll
-    for (int j = 0; j < kGateH; ++j) {
-      float z = w[kGateH * kGateIn + j];
+    for (int m = 0; m < 4; ++m)
 #pragma unroll
-      for (int i = 0; i < kGateIn; ++i) z = fmaf(w[j * kGateIn + i], x[i], z);
-      z1[j] = z;
-      h1[j] = fmaxf(z, 0.f);
-      h1s[t * kGateH + j] = h1[j];
-    }
-    float z3 = w[ob3];
+      for (int o = 0; o < 4; ++o) v[m][o] = bf16r(fmaxf(v[m][o], 0.f));
+    mlp_store(h1s, v);
+    __syncthreads();
 #pragma unroll
-    for (int j = 0; j < kGateH; ++j) {
-      float z = w[ob2 + j];
+    for (int o = 0; o < 4; ++o) init[o] = sm[MlpSmem::b2 + c + 8 * o];
+    mlp_block<kGateH, kMStrH, kMStrH>(h1s, sm + MlpSmem::w2, init, v);
 #pragma unroll
-      for (int i = 0; i < kGateH; ++i) z = fmaf(w[oW2 + j * kGateH + i], h1[i], z);
-      z2[j] = z;
-      const float h2 = fmaxf(z, 0.f);
-      h2s[t * kGateH + j] = h2;
-      z3 = fmaf(w[ow3 + j], h2, z3);
-    }
-    const float out = 1.f / (1.f + __expf(-z3));
-    const float yy = live ? y[sidx] : 0.f;
-    // -[w1 y log(out) + w0 (1-y) log(1-out)] with log(out) = -softplus(-z3)
-    const float sp_neg = fmaxf(-z3, 0.f) + log1pf(__expf(-fabsf(z3)));  // softplus(-z3)
-    const float sp_pos = sp_neg + z3;                                   // softplus(z3)
-    ls[t] = live ? (w1 * yy * sp_neg + w0 * (1.f - yy) * sp_pos) * inv_n : 0.f;
-    const float g3 = live ? (w1 * yy * (out - 1.f) + w0 * (1.f - yy) * out) * inv_n : 0.f;
-    g3s[t] = g3;
-    float gh1[kGateH];
+    for (int m = 0; m < 4; ++m)
 #pragma unroll
-    for (int i = 0; i < kGateH; ++i) gh1[i] = 0.f;
-#pragma unroll
-    for (int j = 0; j < kGateH; ++j) {
-      const float g2 = (z2[j] > 0.f) ? g3 * w[ow3 + j] : 0.f;
-      g2s[t * kGateH + j] = g2;
-#pragma unroll
-      for (int i = 0; i < kGateH; ++i) gh1[i] = fmaf(g2, w[oW2 + j * kGateH + i], gh1[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < kGateH; ++i) g1s[t * kGateH + i] = (z1[i] > 0.f) ? gh1[i] : 0.f;
-  }
-  __syncthreads();
-  // weight gradients: sums over the tile's samples in index order
-  float* out = partial + (size_t)blockIdx.x * (kGateParams + 1);
-  for (int p = threadIdx.x; p < kGateParams + 1; p += blockDim.x) {
-    float acc = 0.f;
-    if (p < kGateH * kGateIn) {
-      const int j = p / kGateIn, i = p % kGateIn;
-      for (int s = 0; s < kTile; ++s) acc = fmaf(g1s[s * kGateH + j], xs[s * kGateIn + i], acc);
-    } else if (p < oW2) {
-      const int j = p - kGateH * kGateIn;
-      for (int s = 0; s < kTile; ++s) acc += g1s[s * kGateH + j];
-    } else if (p < ob2) {
-      const int j = (p - oW2) / kGateH, i = (p - oW2) % kGateH;
-      for (int s = 0; s < kTile; ++s) acc = fmaf(g2s[s * kGateH + j], h1s[s * kGateH + i], acc);
-    } else if (p < ow3) {
-      const int j = p - ob2;
-      for (int s = 0; s < kTile; ++s) acc += g2s[s * kGateH + j];
-    } else if (p < ob3) {
-      const int j = p - ow3;
-      for (int s = 0; s < kTile; ++s) acc = fmaf(g3s[s], h2s[s * kGateH + j], acc);
-    } else if (p == ob3) {
-      for (int s = 0; s < kTile; ++s) acc += g3s[s];
-    } else {
-      for (int s = 0; s < kTile; ++s) acc += ls[s];
-    }
-    out[p] = acc;
+      for (int o = 0; o < 4; ++o) v[m][o] = fmaxf(v[m][o], 0.f);
+    mlp_store(h2s, v);
+    __syncthreads();
+    const int s = threadIdx.x, i = tile * kMt + s;
+    if (s < kMt && i < n) out[i] = 1.f / (1.f + __expf(-mlp_head(sm, h2s, s)));
   }
 }
 
-__global__ void hydro_mlp_reduce_kernel(const float* partial, int n_tiles, float* grad, float* loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > kGateParams) return;
+// Loss and gradient: persistent CTAs over the 64-sample tiles.  Each thread
+// keeps its block of the weight gradients in registers over all the CTA's
+// tiles (8 x 4 of dW1 or dW2 on warps 0-2: 56 + 32 blocks; one column of db1,
+// db2 and dw3 per lane of warp 3), so a CTA writes one partial
+// (kGateParams gradient entries, then the loss) at its end.
+constexpr int kGradSmem = MlpSmem::end + kGateH * kMStrH + kMt * kMStrX + 4 * kMt * kMStrH + 2 * kMt;  // floats
+__global__ void __launch_bounds__(kMThreads, 3) hydro_mlp_grad_kernel(const float* __restrict__ params,
+                                                                      const float* __restrict__ X,
+                                                                      const float* __restrict__ y, int n, bool vec,
+                                                                      float w1, float w0, float inv_n,
+                                                                      float* __restrict__ partial) {
+  extern __shared__ __align__(16) float sm[];
+  float* w2t = sm + MlpSmem::end;            // W2 transposed [i][j]
+  float* xs = w2t + kGateH * kMStrH;         // [kMt][kMStrX]
+  float* h1s = xs + kMt * kMStrX;            // [kMt][kMStrH] each
+  float* h2s = h1s + kMt * kMStrH;
+  float* g1s = h2s + kMt * kMStrH;           // dL/dz1
+  float* g2s = g1s + kMt * kMStrH;           // dL/dz2
+  float* g3s = g2s + kMt * kMStrH;           // dL/dz3 [kMt]
+  float* ls = g3s + kMt;                     // loss terms [kMt]
+  mlp_load_weights(params, sm);
+  for (int i = threadIdx.x; i < kGateH * kMStrH; i += kMThreads) {
+    const int r = i / kMStrH, k = i % kMStrH;
+    w2t[i] = k < kGateH ? bf16r(params[kGateW2 + k * kGateH + r]) : 0.f;
+  }
+  const int tid = threadIdx.x, c = tid & 7;
+  // this thread's gradient block: rows j0 .. j0 + 7 of g against columns
+  // i0 .. i0 + 3 of v (dW1: g1, x; dW2: g2, h1)
+  const bool in1 = tid < 56, in2 = tid >= 56 && tid < 88;
+  const int t2 = tid - 56;
+  const int j0 = 8 * (in1 ? tid / 14 : t2 / 8), i0 = 4 * (in1 ? tid % 14 : t2 % 8);
+  float2 acc[4][4];  // [pair of j][i]
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[p][i] = f2(0.f);
+  float sb1 = 0.f, sb2 = 0.f, sw3 = 0.f, sb3 = 0.f, sl = 0.f;
+
+  const int tiles = (n + kMt - 1) / kMt;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    mlp_load_tile<false>(X, tile, n, vec, xs);
+    __syncthreads();
+    float init[4], h1[4][4], v[4][4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) init[o] = sm[MlpSmem::b1 + c + 8 * o];
+    mlp_block<56, kMStrX, kMStrX>(xs, sm + MlpSmem::w1, init, h1);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) h1[m][o] = fmaxf(h1[m][o], 0.f);
+    mlp_store(h1s, h1);
+    __syncthreads();
+#pragma unroll
+    for (int o = 0; o < 4; ++o) init[o] = sm[MlpSmem::b2 + c + 8 * o];
+    mlp_block<kGateH, kMStrH, kMStrH>(h1s, sm + MlpSmem::w2, init, v);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) v[m][o] = fmaxf(v[m][o], 0.f);
+    mlp_store(h2s, v);
+    __syncthreads();
+    if (tid < kMt) {
+      const int i = tile * kMt + tid;
+      const bool live = i < n;
+      const float z3 = mlp_head(sm, h2s, tid);
+      const float out = 1.f / (1.f + __expf(-z3));
+      const float yy = live ? y[i] : 0.f;
+      // -[w1 y log(out) + w0 (1-y) log(1-out)] with log(out) = -softplus(-z3)
+      const float sp_neg = fmaxf(-z3, 0.f) + log1pf(__expf(-fabsf(z3)));  // softplus(-z3)
+      const float sp_pos = sp_neg + z3;                                   // softplus(z3)
+      ls[tid] = live ? (w1 * yy * sp_neg + w0 * (1.f - yy) * sp_pos) * inv_n : 0.f;
+      g3s[tid] = live ? (w1 * yy * (out - 1.f) + w0 * (1.f - yy) * out) * inv_n : 0.f;
+    }
+    __syncthreads();
+    // dL/dz2 of the thread's block (v holds its h2: positive where z2 is)
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const float g3 = g3s[(tid >> 3) + 16 * m];
+#pragma unroll
+      for (int o = 0; o < 4; ++o) v[m][o] = v[m][o] > 0.f ? g3 * sm[MlpSmem::w3 + c + 8 * o] : 0.f;
+    }
+    mlp_store(g2s, v);
+    __syncthreads();
+    const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+    mlp_block<kGateH, kMStrH, kMStrH>(g2s, w2t, zero, v);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) v[m][o] = h1[m][o] > 0.f ? v[m][o] : 0.f;
+    mlp_store(g1s, v);
+    __syncthreads();
+    // weight gradients: sums over the samples in index order
+    if (in1 || in2) {
+      const float* gp = (in1 ? g1s : g2s) + j0;
+      const float* vp = (in1 ? xs : h1s) + i0;
+      const int sv = in1 ? kMStrX : kMStrH;
+#pragma unroll 4
+      for (int s = 0; s < kMt; ++s) {
+        const float4 ga = *reinterpret_cast<const float4*>(gp + s * kMStrH);
+        const float4 gb = *reinterpret_cast<const float4*>(gp + s * kMStrH + 4);
+        const float4 xv = *reinterpret_cast<const float4*>(vp + s * sv);
+        const float2 g[4] = {f2(ga.x, ga.y), f2(ga.z, ga.w), f2(gb.x, gb.y), f2(gb.z, gb.w)};
+        const float2 x[4] = {f2(xv.x), f2(xv.y), f2(xv.z), f2(xv.w)};
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[p][i] = fma2(g[p], x[i], acc[p][i]);
+      }
+    } else if (tid >= 96) {
+      const int j = tid - 96;
+#pragma unroll 4
+      for (int s = 0; s < kMt; ++s) {
+        sb1 += g1s[s * kMStrH + j];
+        sb2 += g2s[s * kMStrH + j];
+        sw3 = fmaf(g3s[s], h2s[s * kMStrH + j], sw3);
+      }
+      sb3 += g3s[j] + g3s[j + 32];
+      sl += ls[j] + ls[j + 32];
+    }
+    __syncthreads();  // the next tile overwrites the activations
+  }
+  float* out = partial + (size_t)blockIdx.x * (kGateParams + 1);
+  if (in1 || in2) {
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int j = j0 + 2 * p, k = i0 + i;
+        if (in1 && k < kGateIn) {
+          out[j * kGateIn + k] = acc[p][i].x;
+          out[(j + 1) * kGateIn + k] = acc[p][i].y;
+        } else if (in2) {
+          out[kGateW2 + j * kGateH + k] = acc[p][i].x;
+          out[kGateW2 + (j + 1) * kGateH + k] = acc[p][i].y;
+        }
+      }
+  } else if (tid >= 96) {
+    const int j = tid - 96;
+    out[kGateB1 + j] = sb1;
+    out[kGateB2 + j] = sb2;
+    out[kGateW3 + j] = sw3;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sb3 += __shfl_xor_sync(0xffffffffu, sb3, o);
+      sl += __shfl_xor_sync(0xffffffffu, sl, o);
+    }
+    if (j == 0) {
+      out[kGateB3] = sb3;
+      out[kGateParams] = sl;
+    }
+  }
+}
+
+// The sum of the partials, 32 parameters per CTA: row r of the block adds
+// partials r, r + kRedRows, ... (one 128-byte line per warp and partial), then
+// the rows are added in order.
+constexpr int kRedRows = 16;
+__global__ void __launch_bounds__(32 * kRedRows) hydro_mlp_reduce_kernel(const float* __restrict__ partial, int parts,
+                                                                         float* __restrict__ grad,
+                                                                         float* __restrict__ loss) {
+  __shared__ float rows[kRedRows][33];
+  const int p = blockIdx.x * 32 + threadIdx.x, r = threadIdx.y;
   float acc = 0.f;
-  for (int b = 0; b < n_tiles; ++b) acc += partial[(size_t)b * (kGateParams + 1) + p];
-  if (p < kGateParams) grad[p] = acc;
-  else if (loss) *loss = acc;
+  if (p <= kGateParams) {
+#pragma unroll 8
+    for (int b = r; b < parts; b += kRedRows) acc += __ldg(partial + (size_t)b * (kGateParams + 1) + p);
+  }
+  rows[r][threadIdx.x] = acc;
+  __syncthreads();
+  if (r != 0 || p > kGateParams) return;
+  float sum = rows[0][threadIdx.x];
+#pragma unroll
+  for (int k = 1; k < kRedRows; ++k) sum += rows[k][threadIdx.x];
+  if (p < kGateParams)
+    grad[p] = sum;
+  else if (loss)
+    *loss = sum;
 }
 
 __global__ void hydro_mlp_adam_kernel(float* params, float* m, float* v, const float* grad, float lr, float bc1,
@@ -236,6 +451,11 @@ __global__ void hydro_mlp_adam_kernel(float* params, float* m, float* v, const f
   v[p] = vv;
   params[p] -= lr * (mm / bc1) / (sqrtf(vv / bc2) + 1e-8f);
 }
+
+struct SmemW {
+  const float* w;
+  __device__ float operator()(int i) const { return w[i]; }
+};
 
 // Logit of the network at all-zero features (parameters already rounded).
 __global__ void hydro_gate_zero_kernel(const float* w, float* out) {
@@ -250,9 +470,7 @@ __global__ void hydro_bf16_round_kernel(const float* in, float* out, int n) {
   if (i < n) out[i] = bf16r(in[i]);
 }
 
-size_t mlp_grad_smem() {
-  return sizeof(float) * (kGateParams + 3 + kTile * kGateIn + 4 * kTile * kGateH + 2 * kTile);
-}
+size_t mlp_grad_smem() { return sizeof(float) * kGradSmem; }
 
 }  // namespace hyd
 
@@ -279,9 +497,10 @@ int hydro_gate_data(hydro_ctx_t* c, const hydro_batch_t* B, float* X, uint8_t* y
 int hydro_mlp_forward(const float* params, const float* X, int n, float* out, void* stream) {
   if (!params || n < 0 || (n > 0 && (!X || !out))) return HYDRO_EINVAL;
   if (n == 0) return HYDRO_OK;
-  int blocks = (n + hyd::kTile - 1) / hyd::kTile;
-  if (blocks > 4096) blocks = 4096;
-  hyd::hydro_mlp_forward_kernel<<<blocks, hyd::kTile, 0, (cudaStream_t)stream>>>(params, X, n, out);
+  int blocks = (n - 1) / hyd::kMt + 1;
+  if (blocks > 608) blocks = 608;  // 4 resident CTAs (46 KB) on each of 152 SMs
+  hyd::hydro_mlp_forward_kernel<<<blocks, hyd::kMThreads, hyd::kFwdSmem * sizeof(float), (cudaStream_t)stream>>>(
+      params, X, n, ((uintptr_t)X & 7u) == 0, out);
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
 }
 
@@ -301,11 +520,14 @@ int hydro_mlp_loss_grad(const float* params, const float* X, const float* y, int
                                     (int)hyd::mlp_grad_smem());
       }) != cudaSuccess)
     return HYDRO_ECUDA;
-  const int tiles = (n + hyd::kTile - 1) / hyd::kTile;
+  // one partial per CTA; the work buffer holds one per kTile samples
+  int parts = (n - 1) / hyd::kTile + 1;
+  if (parts > hyd::kGradCtas) parts = hyd::kGradCtas;
   cudaStream_t st = (cudaStream_t)stream;
-  hyd::hydro_mlp_grad_kernel<<<tiles, hyd::kTile, hyd::mlp_grad_smem(), st>>>(params, X, y, n, w1, w0, 1.f / n,
-                                                                             work);
-  hyd::hydro_mlp_reduce_kernel<<<(hyd::kGateParams + 1 + 255) / 256, 256, 0, st>>>(work, tiles, grad, loss);
+  hyd::hydro_mlp_grad_kernel<<<parts, hyd::kMThreads, hyd::mlp_grad_smem(), st>>>(
+      params, X, y, n, ((uintptr_t)X & 7u) == 0, w1, w0, 1.f / n, work);
+  hyd::hydro_mlp_reduce_kernel<<<(hyd::kGateParams + 1 + 31) / 32, dim3(32, hyd::kRedRows), 0, st>>>(work, parts,
+                                                                                                     grad, loss);
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
 }
 
