@@ -41,32 +41,63 @@ struct GateDataArgs {
   float gamma, gm1;
 };
 
-__global__ void __launch_bounds__(256, 2) hydro_gate_data_kernel(GateDataArgs A) {
-  extern __shared__ __align__(128) float Qf[];
+// The seven fields that features and labels read (rho, v, eps, tau, species),
+// as slots of the shared primitive array.
+constexpr int kLabelF = 7;
+constexpr int kLabelThreads = 512;
+
+// One CTA of 512 threads per 8^3 sub-grid (77 KB, 2 resident CTAs).  The
+// features are written as the contiguous [512][54] block they form, so that a
+// warp's stores fill whole 128-byte lines (a thread per cell wrote one value
+// to each of 32 rows of 216 bytes per store); the labels, a thread per cell,
+// are bound by FP32 issue: 13 lines x 7 fields x the limited and the central
+// pair.  A sub-grid whose padded block is one uniform state needs neither:
+// every difference is zero, so its features are 0 and its labels 0 (most of a
+// blast's mesh; the indicator's step phase skips it likewise).
+__global__ void __launch_bounds__(kLabelThreads, 2) hydro_gate_data_kernel(GateDataArgs A) {
+  extern __shared__ __align__(128) float Qf[];  // [kLabelF][S3]
+  __shared__ int off[kGateIn];                  // feature j's neighbour relative to the cell (field included)
+  for (int j = threadIdx.x; j < kGateIn; j += kLabelThreads) off[j] = c_gate_off.off[j];
   for (int s = blockIdx.x; s < A.n_sub; s += gridDim.x) {
     const double* Us = A.U + (size_t)s * F * S3;
-    for (int c = threadIdx.x; c < S3; c += blockDim.x) {
+    for (int c = threadIdx.x; c < S3; c += kLabelThreads) {
       double u[F];
 #pragma unroll
-      for (int k = 0; k < F; ++k) u[k] = __ldg(Us + (size_t)k * S3 + c);
+      for (int k = 0; k < F; ++k) u[k] = (k == ZX || k == ZY || k == ZZ) ? 0.0 : __ldg(Us + (size_t)k * S3 + c);
       float q[F];
       prims_mixed(u, A.eta1, A.gamma, q);
 #pragma unroll
-      for (int k = 0; k < F; ++k) Qf[k * S3 + c] = q[k];
+      for (int k = 0; k < kLabelF; ++k) Qf[k * S3 + c] = q[k < ZX ? k : SP0];
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < N3; i += blockDim.x) {
-      const int x = i & (N - 1), yy = (i >> 3) & (N - 1), z = i >> 6;
-      const int c = ((z + G) * S + (yy + G)) * S + (x + G);
-      const size_t cell = (size_t)s * N3 + i;
-      if (A.X) {
-        float f[54];
-        gate_features(Qf, c, A.gm1, f);
+    bool same = Qf[RHO * S3] > 1e-30f && A.gm1 * Qf[EGAS * S3] > 1e-30f;  // 0 / subnormal is left to the division
+    for (int c = threadIdx.x; c < S3; c += kLabelThreads)
 #pragma unroll
-        for (int k = 0; k < 54; ++k) A.X[cell * 54 + k] = f[k];
+      for (int k = 0; k < kLabelF; ++k) {
+        const float d = Qf[k * S3 + c] - Qf[k * S3];  // NaN for infinities
+        same &= d == 0.f;
       }
-      if (A.y) {
-        bool fired = false;
+    const bool uniform = __syncthreads_and(same);
+    if (A.X) {
+      float* X = A.X + (size_t)s * N3 * kGateIn;
+      for (int e = threadIdx.x; e < N3 * kGateIn; e += kLabelThreads) {
+        float v = 0.f;
+        if (!uniform) {
+          const int i = e / kGateIn, j = e - i * kGateIn;
+          const int c = (((i >> 6) + G) * S + (((i >> 3) & (N - 1)) + G)) * S + ((i & (N - 1)) + G);
+          const float q0 = Qf[(j < 27 ? RHO : EGAS) * S3 + c], q1 = Qf[c + off[j]];
+          const float qc = j < 27 ? q0 : A.gm1 * q0, qk = j < 27 ? q1 : A.gm1 * q1;
+          v = __fdividef(qk - qc, fabsf(qk) + fabsf(qc));
+        }
+        X[e] = v;
+      }
+    }
+    if (A.y) {
+      const int i = threadIdx.x;
+      static_assert(kLabelThreads == N3, "a thread per cell");
+      const int c = (((i >> 6) + G) * S + (((i >> 3) & (N - 1)) + G)) * S + ((i & (N - 1)) + G);
+      bool fired = false;
+      if (!uniform) {
         // scales: |q0| for density, eps, tau, species; |v| + c for velocity
         const float rho0 = Qf[RHO * S3 + c], eps0 = Qf[EGAS * S3 + c];
         const float vs = fabsf(Qf[SX * S3 + c]) + fabsf(Qf[SY * S3 + c]) + fabsf(Qf[SZ * S3 + c]) +
@@ -81,15 +112,14 @@ __global__ void __launch_bounds__(256, 2) hydro_gate_data_kernel(GateDataArgs A)
               if (dz == 0 && (dy < 0 || (dy == 0 && dx <= 0))) continue;
               const int st = (dz * S + dy) * S + dx;
 #pragma unroll
-              for (int k = 0; k < F; ++k) {
-                if (k == ZX || k == ZY || k == ZZ) continue;  // spin: always limited, never labelled
+              for (int k = 0; k < kLabelF; ++k) {  // the spin: always limited, never labelled
                 const float* q = Qf + k * S3 + c;
                 const float scale = (k >= SX && k <= SZ) ? vs : fabsf(q[0]);
                 fired |= ppm32_significant(q[-2 * st], q[-st], q[0], q[st], q[2 * st], scale);
               }
             }
-        A.y[cell] = fired ? 1 : 0;
       }
+      A.y[(size_t)s * N3 + i] = fired ? 1 : 0;
     }
     __syncthreads();
   }
@@ -481,7 +511,7 @@ int hydro_gate_data(hydro_ctx_t* c, const hydro_batch_t* B, float* X, uint8_t* y
   if (c->N != hyd::N) return HYDRO_EUNSUP;
   if (B->n_sub == 0) return HYDRO_OK;
   if (!B->U) return HYDRO_EINVAL;
-  const size_t smem = (size_t)hyd::F * hyd::S3 * sizeof(float);
+  const size_t smem = (size_t)hyd::kLabelF * hyd::S3 * sizeof(float);
   static unsigned long long attr = 0;
   if (hyd::once_per_device(&attr, [smem] {
         return cudaFuncSetAttribute(hyd::hydro_gate_data_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -490,7 +520,7 @@ int hydro_gate_data(hydro_ctx_t* c, const hydro_batch_t* B, float* X, uint8_t* y
     return HYDRO_ECUDA;
   hyd::GateDataArgs A{B->U, X, y, B->n_sub, c->mode.de_eta1, (float)c->gamma, (float)(c->gamma - 1.0)};
   const int grid = B->n_sub < 2 * c->num_sms ? B->n_sub : 2 * c->num_sms;
-  hyd::hydro_gate_data_kernel<<<grid, 256, smem, (cudaStream_t)stream>>>(A);
+  hyd::hydro_gate_data_kernel<<<grid, hyd::kLabelThreads, smem, (cudaStream_t)stream>>>(A);
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
 }
 

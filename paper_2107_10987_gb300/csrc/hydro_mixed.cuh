@@ -375,24 +375,6 @@ __device__ __forceinline__ bool prims_mixed(const double u[F], double eta1, floa
   return (rho > 0.0) && (eps > 0.f);
 }
 
-// Indicator features of cell c (54: density then pressure over the 3x3x3
-// neighbourhood in (z, y, x) order): (q_k - q_c) / (|q_k| + |q_c|).
-__device__ __forceinline__ void gate_features(const float* __restrict__ Q, int c, float gm1, float x[54]) {
-  const float rc = Q[RHO * S3 + c], pc = gm1 * Q[EGAS * S3 + c];
-  int j = 0;
-#pragma unroll
-  for (int dz = -1; dz <= 1; ++dz)
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx, ++j) {
-        const int ck = c + (dz * S + dy) * S + dx;
-        const float rk = Q[RHO * S3 + ck], pk = gm1 * Q[EGAS * S3 + ck];
-        x[j] = __fdividef(rk - rc, fabsf(rk) + fabsf(rc));
-        x[27 + j] = __fdividef(pk - pc, fabsf(pk) + fabsf(pc));
-      }
-}
-
 // Indicator network: 54 -> 32 (ReLU) -> 32 (ReLU) -> 1 (logit).  Parameters
 // packed W1[32][54], b1[32], W2[32][32], b2[32], w3[32], b3.
 constexpr int kGateIn = 54, kGateH = 32;
