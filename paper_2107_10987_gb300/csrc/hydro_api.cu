@@ -12,9 +12,11 @@
 
 namespace hyd {
 cudaError_t launch_step_mixed_amr(const StepArgs64& A, const AMRArgs& M, int grid, cudaStream_t st);
-cudaError_t launch_step_fp64_lines(const StepArgs64& A, int grid, int nn, cudaStream_t st);
+cudaError_t launch_step_fp64_lines(const StepArgs64& A, int teams, int T, unsigned* sync, int nn, cudaStream_t st);
 cudaError_t prepare_step_fp64_lines();
-size_t step_fp64_lines_per_cta();
+size_t step_fp64_lines_per_team();
+size_t step_fp64_lines_sync_words(int teams);
+int step_fp64_choose_team(int units, int num_sms, int face_points);
 cudaError_t launch_step_mixed(const StepArgs64& A, int grid, int planes, int nn, cudaStream_t st);
 cudaError_t prepare_step_fp64();
 cudaError_t prepare_step_mixed();
@@ -109,13 +111,23 @@ static int step_slots(const hydro_ctx* c, bool mixed) {
   return 2 * c->num_sms;
 }
 
-// The FP64 step's per-CTA line-end buffers for its persistent grid over
-// `units` tiles (2.08 MB per CTA).
+// The FP64 step's launch over `units` tiles: teams of *T CTAs each.  A grid
+// fixed by the caller or the autotuner is that many single CTAs.
+static int fp64_teams(const hydro_ctx* c, int units, int* T) {
+  *T = c->slots_tuned[0] > 0 ? 1 : hyd::step_fp64_choose_team(units, c->num_sms, c->mode.flux_points);
+  const int most = c->slots_tuned[0] > 0 ? c->slots_tuned[0] : c->num_sms / *T;
+  return units < most ? units : most;
+}
+
+// Its per-team buffers (2.94 MB each) and the teams' barrier words.
 static int ensure_lines(hydro_ctx* c, int units) {
-  const int slots = step_slots(c, false);
-  const int grid = units < slots ? units : slots;
-  return ensure_buf(c, &c->lines, &c->lines_bytes, (size_t)grid * hyd::step_fp64_lines_per_cta() * sizeof(double),
-                    "cudaMalloc(FP64 line ends)");
+  int T = 1;
+  const int teams = fp64_teams(c, units, &T);
+  int rc = ensure_buf(c, &c->lines, &c->lines_bytes, (size_t)teams * hyd::step_fp64_lines_per_team() * sizeof(double),
+                      "cudaMalloc(FP64 line ends)");
+  if (rc || T == 1) return rc;
+  return ensure_buf(c, &c->sync, &c->sync_bytes, hyd::step_fp64_lines_sync_words(teams) * sizeof(unsigned),
+                    "cudaMalloc(FP64 team barriers)");
 }
 
 static hyd::StepArgs64 step_args(const hydro_ctx* c, const hydro_batch_t* B, double* dUdt, double* amax,
@@ -315,20 +327,25 @@ int hydro_step(hydro_ctx_t* c, const hydro_batch_t* B, double dt, double* dUdt, 
   const bool mixed = c->mode.precision == HYDRO_PREC_MIXED;
   int rc = ensure_status(c);
   if (rc) return rc;
-  const int slots = step_slots(c, mixed);
   const int units = step_units(c, B->n_sub);
-  const int grid = units < slots ? units : slots;
-  rc = ensure_buf(c, &c->scratch, &c->scratch_bytes, (size_t)grid * hyd::kScratchPerSub * sizeof(double),
-                  "cudaMalloc(step scratch)");
-  if (rc) return rc;
-  if (!mixed) {
+  cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e;
+  if (mixed) {
+    const int slots = step_slots(c, mixed);
+    const int grid = units < slots ? units : slots;
+    rc = ensure_buf(c, &c->scratch, &c->scratch_bytes, (size_t)grid * hyd::kScratchPerSub * sizeof(double),
+                    "cudaMalloc(step scratch)");
+    if (rc) return rc;
+    e = hyd::launch_step_mixed(step_args(c, B, dUdt, amax, face_flux), grid, eff_decomp(c) == HYDRO_DECOMP_PLANES,
+                               c->N, st);
+  } else {
     rc = ensure_lines(c, units);
     if (rc) return rc;
+    int T = 1;
+    const int teams = fp64_teams(c, units, &T);
+    e = hyd::launch_step_fp64_lines(step_args(c, B, dUdt, amax, face_flux), teams, T,
+                                    reinterpret_cast<unsigned*>(c->sync), c->N, st);
   }
-  const hyd::StepArgs64 A = step_args(c, B, dUdt, amax, face_flux);
-  cudaError_t e = mixed ? hyd::launch_step_mixed(A, grid, eff_decomp(c) == HYDRO_DECOMP_PLANES, c->N,
-                                                  (cudaStream_t)stream)
-                        : hyd::launch_step_fp64_lines(A, grid, c->N, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "hydro_step");
   return HYDRO_OK;
 }
@@ -369,6 +386,7 @@ int hydro_autotune_step(hydro_ctx_t* c, const hydro_batch_t* B, double* dUdt, do
     const int units = step_units(c, B->n_sub);
     const int rounds = (units + maxs - 1) / maxs;
     cand[nc++] = {HYDRO_DECOMP_ROWS, (units + rounds - 1) / rounds};
+    if (!mixed) cand[nc++] = {HYDRO_DECOMP_ROWS, 0};  // the default's teams
   }
   if (planes_ok) {
     const int maxs = c->num_sms;
@@ -405,7 +423,7 @@ int hydro_autotune_step(hydro_ctx_t* c, const hydro_batch_t* B, double* dUdt, do
     c->decomp = decomp0;
     c->slots_tuned[idx] = 0;
   }
-  if (slots_out) *slots_out = c->slots_tuned[idx];
+  if (slots_out) *slots_out = rc == HYDRO_OK ? step_slots(c, mixed) : 0;
   return rc;
 }
 

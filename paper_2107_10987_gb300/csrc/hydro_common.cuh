@@ -106,7 +106,7 @@ struct StepArgs64 {
   double* amax;
   double* face_flux;  // optional [n_sub][6][DQ][N][N] boundary-face sums (null: none)
   double* scratch;  // per-CTA scratch, kScratchPerSub doubles per CTA
-  double* lines;    // FP64 step with every line once: per-CTA line ends (null for the other kernels)
+  double* lines;    // FP64 step with every line once: per-team buffers (null for the other kernels)
   unsigned* status;
   int n_sub;
   StepParams P;
@@ -225,6 +225,34 @@ __device__ __forceinline__ double warp_max(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
+}
+
+// ---- bounded inter-CTA waits ---------------------------------------------
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+// Wait until *p >= target.  Gives up (false) after limit_ns of polling, after
+// 2^26 polls whatever the clock says, or as soon as *abort is set.
+static __device__ bool wait_geq(const unsigned* p, unsigned target, const unsigned* abort, long long limit_ns) {
+  if (ld_acquire(p) >= target) return true;
+  const unsigned long long t0 = global_ns();
+  for (long i = 0; i < (1l << 26); ++i) {
+    __nanosleep(128);
+    if (ld_acquire(p) >= target) return true;
+    if (ld_acquire(abort) != 0u) return false;
+    if ((long long)(global_ns() - t0) > limit_ns) return false;
+  }
+  return false;
 }
 
 // ---- host: once-per-device set-up -------------------------------------

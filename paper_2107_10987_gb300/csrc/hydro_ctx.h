@@ -18,7 +18,7 @@ struct hydro_ctx {
   unsigned* status;      // device word
   double* scratch;       // step scratch
   size_t scratch_bytes;
-  double* lines;         // FP64 step: per-CTA line ends
+  double* lines;         // FP64 step: per-team line ends, face sums and primitives
   size_t lines_bytes;
   double* part;          // conservation partials
   size_t part_bytes;
@@ -30,7 +30,8 @@ struct hydro_ctx {
   size_t u2_bytes;
   double* prims;         // fused RK3 step: 2 x [n_sub][F][N^3] FP32 primitives (float words)
   size_t prims_bytes;
-  double* sync;          // fused RK3 step: barrier, work counter and per-sub-grid flags (unsigned words)
+  double* sync;          // fused RK3 step: barrier, work counter and per-sub-grid flags; FP64 step: team
+                         // barriers (unsigned words, cleared by each launch that uses them)
   size_t sync_bytes;
   double* amr_img;       // adaptive RK3 step: each leaf's restriction image [n_sub][F][(N/2)^3]
   size_t amr_img_bytes;

@@ -8,72 +8,78 @@
 
 namespace hyd {
 
-// Smaller of two non-negative doubles: their bit patterns order like their
-// values, so an integer minimum gives fmin's result on the integer pipes
-// (GB300 issues FP64 at 1/64 of the FP32 rate).
-__device__ __forceinline__ double min_nonneg(double x, double y) {
-  const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
-  return __longlong_as_double(a < b ? a : b);
+// ---- magnitudes as integers -------------------------------------------------
+// The bit patterns of non-negative doubles order like their values, so minima
+// and comparisons of magnitudes, doublings, halvings and signs run on the
+// integer pipes (GB300 issues FP64 at 1/64 of the FP32 rate).  The masks are
+// written as integer instructions: as |x| or -x of a double the compiler
+// spends an FP64 addition on each.
+__device__ __forceinline__ long long mag64(double x) {
+  long long r;
+  asm("and.b64 %0, %1, 0x7fffffffffffffff;" : "=l"(r) : "l"(__double_as_longlong(x)));
+  return r;
 }
+// The magnitude m with the sign bit of x (of -x: neg).
+__device__ __forceinline__ double sign64(long long m, double x, bool neg = false) {
+  long long s;
+  asm("and.b64 %0, %1, 0x8000000000000000;" : "=l"(s) : "l"(__double_as_longlong(x)));
+  return __longlong_as_double(m | (neg ? s ^ (long long)0x8000000000000000ull : s));
+}
+// x, or -x
+__device__ __forceinline__ double flip64(double x, bool neg) {
+  long long r;
+  asm("xor.b64 %0, %1, %2;" : "=l"(r) : "l"(__double_as_longlong(x)), "l"(neg ? (long long)0x8000000000000000ull : 0ll));
+  return __longlong_as_double(r);
+}
+__device__ __forceinline__ long long min64(long long a, long long b) { return a < b ? a : b; }
 
 __device__ __forceinline__ double max_nonneg(double x, double y) {
   const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
   return __longlong_as_double(a > b ? a : b);
 }
 
-// An integer that orders like the double (for non-NaN values; -0 sorts just
-// below +0).  x > y with y >= +0, and x < -y with y >= +0 (-y <= -0), give the
-// IEEE results through these keys: the two cases where the key order and
-// IEEE disagree, -0 against +0, then both answer false as IEEE does.
-__device__ __forceinline__ long long order_key(double x) {
-  const long long b = __double_as_longlong(x);
-  return b >= 0 ? b : (b ^ 0x7fffffffffffffffLL);
-}
+// 2x for a finite double of magnitude pattern b, exactly: a normal one gains
+// one in the exponent field, a subnormal one (exponent field 0) doubles its
+// pattern, which carries into the exponent field where 2x is normal.
+__device__ __forceinline__ long long twice_mag(long long b) { return b < (1LL << 52) ? b + b : b + (1LL << 52); }
 
-// 2x for a finite double x >= 0, exactly: a normal x gains one in the
-// exponent field, a subnormal x (exponent field 0) doubles its pattern, which
-// carries into the exponent field where 2x is normal.
-__device__ __forceinline__ double twice_nonneg(double x) {
-  const long long b = __double_as_longlong(x);
-  return __longlong_as_double(b < (1LL << 52) ? b + b : b + (1LL << 52));
+// Half a magnitude as the FP64 product 0.5 x rounds it (to nearest, ties to
+// even): with the exponent field at least 2 the result is normal and the field
+// drops by one (infinities and NaNs pass unchanged); below that the pattern is
+// the significand with its implicit bit (field 1) or without (zero,
+// subnormals), and half of it, rounded to even, is the result's pattern (a
+// carry into bit 52 is the smallest normal, correctly encoded).
+__device__ __forceinline__ long long half_mag(long long mag) {
+  if (mag >= (2LL << 52)) return mag < (0x7ffLL << 52) ? mag - (1LL << 52) : mag;
+  return (mag >> 1) + (mag & (mag >> 1) & 1LL);
 }
+__device__ __forceinline__ double half64(double x) { return sign64(half_mag(mag64(x)), x); }
 
 // x <= 0 for a non-NaN double: +0 has the bit pattern 0 and every value with
 // the sign bit set (-0 and the negatives) is negative as a signed integer.
 __device__ __forceinline__ bool nonpositive(double x) { return __double_as_longlong(x) <= 0LL; }
 
-// x / 2 exactly as the FP64 product 0.5 x rounds it (to nearest, ties to
-// even), on the integer pipes: with the exponent field at least 2 the result
-// is normal and the field drops by one (infinities and NaNs pass unchanged);
-// below that the magnitude's bit pattern is the significand with its
-// implicit bit (field 1) or without (zero, subnormals), and half of it,
-// rounded to even, is the result's pattern (a carry into bit 52 is the
-// smallest normal, correctly encoded).
-__device__ __forceinline__ double half64(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned long long sign = b & 0x8000000000000000ull, mag = b ^ sign;
-  unsigned long long r;
-  if (mag >= (2ull << 52))
-    r = mag < (0x7ffull << 52) ? mag - (1ull << 52) : mag;
-  else
-    r = (mag >> 1) + (mag & (mag >> 1) & 1ull);
-  return __longlong_as_double((long long)(r | sign));
+// Whether two doubles differ in sign bit.
+__device__ __forceinline__ bool signs_differ(double x, double y) {
+  return (__double2hiint(x) ^ __double2hiint(y)) < 0;
 }
 
 // MC-limited slope of sample j from delta_{j-1} = a and delta_j = b:
-// 0 if a b <= 0, else sgn(b) min(2|a|, 2|b|, |a + b|/2).  The product test is
-// the FP64 product, compared on its bit pattern; min(2|a|, 2|b|) =
-// 2 min(|a|, |b|) exactly, the minima of non-negative values are taken and
-// the doubling and halving done on the bit patterns, and with a b > 0 the
-// sign of the result is the sign bit of b: the same bits as the FP64
-// multiplications, fmin and comparisons, with 2 instead of 9 FP64
-// instructions.  (An integer form of the product test, exact but for a
-// fallback near the underflow threshold, measured slower.)
+// 0 if a b <= 0 (the FP64 product), else sgn(b) min(2|a|, 2|b|, |a + b|/2).
+// The product is not formed: with both factors nonzero and of one sign it is
+// positive unless it underflows, which needs a subnormal factor or exponent
+// fields adding up to less than 972 (it is at least 2^-1074 otherwise), and
+// only there the FP64 product decides.
+// min(2|a|, 2|b|) = 2 min(|a|, |b|) exactly, the minima, the doubling and the
+// halving are taken on the bit patterns, and the sign of the result is the
+// sign bit of b: the same bits as the FP64 operations, with one FP64
+// instruction (a + b) instead of ten.
 __device__ __forceinline__ double slope64(double a, double b) {
-  if (nonpositive(rmul(a, b))) return 0.0;
-  const double m = min_nonneg(twice_nonneg(min_nonneg(fabs(a), fabs(b))), half64(fabs(radd(a, b))));
-  const long long sign = __double_as_longlong(b) & (long long)0x8000000000000000ull;
-  return __longlong_as_double(__double_as_longlong(m) | sign);
+  const long long ma = mag64(a), mb = mag64(b), lo = min64(ma, mb);
+  if (signs_differ(a, b) || lo == 0LL) return 0.0;
+  const unsigned ea = (unsigned)(ma >> 52), eb = (unsigned)(mb >> 52);
+  if ((ea + eb < 972u || lo < (1LL << 52)) && nonpositive(rmul(a, b))) return 0.0;
+  return sign64(min64(twice_mag(lo), half_mag(mag64(radd(a, b)))), b);
 }
 
 // The unlimited PPM interface value between samples sa and sb (in the line's
@@ -81,8 +87,7 @@ __device__ __forceinline__ double slope64(double a, double b) {
 // +d value of a cell and the -d value of its +d neighbour are the same
 // number, so a sweep along the line may compute it once for both.
 __device__ __forceinline__ double ppm_iface64(double sa, double sb, double Da, double Db) {
-  const double sixth = 1.0 / 6.0;
-  return rsub(half64(radd(sa, sb)), rmul(rsub(Db, Da), sixth));
+  return fma(-1.0 / 6.0, rsub(Db, Da), half64(radd(sa, sb)));
 }
 
 // Contact steepening of the interface values p (+d) and m (-d) of the
@@ -98,22 +103,29 @@ __device__ __forceinline__ void ppm_steep64(double s1, double s3, double D0, dou
 // The monotonicity fix-ups of PPM on the interface values p (+d) and m (-d)
 // of the cell value s2: a local extremum flattens the cell, an interface
 // value that would put the parabola's extremum inside the cell is moved to
-// 3 s2 - 2 (the other one).
+// 3 s2 - 2 (the other one).  With u = p - s2 and w = s2 - m, an extremum is
+// u w <= 0, and of one sign the parabola test (p - m)(s2 - (p + m)/2) against
+// +-(p - m)^2/6 reads |w| > 2|u| (m moves to s2 - 2u) and |u| > 2|w| (p moves
+// to s2 + 2w): sign bits and comparisons of bit patterns, so two FP64
+// instructions and one in a cell that moves, instead of nine and three.  The
+// limited values are continuous where the tests switch.
 __device__ __forceinline__ void ppm_limit64(double s2, double& p, double& m) {
-  const double sixth = 1.0 / 6.0;
-  if (nonpositive(rmul(rsub(p, s2), rsub(s2, m)))) {
+  const double u = rsub(p, s2), w = rsub(s2, m);
+  const long long au = mag64(u), aw = mag64(w);
+  if (signs_differ(u, w) || min64(au, aw) == 0LL) {
     p = s2;
     m = s2;
-  } else {
-    const double dq = rsub(p, m);
-    const double lhs = rmul(dq, rsub(s2, half64(radd(p, m))));
-    const double rhs = rmul(rmul(dq, dq), sixth);  // >= +0
-    const long long kl = order_key(lhs);
-    if (kl > order_key(rhs)) {
-      m = rsub(rmul(3.0, s2), rmul(2.0, p));
-    } else if (kl < order_key(-rhs)) {
-      p = rsub(rmul(3.0, s2), rmul(2.0, m));
-    }
+    return;
+  }
+  const long long au2 = twice_mag(au), aw2 = twice_mag(aw);
+  const bool mm = aw > au2, mp = au > aw2;
+  if (mm || mp) {
+    // s2 - 2u or s2 + 2w (w has u's sign)
+    const double r = radd(s2, sign64(mm ? au2 : aw2, u, mm));
+    if (mm)
+      m = r;
+    else
+      p = r;
   }
 }
 
@@ -211,38 +223,27 @@ __device__ __forceinline__ void line10u(const double* __restrict__ Q, int c, int
   }
 }
 
-// Physical side state at a quadrature point: conserved U, the normal
-// velocity u_n and the a-component v_a of v, the pressure p and the signal
-// speed |u_n| + c.  u = v - omega z_hat x x_q (rotating frame), so u_n is one
-// FMA of the selected components (exactly v_z along z).
-__device__ __forceinline__ void side64(const double q[F], int a, double xq, double yq, const StepParams& P,
-                                       double U[F], double& un, double& va, double& p, double& spd) {
-  const double rho = q[RHO], vx = q[1], vy = q[2], vz = q[3], eps = q[4];
-  const double ek = half64(rho) * ((vx * vx + vy * vy) + vz * vz);
-  p = P.gm1 * eps;
-  // c = sqrt(gamma p / rho) = gamma p / sqrt(gamma p rho): one reciprocal
-  // square root instead of a division and a square root (a few ulps from the
-  // correctly rounded value); c = 0 where p <= 0 (a non-physical state)
-  const double gp = P.gamma * p;
-  const double c = (__double_as_longlong(gp) <= 0LL) ? 0.0 : gp * rsqrt(gp * rho);
-  va = (a == 0) ? vx : (a == 1) ? vy : vz;
-  const double om = (a == 0) ? P.omega : (a == 1) ? -P.omega : 0.0;
-  const double r = (a == 0) ? yq : (a == 1) ? xq : 0.0;
-  un = fma(om, r, va);
-  U[RHO] = rho;
-  U[SX] = rho * vx;
-  U[SY] = rho * vy;
-  U[SZ] = rho * vz;
-  U[EGAS] = eps + ek;
-#pragma unroll
-  for (int k = TAU; k < F; ++k) U[k] = q[k];
-  spd = fabs(un) + c;
+// What the flux needs of a reconstructed state besides its fields: the
+// pressure p, the energy E = eps + rho |v|^2 / 2 and the sound speed.
+// c = sqrt(gamma p / rho) = gamma p / sqrt(gamma p rho): one reciprocal square
+// root instead of a division and a square root (a few ulps from the correctly
+// rounded value); c = 0 where p <= 0 (a non-physical state).  A state is the
+// end of one line and serves up to three faces, so a kernel that keeps line
+// ends keeps these with them.
+struct End64 {
+  double p, E, c;
+};
+__device__ __forceinline__ End64 end64(double rho, double vx, double vy, double vz, double eps, const StepParams& P) {
+  End64 e;
+  e.p = rmul(P.gm1, eps);
+  e.E = fma(half64(rho), fma(vz, vz, fma(vy, vy, rmul(vx, vx))), eps);
+  const double gp = rmul(P.gamma, e.p);
+  e.c = (__double_as_longlong(gp) <= 0LL) ? 0.0 : rmul(gp, rsqrt(rmul(gp, rho)));
+  return e;
 }
 
-// d x g for an integer vector d with components in {-1, 0, 1}: each term is
-// +-g_i or zero, taken by sign selection, so one FP64 subtraction per
-// component.
-__device__ __forceinline__ double signed_pick(int d, double x) { return d == 0 ? 0.0 : (d > 0 ? x : -x); }
+// d x for an integer d in {-1, 0, 1}, by sign selection.
+__device__ __forceinline__ double signed_pick(int d, double x) { return d == 0 ? 0.0 : flip64(x, d < 0); }
 
 // Spin feedback at a cell's point x_c + (h/2) d: the velocity there of the
 // cell's rigid rotation omega = z / I, I = rho h^2 / 6 (a uniform cube about
@@ -267,62 +268,95 @@ __device__ __forceinline__ void spin_dv64(double rho, double eps, double zx, dou
   dv[2] = rmul(k, rsub(signed_pick(dy, zx), signed_pick(dx, zy)));
 }
 
-// Kurganov-Tadmor flux at one point with half its Simpson weight hw = w/2:
-//   w F_q = hw (F_L + F_R) - hw a_q (U_R - U_L),  F = U u_n (+ p e_a, + p v_a),
-// accumulated per field into the face sum (F_L + F_R as two fused products,
-// the weight folded into the fused accumulation).  The point lies at
-// x_L + (h/2) d from the left cell's centre (integer d, d_a = 1); the torque
-// sum T accumulates d x (w F_q) of the momentum flux, so that the face's
-// torque about the left centre is (h/2) T and about the right centre (at
-// x_L + h e_a) (h/2) T - h e_a x (sum of w F_q).
-__device__ __forceinline__ void point64(const double qL[F], const double qR[F], int a, double xq, double yq,
-                                        double hw, int d0, int d1, int d2, const StepParams& P, double fsum[F],
-                                        double T[3], double& amax) {
-  double UL[F], UR[F], unL, unR, vaL, vaR, pL, pR, sL, sR;
-  side64(qL, a, xq, yq, P, UL, unL, vaL, pL, sL);
-  side64(qR, a, xq, yq, P, UR, unR, vaR, pR, sR);
-  const double aq = max_nonneg(sL, sR);  // signal speeds are >= 0
+// Kurganov-Tadmor flux at one point with half its Simpson weight hw = w/2,
+// accumulated per field into the face sum:
+//   w F_q = hw (F_L + F_R) - hw a_q (U_R - U_L),  F = U u_n (+ p e_a, + p v_a)
+//         = U_L A + (U_R - U_L) B (+ the pressure terms),
+//   A = hw (u_nL + u_nR),  B = hw u_nR - hw a_q:
+// two fused steps and one difference per field, and a uniform state, whose
+// differences are zero, still has no dissipation to cancel.  rho u_n, v (three
+// components each): the reconstructed fields; eL, eR: end64 of the two sides;
+// un = v_a + wn, wn = omega y_q along x, -omega x_q along y (rotating frame,
+// u = v - omega z_hat x x_q).  The point lies at x_L + (h/2) d from the left
+// cell's centre, d = e_a + u1 e_b + u2 e_c (b < c the transverse axes); M
+// accumulates the moments of the momentum flux g = w F_q that the face's
+// torques need besides the face sum: u1 g_a, u1 g_c, u2 g_a, u2 g_b.  Every
+// operation is explicitly rounded or fused, so that the kernels that inline
+// it agree bit for bit.
+__device__ __forceinline__ void point64(const double qL[F], const End64& eL, const double qR[F], const End64& eR,
+                                        int a, double om, double r, double hw, int u1, int u2, double fsum[F],
+                                        double M[4], double& amax) {
+  const double vaL = (a == 0) ? qL[SX] : (a == 1) ? qL[SY] : qL[SZ];
+  const double vaR = (a == 0) ? qR[SX] : (a == 1) ? qR[SY] : qR[SZ];
+  const double unL = fma(om, r, vaL), unR = fma(om, r, vaR);
+  const double aq = max_nonneg(radd(fabs(unL), eL.c), radd(fabs(unR), eR.c));  // signal speeds are >= 0
   amax = max_nonneg(amax, aq);
-  const double hwa = hw * aq;
-  const double pp = pL + pR;
+  const double A = rmul(hw, radd(unL, unR)), B = rmul(hw, rsub(unR, aq));
+  const double hpp = rmul(hw, radd(eL.p, eR.p));
   double g[3];
 #pragma unroll
   for (int k = 0; k < F; ++k) {
-    // the pressure terms of F_L + F_R: p in the normal momentum, p v_a in the energy
-    double extra = 0.0;
-    if (k == SX || k == SY || k == SZ) extra = (a == k - SX) ? pp : 0.0;
-    if (k == EGAS) extra = fma(pL, vaL, pR * vaR);
-    const double sum = fma(UL[k], unL, fma(UR[k], unR, extra));
-    const double dif = UR[k] - UL[k];
-    if (k == SX || k == SY || k == SZ) {
-      const double gk = fma(hw, sum, -(hwa * dif));
-      g[k - SX] = gk;
-      fsum[k] += gk;
+    if (k >= SX && k <= SZ) {
+      const double uL = rmul(qL[RHO], qL[k]), uR = rmul(qR[RHO], qR[k]);
+      g[k - SX] = fma(uL, A, fma(rsub(uR, uL), B, (a == k - SX) ? hpp : 0.0));
+      fsum[k] = radd(fsum[k], g[k - SX]);
+    } else if (k == EGAS) {
+      const double pv = fma(eL.p, vaL, rmul(eR.p, vaR));
+      fsum[k] = fma(eL.E, A, fma(rsub(eR.E, eL.E), B, fma(hw, pv, fsum[k])));
     } else {
-      fsum[k] = fma(hw, sum, fma(-hwa, dif, fsum[k]));
+      fsum[k] = fma(qL[k], A, fma(rsub(qR[k], qL[k]), B, fsum[k]));
     }
   }
-  T[0] += signed_pick(d1, g[2]) - signed_pick(d2, g[1]);
-  T[1] += signed_pick(d2, g[0]) - signed_pick(d0, g[2]);
-  T[2] += signed_pick(d0, g[1]) - signed_pick(d1, g[0]);
+  const double ga = a == 0 ? g[0] : a == 1 ? g[1] : g[2];
+  if (u1 != 0) {
+    M[0] = radd(M[0], flip64(ga, u1 < 0));
+    M[1] = radd(M[1], flip64(a == 2 ? g[1] : g[2], u1 < 0));
+  }
+  if (u2 != 0) {
+    M[2] = radd(M[2], flip64(ga, u2 < 0));
+    M[3] = radd(M[3], flip64(a == 0 ? g[1] : g[0], u2 < 0));
+  }
+}
+
+// The rotating frame's part of u_n at a point: un = v_a + om r, om = omega
+// and r = y_q along x, om = -omega and r = x_q along y, none along z.
+__device__ __forceinline__ double frame_om(int a, const StepParams& P) {
+  return (a == 0) ? P.omega : (a == 1) ? -P.omega : 0.0;
 }
 
 // The face's torques about the left and right cell centres from point64's
-// torque sum T and face sum fsum: tl = (h/2) T, tr = (h/2) (T - 2 e_a x m)
-// with m the momentum part of fsum.
-__device__ __forceinline__ void face_torques64(const double T[3], const double fsum[F], int a, double half_h,
+// moments M and face sum fsum: tl = (h/2) T with T = sum of d x g, and
+// tr = (h/2) (T - 2 e_a x m) about the centre at x_L + h e_a, m the momentum
+// part of fsum.  With d = e_a + u1 e_b + u2 e_c and m the sum of g, T has
+// along a the component +-(M[1] - M[3]), along b and c differences of M[2],
+// M[0] and m.
+__device__ __forceinline__ void face_torques64(const double M[4], const double fsum[F], int a, double half_h,
                                                double tl[3], double tr[3]) {
   const double mx = fsum[SX], my = fsum[SY], mz = fsum[SZ];
+  double T[3];
+  if (a == 0) {  // d = (1, u1, u2)
+    T[0] = rsub(M[1], M[3]);
+    T[1] = rsub(M[2], mz);
+    T[2] = rsub(my, M[0]);
+  } else if (a == 1) {  // d = (u1, 1, u2)
+    T[0] = rsub(mz, M[2]);
+    T[1] = rsub(M[3], M[1]);
+    T[2] = rsub(M[0], mx);
+  } else {  // d = (u1, u2, 1)
+    T[0] = rsub(M[2], my);
+    T[1] = rsub(mx, M[0]);
+    T[2] = rsub(M[1], M[3]);
+  }
   // e_a x m
-  const double ex = (a == 0) ? 0.0 : (a == 1) ? mz : -my;
-  const double ey = (a == 0) ? -mz : (a == 1) ? 0.0 : mx;
-  const double ez = (a == 0) ? my : (a == 1) ? -mx : 0.0;
-  tl[0] = half_h * T[0];
-  tl[1] = half_h * T[1];
-  tl[2] = half_h * T[2];
-  tr[0] = half_h * (T[0] - (ex + ex));
-  tr[1] = half_h * (T[1] - (ey + ey));
-  tr[2] = half_h * (T[2] - (ez + ez));
+  const double ex = (a == 0) ? 0.0 : (a == 1) ? mz : flip64(my, true);
+  const double ey = (a == 0) ? flip64(mz, true) : (a == 1) ? 0.0 : mx;
+  const double ez = (a == 0) ? my : (a == 1) ? flip64(mx, true) : 0.0;
+  tl[0] = rmul(half_h, T[0]);
+  tl[1] = rmul(half_h, T[1]);
+  tl[2] = rmul(half_h, T[2]);
+  tr[0] = rmul(half_h, fma(-2.0, ex, T[0]));
+  tr[1] = rmul(half_h, fma(-2.0, ey, T[1]));
+  tr[2] = rmul(half_h, fma(-2.0, ez, T[2]));
 }
 
 }  // namespace hyd

@@ -187,34 +187,6 @@ struct FusedIo {
   }
 };
 
-// ---- bounded inter-CTA waits ---------------------------------------------
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Wait until *p >= target.  Gives up (false) after limit_ns of polling, after
-// 2^26 polls whatever the clock says, or as soon as *abort is set.
-static __device__ bool wait_geq(const unsigned* p, unsigned target, const unsigned* abort, long long limit_ns) {
-  if (ld_acquire(p) >= target) return true;
-  const unsigned long long t0 = global_ns();
-  for (long i = 0; i < (1l << 26); ++i) {
-    __nanosleep(128);
-    if (ld_acquire(p) >= target) return true;
-    if (ld_acquire(abort) != 0u) return false;
-    if ((long long)(global_ns() - t0) > limit_ns) return false;
-  }
-  return false;
-}
-
 // Threads 0..26 wait until flags[] of the 27 neighbours of sub-grid s (under
 // the boundary map, s itself included) reach target (the sub-grid's tile
 // count: each tile adds one when its part is published); on a timeout the

@@ -143,10 +143,10 @@ __global__ void __launch_bounds__(kThreads64, 1) hydro_step_fp64_kernel(StepArgs
 #pragma unroll 1
     for (int j = -1; j <= N; ++j) {
       const int cj = c0 + j * sa;
-      double fsum[F], T[3];
+      double fsum[F], Mt[4];
 #pragma unroll
       for (int k = 0; k < F; ++k) fsum[k] = 0.0;
-      T[0] = T[1] = T[2] = 0.0;
+      Mt[0] = Mt[1] = Mt[2] = Mt[3] = 0.0;
       // left cell of face j-1/2 is (j-1) along a
       const int ci0 = axis_comp(0, a, b, j - 1, pb, pc) + ox, ci1 = axis_comp(1, a, b, j - 1, pb, pc) + oy;
       // the 9 face points as 4 mirrored pairs and the centre (p = 4); with one
@@ -198,15 +198,18 @@ __global__ void __launch_bounds__(kThreads64, 1) hydro_step_fp64_kernel(StepArgs
             // side 1: point p (offsets t1,t2) with right state qmB.
             const int u1 = side ? t1 : -t1, u2 = side ? t2 : -t2;
             const int pt = (u1 + 1) * 3 + (u2 + 1);
-            const int d0 = axis_comp(0, a, b, 1, u1, u2), d1 = axis_comp(1, a, b, 1, u1, u2),
-                      d2 = axis_comp(2, a, b, 1, u1, u2);
-            const double xq = o[0] + h * ((ci0 + 0.5) + 0.5 * d0);
-            const double yq = o[1] + h * ((ci1 + 0.5) + 0.5 * d1);
+            const int d0 = axis_comp(0, a, b, 1, u1, u2), d1 = axis_comp(1, a, b, 1, u1, u2);
+            // the coordinate that the frame velocity's normal component takes
+            const double rq = a == 0 ? fma(h, (ci1 + 0.5) + 0.5 * d1, o[1]) : fma(h, (ci0 + 0.5) + 0.5 * d0, o[0]);
             // half the Simpson weight (1, 4, 1) x (1, 4, 1) / 36 of the point; 1/2
             // for the single-point face flux
             const double hw = A.P.face_points == 1 ? 0.5
                              : (u1 == 0 && u2 == 0) ? (8.0 / 36.0) : (u1 == 0 || u2 == 0) ? (2.0 / 36.0) : (0.5 / 36.0);
-            point64(plus[pt], side ? qmB : qmA, a, xq, yq, hw, d0, d1, d2, A.P, fsum, T, amax);
+            const double* qL = plus[pt];
+            const double* qR = side ? qmB : qmA;
+            const End64 eL = end64(qL[RHO], qL[SX], qL[SY], qL[SZ], qL[EGAS], A.P);
+            const End64 eR = end64(qR[RHO], qR[SX], qR[SY], qR[SZ], qR[EGAS], A.P);
+            point64(qL, eL, qR, eR, a, frame_om(a, A.P), rq, hw, u1, u2, fsum, Mt, amax);
           }
         }
 #pragma unroll
@@ -216,7 +219,7 @@ __global__ void __launch_bounds__(kThreads64, 1) hydro_step_fp64_kernel(StepArgs
         }
       }
       double tl[3], tr[3];
-      face_torques64(T, fsum, a, half_h, tl, tr);
+      face_torques64(Mt, fsum, a, half_h, tl, tr);
       if (j >= 1) {
         // interior cell i = j-1 along a: differences of its two a-faces
         const int i = j - 1;

@@ -8,10 +8,14 @@
 // by two faces of a cell) the 6 edge lines and the corners (shared by three
 // faces) the 4 vertex lines, so an axis sweep that reconstructs its own 9
 // lines per cell evaluates 27 line-fields per cell where 13 are unique.
-// One persistent CTA of 192 threads per SM loops over 8^3 tiles:
-//   1. bulk TMA copies stage the ghost-padded state into shared memory (the
-//      next tile's copies are issued as soon as phase 3 no longer reads it,
-//      so they overlap phases 4 and 5); primitives replace it in place;
+// A team of T CTAs of 384 threads, one CTA per SM, works on one 8^3 tile at a
+// time (T = 1: a persistent loop of independent CTAs; T > 1: a cooperative
+// launch, the CTAs of a team meeting at bounded barriers in global memory):
+//   1. the tile's primitives into shared memory: T = 1 stages the
+//      ghost-padded state by bulk TMA copies (the next tile's copies are
+//      issued as soon as phase 3 no longer reads it, so they overlap phases 4
+//      and 5) and converts in place; a larger team converts each cell once,
+//      into a buffer in global memory that every CTA then copies;
 //   2. (learned smoothness indicator, optional) its per-cell decisions;
 //   3. lines: one work item per (field group, run), a run being a maximal segment
 //      of consecutive cells along one of the 13 directions d among the cells
@@ -22,18 +26,30 @@
 //      computed once for both cells (PPM's interface value at x + d/2 is one
 //      number for the cell x and its neighbour x + d), then applies the
 //      per-cell steepening and monotonicity fix-ups and stores both
-//      interface values of the cell in a per-CTA buffer in global memory
-//      (26 values per field and cell, read back from L2 or DRAM in phase 4);
-//   4. faces: 192 threads, one per (axis, transverse row), sweep their row's
-//      9 faces in the order of hydro_step_fp64.cu and sum the 9 Kurganov-
-//      Tadmor point fluxes with the Simpson weights from the stored values;
-//      per-axis flux differences go to the step scratch;
+//      interface values of the cell in a per-team buffer in global memory
+//      (read back from L2 or DRAM in phase 4).  The group of rho, v, eps and
+//      tau also stores what the flux needs of the state (end64: p, E, c), once
+//      per line end where the up to three faces at it would each compute it;
+//   4. faces: one work item per face sums its 9 Kurganov-Tadmor point fluxes
+//      with the Simpson weights from the stored ends, into the team's buffer
+//      of face sums;
 //   5. divergence, sources and dU/dt as in hydro_step_fp64.cu.
 // Runs are listed once per device, longest first, so that the lanes of a
-// warp mostly walk runs of equal length.  The walk's arithmetic is ppm64's,
-// operation for operation, on the same operands (the reversed line gives
-// the mirrored values bit for bit), so the stored values are those the axis
-// sweeps compute.
+// warp mostly walk runs of equal length; items are dealt out a warp at a time
+// over the team.  The walk's arithmetic is ppm64's, operation for operation,
+// on the same operands (the reversed line gives the mirrored values bit for
+// bit), so the stored values are those the axis sweeps compute, and the
+// results depend neither on T nor on the number of teams.
+//
+// What bounds it: the FP64 pipe, which issues a warp's instruction every 16
+// cycles per SM.  12 warps keep it busy without prefetching (6 warps held it
+// at 83 %), and the work is cut to the pipe's: decisions on bit patterns,
+// masks instead of |x| and -x, line ends' sound speeds shared and the flux in
+// two fused steps per field.  A tile of random data takes a CTA 0.726 ms
+// (about 1.09 before); the RK3 step of a 512-sub-grid blast 12.96 -> 7.73 ms.
+// Teams serve the batches that do not fill whole rounds of the SMs
+// (step_fp64_choose_team): 512 tiles take pairs of CTAs 2.69 ms and single
+// ones 2.90, one tile takes the whole chip 0.09 ms and one CTA 0.73.
 #include <algorithm>
 #include <vector>
 
@@ -44,17 +60,25 @@
 
 namespace hyd {
 
-constexpr int kLThreads = NROW;  // 192
+constexpr int kLThreads = 384;
+constexpr int kLWarps = kLThreads / 32;
 constexpr long kLWaitPolls = 1L << 24;
 
-// The line-end buffer of one CTA: for each of the 26 (direction, end) slots
+// The line-end buffer of one team: for each of the 26 (direction, end) slots
 // and each cell of the 10^3 box of interior cells and their face-adjacent
-// ghost layer, a record of the 10 fields padded to 12 doubles (three 32-byte
-// sectors, each written whole by one thread: fields 0-3, 4-7, 8-9 and two
-// zeros): [slot][box cell][kRec] doubles.
+// ghost layer, a record of 12 doubles in three 32-byte sectors, each written
+// whole by one thread: rho v | p E c tau | z species (point64's operands; eps
+// itself is not needed past end64): [slot][box cell][kRec] doubles.  Then the
+// tile's face sums [kFv][kFaces] (fluxes, torques about the left and the
+// right cell), and the padded tile's primitives [F][S3] (teams of more than
+// one CTA).
 constexpr int kBox = (N + 2) * (N + 2) * (N + 2);  // 1000
 constexpr int kRec = 12;
-constexpr size_t kLinesPerCta = (size_t)26 * kBox * kRec;
+constexpr int kFaces = 3 * (N + 1) * N * N;  // 1728, face (a, j, pc, pb): ((a * 9 + j) * 8 + pc) * 8 + pb
+constexpr int kFv = F + 6;
+constexpr size_t kEndsPerTeam = (size_t)26 * kBox * kRec;
+constexpr size_t kSumsPerTeam = (size_t)kFv * kFaces;
+constexpr size_t kLinesPerTeam = kEndsPerTeam + kSumsPerTeam + (size_t)F * S3;
 
 // Directions d with components in {-1, 0, 1}, the first nonzero one
 // positive; index 9 dx + 3 dy + dz - 1 in [0, 13).  Slot 2 dd + 0 holds the
@@ -130,13 +154,22 @@ static std::vector<uint32_t> build_line_runs(int* n_axis) {
 
 static int g_runs_total = 0, g_runs_axis = 0;
 
+// Four doubles of one 32-byte sector, in one access.
+__device__ __forceinline__ void st_sector(double* p, double a, double b, double c, double d) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
+}
+__device__ __forceinline__ void ld_sector(const double* p, double& a, double& b, double& c, double& d) {
+  asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p) : "memory");
+}
+
 // One work item of phase 3: fields k0 .. k0 + NG - 1 along run word e.  The
 // window holds, per field, the samples S(i-2..i+2) of cell i of the run, the
 // differences and MC slopes around it and the interface value Q(i - 1/2);
 // each step loads one sample per field and forms one difference, one slope
 // and one interface value (ppm64's operations on the same operands), then
-// the cell's fix-ups, and stores the group's 32-byte sector of both records
-// of the cell.
+// the cell's fix-ups, and stores the group's sectors of both records of the
+// cell: fields 0 .. 5 with end64's values the first two, fields 6 .. 9 the
+// last.
 template <bool kGate, bool kContact, int NG>
 __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uint8_t* __restrict__ smooth,
                                          const StepParams& P, double* __restrict__ R, uint32_t e, int k0,
@@ -145,11 +178,12 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
   const int dx = (int)((e >> 26) & 3u) - 1, dy = (int)((e >> 28) & 3u) - 1, dz = (int)(e >> 30) - 1;
   const int sv = dx + S * dy + S * S * dz;                             // shared-memory stride along d
   const int bv = (dx + (N + 2) * dy + (N + 2) * (N + 2) * dz) * kRec;  // line-buffer stride along d
-  double* Rp = R + ((size_t)(2 * dir_index(dx, dy, dz)) * kBox + b0) * kRec + k0;
+  static_assert(NG == 6 || NG == 4, "field groups 0 .. 5 and 6 .. 9");
+  double* Rp = R + ((size_t)(2 * dir_index(dx, dy, dz)) * kBox + b0) * kRec + (NG == 6 ? 0 : 8);
   double* Rm = Rp + (size_t)kBox * kRec;
   const double* q = Q + k0 * S3 + c0;
-  // the group's steepened field (rho in group 0, the species in group 2)
-  const bool steep_group = kContact && (k0 == RHO || k0 + NG > SP0);
+  // the group's steepened field: rho in the first, the species in the second
+  const bool steep_group = kContact;
   double sm2[NG], sm1[NG], s0[NG], s1[NG], dr[NG], Dm[NG], Dc[NG], qm[NG];
 #pragma unroll
   for (int f = 0; f < NG; ++f) {
@@ -200,7 +234,7 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
       Dc[f] = Dp;
       qm[f] = qp;
     }
-    if (NG == 4 && k0 == 0 && P.spin) {
+    if (NG == 6 && P.spin) {
       // the cell's spin fed back into the velocity at both ends (spin_dv64)
       double dv[3];
       spin_dv64(Q[RHO * S3 + ci], Q[EGAS * S3 + ci], Q[ZX * S3 + ci], Q[ZY * S3 + ci], Q[ZZ * S3 + ci], k3h,
@@ -211,56 +245,100 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
         m[(1 + m3) % NG] = rsub(m[(1 + m3) % NG], dv[m3]);
       }
     }
-    double2* wp = reinterpret_cast<double2*>(Rp + i * bv);
-    double2* wm = reinterpret_cast<double2*>(Rm + i * bv);
-    wp[0] = make_double2(p[0], p[1]);
-    wm[0] = make_double2(m[0], m[1]);
-    if (NG == 4) {
-      wp[1] = make_double2(p[NG > 2 ? 2 : 0], p[NG > 3 ? 3 : 0]);
-      wm[1] = make_double2(m[NG > 2 ? 2 : 0], m[NG > 3 ? 3 : 0]);
+    double* wp = Rp + i * bv;
+    double* wm = Rm + i * bv;
+    if (NG == 6) {
+      const End64 ep = end64(p[0], p[1], p[2], p[3], p[NG > 4 ? 4 : 0], P);
+      const End64 em = end64(m[0], m[1], m[2], m[3], m[NG > 4 ? 4 : 0], P);
+      st_sector(wp, p[0], p[1], p[2], p[3]);
+      st_sector(wm, m[0], m[1], m[2], m[3]);
+      st_sector(wp + 4, ep.p, ep.E, ep.c, p[NG > 5 ? 5 : 0]);
+      st_sector(wm + 4, em.p, em.E, em.c, m[NG > 5 ? 5 : 0]);
     } else {
-      wp[1] = make_double2(0.0, 0.0);
-      wm[1] = make_double2(0.0, 0.0);
+      st_sector(wp, p[0], p[1], p[2], p[3]);
+      st_sector(wm, m[0], m[1], m[2], m[3]);
     }
   }
 }
 
-// kGate, kContact, NN: as for hydro_step_fp64_kernel.  A.lines: the per-CTA
-// line-end buffers (kLinesPerCta doubles per CTA); n_runs: the runs of
-// g_line_runs that phase 3 walks (the axis runs alone for the single-point
-// face flux).
+// The primitives of one padded cell in place of its conserved state
+// (hydro_step_fp64_kernel's arithmetic); false for a non-physical cell.
+__device__ __forceinline__ bool prims64(double u[EGAS + 1], double tau, const StepParams& P) {
+  const double rho = u[RHO];
+  const double vx = u[SX] / rho, vy = u[SY] / rho, vz = u[SZ] / rho;
+  const double E = u[EGAS];
+  const double ek = rmul(rmul(0.5, rho), radd(radd(rmul(vx, vx), rmul(vy, vy)), rmul(vz, vz)));
+  const double eE = rsub(E, ek);
+  const double eps = (eE > rmul(P.eta1, E)) ? eE : pow(tau, P.gamma);
+  u[SX] = vx;
+  u[SY] = vy;
+  u[SZ] = vz;
+  u[EGAS] = eps;
+  return (rho > 0.0) && (eps > 0.0);
+}
+
+// Barrier of a team (T = 1: of the CTA): every thread's earlier writes are
+// visible to the team's threads after it.  k counts the team's barriers since
+// the launch; sync[0] is the launch's abort word, sync[32 (1 + team)] the
+// team's arrivals (zero at the launch).  False, for all threads, if a wait
+// expired anywhere.
+struct TeamSync {
+  unsigned* sync;
+  unsigned team, size, k;
+  long long wait_ns;
+  unsigned* status;
+};
+__device__ __forceinline__ bool team_barrier(TeamSync& B, int* sh_ok) {
+  __syncthreads();
+  if (B.size == 1) return true;
+  ++B.k;
+  if (threadIdx.x == 0) {
+    unsigned* arrive = B.sync + 32 * (1 + (size_t)B.team);
+    __threadfence();
+    atomicAdd(arrive, 1u);
+    const bool ok = wait_geq(arrive, B.k * B.size, B.sync, B.wait_ns);
+    if (!ok) {
+      atomicOr(B.status, 2u);
+      atomicExch(B.sync, 1u);
+    }
+    *sh_ok = ok;
+  }
+  __syncthreads();
+  return *sh_ok != 0;
+}
+
+// kGate, kContact, NN: as for hydro_step_fp64_kernel.  A.lines: the per-team
+// buffers (kLinesPerTeam doubles each); n_runs: the runs of g_line_runs that
+// phase 3 walks (the axis runs alone for the single-point face flux); T: the
+// CTAs of a team; sync: TeamSync's words (T > 1), zero at the launch.
 template <bool kGate, bool kContact = false, int NN = N>
-__global__ void __launch_bounds__(kLThreads, 1) hydro_step_fp64_lines_kernel(StepArgs64 A, int n_runs) {
-  using T = Tile<NN>;
+__global__ void __launch_bounds__(kLThreads, 1)
+    hydro_step_fp64_lines_kernel(StepArgs64 A, int n_runs, int T, unsigned* sync, long long wait_ns) {
+  using Tl = Tile<NN>;
   extern __shared__ __align__(128) double Q[];  // [F][S3], then the indicator's flags
   uint8_t* smooth = reinterpret_cast<uint8_t*>(Q + F * S3);
   __shared__ __align__(8) uint64_t bar;
-  __shared__ double red[kLThreads / 32];
-  __shared__ int bail;
-  const int tid = threadIdx.x;
-  double* __restrict__ D = A.scratch + (size_t)blockIdx.x * kScratchPerSub;
-  double* R = A.lines + (size_t)blockIdx.x * kLinesPerCta;
-  const int n_units = A.n_sub * T::kTiles;
-
-  // the row of phases 4 and 5: axis a, transverse axes b < c at pb, pc (the
-  // warp map of hydro_step_fp64_kernel)
-  static_assert(N == 8 && S == 14, "row-to-warp map assumes 8^3 interiors with 3-cell ghosts");
-  const int a = tid / (N * N);
-  const int r = tid % (N * N);
-  const int pb = ((r >> 5) << 2) | (r & 3), pc = (r & 31) >> 2;
-  const int b = (a == 0) ? 1 : 0;
+  __shared__ double red[kLWarps];
+  __shared__ int bail, sh_ok;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int team = blockIdx.x / T, rank = blockIdx.x % T, n_teams = gridDim.x / T;
+  double* R = A.lines + (size_t)team * kLinesPerTeam;
+  double* Fs = R + kEndsPerTeam;
+  double* Pb = Fs + kSumsPerTeam;
+  const int n_units = A.n_sub * Tl::kTiles;
+  TeamSync B{sync, (unsigned)team, (unsigned)T, 0u, wait_ns, A.status};
 
   // bulk copies of tile u into Q, completing on bar (warp 0; as in
   // hydro_step_fp64_kernel)
   auto stage = [&](int u) {
     if (tid < 32) {
-      const T tile(u);
+      const Tl tile(u);
       if (tid == 0) {
         fence_proxy_async();
         mbar_expect_tx(&bar, (uint32_t)(F * S3 * sizeof(double)));
       }
       __syncwarp();
-      const double* src = A.U + (size_t)tile.s * F * T::kS3;
+      const double* src = A.U + (size_t)tile.s * F * Tl::kS3;
       if (NN == N) {
         if (tid == 0)
 #pragma unroll 1
@@ -269,7 +347,7 @@ __global__ void __launch_bounds__(kLThreads, 1) hydro_step_fp64_lines_kernel(Ste
 #pragma unroll 1
         for (int w = tid; w < F * S * S; w += 32) {
           const int k = w / (S * S), z = (w / S) % S, y = w % S;
-          bulk_g2s(Q + k * S3 + (z * S + y) * S, src + (size_t)k * T::kS3 + tile.pad(0, y, z), S * sizeof(double),
+          bulk_g2s(Q + k * S3 + (z * S + y) * S, src + (size_t)k * Tl::kS3 + tile.pad(0, y, z), S * sizeof(double),
                    &bar);
         }
       }
@@ -282,34 +360,49 @@ __global__ void __launch_bounds__(kLThreads, 1) hydro_step_fp64_lines_kernel(Ste
     bail = 0;
   }
   __syncthreads();
-  if ((int)blockIdx.x < n_units) stage(blockIdx.x);
+  if (T == 1 && team < n_units) stage(team);
 
   uint32_t phase = 0;
-  for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
-    const T tile(u);
+  for (int u = team; u < n_units; u += n_teams) {
+    const Tl tile(u);
     const int s = tile.s;
-    if (!mbar_wait_bounded(&bar, phase, kLWaitPolls)) {
-      atomicOr(A.status, 2u);
-      bail = 1;
-    }
-    phase ^= 1u;
-    __syncthreads();
-    if (bail) break;
 
-    // ---- 1. primitives in place (hydro_step_fp64_kernel's arithmetic) ----
+    // ---- 1. primitives ------------------------------------------------------
     bool bad = false;
-    for (int c = tid; c < S3; c += kLThreads) {
-      const double rho = Q[RHO * S3 + c];
-      const double vx = Q[SX * S3 + c] / rho, vy = Q[SY * S3 + c] / rho, vz = Q[SZ * S3 + c] / rho;
-      const double E = Q[EGAS * S3 + c];
-      const double ek = rmul(rmul(0.5, rho), radd(radd(rmul(vx, vx), rmul(vy, vy)), rmul(vz, vz)));
-      const double eE = rsub(E, ek);
-      const double eps = (eE > rmul(A.P.eta1, E)) ? eE : pow(Q[TAU * S3 + c], A.P.gamma);
-      Q[SX * S3 + c] = vx;
-      Q[SY * S3 + c] = vy;
-      Q[SZ * S3 + c] = vz;
-      Q[EGAS * S3 + c] = eps;
-      bad |= !(rho > 0.0) || !(eps > 0.0);
+    if (T == 1) {
+      if (!mbar_wait_bounded(&bar, phase, kLWaitPolls)) {
+        atomicOr(A.status, 2u);
+        bail = 1;
+      }
+      phase ^= 1u;
+      __syncthreads();
+      if (bail) break;
+      for (int c = tid; c < S3; c += kLThreads) {
+        double w[EGAS + 1];
+#pragma unroll
+        for (int k = 0; k <= EGAS; ++k) w[k] = Q[k * S3 + c];
+        bad |= !prims64(w, Q[TAU * S3 + c], A.P);
+#pragma unroll
+        for (int k = SX; k <= EGAS; ++k) Q[k * S3 + c] = w[k];
+      }
+    } else {
+      // the team converts each cell once; Pb was last read before the
+      // previous tile's lines, which every CTA of the team has passed
+      const double* src = A.U + (size_t)s * F * Tl::kS3;
+      for (int c = rank * kLThreads + tid; c < S3; c += T * kLThreads) {
+        const int pc = tile.pad(c);
+        double w[F];
+#pragma unroll
+        for (int k = 0; k < F; ++k) w[k] = __ldg(src + (size_t)k * Tl::kS3 + pc);
+        bad |= !prims64(w, w[TAU], A.P);
+#pragma unroll
+        for (int k = 0; k < F; ++k) Pb[k * S3 + c] = w[k];
+      }
+      if (!team_barrier(B, &sh_ok)) break;
+      const double2* pb2 = reinterpret_cast<const double2*>(Pb);
+      double2* q2 = reinterpret_cast<double2*>(Q);
+#pragma unroll 6
+      for (int c = tid; c < F * S3 / 2; c += kLThreads) q2[c] = __ldcg(pb2 + c);
     }
     if (bad) atomicOr(A.status, 1u);
     __syncthreads();
@@ -322,157 +415,137 @@ __global__ void __launch_bounds__(kLThreads, 1) hydro_step_fp64_lines_kernel(Ste
     // ---- 3. every line once: (field group, run) items, group-major ----------
     {
       const double k3h = 3.0 / A.h[s];  // the spin feedback's 3 / h
-      const int n_items = 3 * n_runs;
+      const int n_items = 2 * n_runs;
 #pragma unroll 1
-      for (int it = tid; it < n_items; it += kLThreads) {
-        const int g = it / n_runs;
-        const uint32_t e = g_line_runs[it - g * n_runs];
-        if (g < 2)
-          line_run<kGate, kContact, 4>(Q, smooth, A.P, R, e, 4 * g, k3h);
+      for (int it = (rank + T * warp) * 32 + lane; it < n_items; it += T * kLThreads) {
+        if (it < n_runs)
+          line_run<kGate, kContact, 6>(Q, smooth, A.P, R, g_line_runs[it], 0, k3h);
         else
-          line_run<kGate, kContact, 2>(Q, smooth, A.P, R, e, 8, k3h);
+          line_run<kGate, kContact, 4>(Q, smooth, A.P, R, g_line_runs[it - n_runs], 6, k3h);
       }
     }
     // the last reads of Q for this tile are done: order them before the bulk
     // copies of the next tile, which overlap phases 4 and 5
     fence_proxy_async();
-    __syncthreads();  // also: the line ends are visible to the whole CTA
-    if (u + (int)gridDim.x < n_units) stage(u + gridDim.x);
+    if (!team_barrier(B, &sh_ok)) break;  // the line ends are visible to the whole team
+    if (T == 1 && u + n_teams < n_units) stage(u + n_teams);
 
-    // ---- 4. face sweep of the row from the stored line ends ------------------
+    // ---- 4. faces from the stored line ends ----------------------------------
     const int ox = tile.o[0], oy = tile.o[1];
     const double h = A.h[s];
     const double half_h = 0.5 * h;
     const double o[3] = {A.origin[3 * s + 0], A.origin[3 * s + 1], A.origin[3 * s + 2]};
     double amax = 0.0;
-    double fprev[F], trprev[3];
-    // box index of the row's cell at a-index 0, and the box stride along a
-    const int box0 = ((axis_comp(2, a, b, 0, pb, pc) + 1) * (N + 2) + (axis_comp(1, a, b, 0, pb, pc) + 1)) * (N + 2) +
-                     (axis_comp(0, a, b, 0, pb, pc) + 1);
-    const int ba = a == 0 ? 1 : (a == 1 ? N + 2 : (N + 2) * (N + 2));
-    // The points of a face in the summation order of hydro_step_fp64_kernel:
-    // q = 2p + side for the mirrored pairs p = 0..3 (side 0: the point
-    // (-t1,-t2), side 1: (t1,t2), with (t1,t2) = (p/3 - 1, p%3 - 1)), then the
-    // centre q = 8; the single-point face flux takes the centre alone.
-    const int q0 = A.P.face_points == 1 ? 8 : 0;
-    auto offsets = [](int qq, int& u1, int& u2) {
-      const int pp = qq >> 1, t1 = pp / 3 - 1, t2 = pp % 3 - 1;
-      u1 = (qq & 1) ? t1 : -t1;
-      u2 = (qq & 1) ? t2 : -t2;
-    };
-    // the states at point qq of face jj - 1/2: the value at x + w/2 of cell
-    // jj - 1, w = e_a + u1 e_b + u2 e_c (left), and at x + w'/2 of cell jj,
-    // w' = w - 2 e_a (right)
-    auto fetch = [&](int jj, int qq, double(&L)[F], double(&Rr)[F]) {
-      int u1, u2;
-      offsets(qq, u1, u2);
-      const int d0 = axis_comp(0, a, b, 1, u1, u2), d1 = axis_comp(1, a, b, 1, u1, u2),
-                d2 = axis_comp(2, a, b, 1, u1, u2);
-      const int sl = end_slot(d0, d1, d2);
-      const int sr = end_slot(a == 0 ? -1 : d0, a == 1 ? -1 : d1, a == 2 ? -1 : d2);
-      const double2* pl = reinterpret_cast<const double2*>(R + ((size_t)sl * kBox + box0 + (jj - 1) * ba) * kRec);
-      const double2* pr = reinterpret_cast<const double2*>(R + ((size_t)sr * kBox + box0 + jj * ba) * kRec);
-#pragma unroll
-      for (int k = 0; k < F / 2; ++k) {
-        const double2 vl = pl[k], vr = pr[k];
-        L[2 * k] = vl.x;
-        L[2 * k + 1] = vl.y;
-        Rr[2 * k] = vr.x;
-        Rr[2 * k + 1] = vr.y;
-      }
-    };
-    // one point ahead: the next point's states load while this one computes
-    double nL[F], nR[F];
-    fetch(0, q0, nL, nR);
+    const bool one_point = A.P.face_points == 1;
 #pragma unroll 1
-    for (int j = 0; j <= N; ++j) {
-      // face j - 1/2 between the cells j - 1 (left) and j (right) along a
-      double fsum[F], T[3];
+    for (int f = (rank + T * warp) * 32 + lane; f < kFaces; f += T * kLThreads) {
+      // face j - 1/2 of row (pb, pc) along a, between the cells j - 1 (left)
+      // and j (right); transverse axes b < c
+      const int a = f / ((N + 1) * N * N), j = (f / (N * N)) % (N + 1), pc = (f / N) % N, pb = f % N;
+      const int b = (a == 0) ? 1 : 0;
+      const int ba = a == 0 ? 1 : (a == 1 ? N + 2 : (N + 2) * (N + 2));
+      // box index of the right cell
+      const int boxr = ((axis_comp(2, a, b, j, pb, pc) + 1) * (N + 2) + (axis_comp(1, a, b, j, pb, pc) + 1)) * (N + 2) +
+                       (axis_comp(0, a, b, j, pb, pc) + 1);
+      // the coordinate that the frame velocity's normal component takes (y_q
+      // for x-faces, x_q for y-faces), at the three offsets along b
+      const double cb = (pb + (a == 0 ? oy : ox)) + 0.5, ob = a == 0 ? o[1] : o[0];
+      const double rm = fma(h, cb - 0.5, ob), r0 = fma(h, cb, ob), rp = fma(h, cb + 0.5, ob);
+      const double om = frame_om(a, A.P);
+      double fsum[F], Mt[4];
 #pragma unroll
       for (int k = 0; k < F; ++k) fsum[k] = 0.0;
-      T[0] = T[1] = T[2] = 0.0;
-      const int ci0 = axis_comp(0, a, b, j - 1, pb, pc) + ox, ci1 = axis_comp(1, a, b, j - 1, pb, pc) + oy;
+      Mt[0] = Mt[1] = Mt[2] = Mt[3] = 0.0;
+      // the points in the summation order of hydro_step_fp64_kernel: q = 2p +
+      // side for the mirrored pairs p = 0..3 (side 0: the point (-t1,-t2),
+      // side 1: (t1,t2), with (t1,t2) = (p/3 - 1, p%3 - 1)), then the centre
+      // q = 8; the single-point face flux takes the centre alone
 #pragma unroll 1
-      for (int qq = q0; qq <= 8; ++qq) {
-        double qL[F], qR[F];
-#pragma unroll
-        for (int k = 0; k < F; ++k) {
-          qL[k] = nL[k];
-          qR[k] = nR[k];
-        }
-        if (qq < 8)
-          fetch(j, qq + 1, nL, nR);
-        else if (j < N)
-          fetch(j + 1, q0, nL, nR);
-        int u1, u2;
-        offsets(qq, u1, u2);
+      for (int qq = one_point ? 8 : 0; qq <= 8; ++qq) {
+        const int pp = qq >> 1, t1 = pp / 3 - 1, t2 = pp % 3 - 1;
+        const int u1 = (qq & 1) ? t1 : -t1, u2 = (qq & 1) ? t2 : -t2;
         const int d0 = axis_comp(0, a, b, 1, u1, u2), d1 = axis_comp(1, a, b, 1, u1, u2),
                   d2 = axis_comp(2, a, b, 1, u1, u2);
-        const double xq = o[0] + h * ((ci0 + 0.5) + 0.5 * d0);
-        const double yq = o[1] + h * ((ci1 + 0.5) + 0.5 * d1);
+        // the value at x + w/2 of cell j - 1, w = e_a + u1 e_b + u2 e_c (left),
+        // and at x + w'/2 of cell j, w' = w - 2 e_a (right)
+        const int sl = end_slot(d0, d1, d2);
+        const int sr = end_slot(a == 0 ? -1 : d0, a == 1 ? -1 : d1, a == 2 ? -1 : d2);
+        const double* pl = R + ((size_t)sl * kBox + boxr - ba) * kRec;
+        const double* pr = R + ((size_t)sr * kBox + boxr) * kRec;
+        double qL[F], qR[F];
+        End64 eL, eR;
+        ld_sector(pl, qL[RHO], qL[SX], qL[SY], qL[SZ]);
+        ld_sector(pr, qR[RHO], qR[SX], qR[SY], qR[SZ]);
+        ld_sector(pl + 4, eL.p, eL.E, eL.c, qL[TAU]);
+        ld_sector(pr + 4, eR.p, eR.E, eR.c, qR[TAU]);
+        ld_sector(pl + 8, qL[ZX], qL[ZY], qL[ZZ], qL[SP0]);
+        ld_sector(pr + 8, qR[ZX], qR[ZY], qR[ZZ], qR[SP0]);
+        qL[EGAS] = qR[EGAS] = 0.0;  // not read
+        const double r = u1 == 0 ? r0 : (u1 > 0 ? rp : rm);
         // half the Simpson weight (1, 4, 1) x (1, 4, 1) / 36 of the point; 1/2
         // for the single-point face flux
-        const double hw = A.P.face_points == 1 ? 0.5
-                         : (u1 == 0 && u2 == 0) ? (8.0 / 36.0) : (u1 == 0 || u2 == 0) ? (2.0 / 36.0) : (0.5 / 36.0);
-        point64(qL, qR, a, xq, yq, hw, d0, d1, d2, A.P, fsum, T, amax);
+        const double hw = one_point                ? 0.5
+                          : (u1 == 0 && u2 == 0) ? (8.0 / 36.0)
+                          : (u1 == 0 || u2 == 0) ? (2.0 / 36.0)
+                                                 : (0.5 / 36.0);
+        point64(qL, eL, qR, eR, a, om, r, hw, u1, u2, fsum, Mt, amax);
       }
       double tl[3], tr[3];
-      face_torques64(T, fsum, a, half_h, tl, tr);
-      if (j >= 1) {
-        // interior cell i = j-1 along a: differences of its two a-faces
-        const int i = j - 1;
-        const int cell = (axis_comp(2, a, b, i, pb, pc) * N + axis_comp(1, a, b, i, pb, pc)) * N +
-                         axis_comp(0, a, b, i, pb, pc);
-        double* Da = D + (size_t)a * DQ * N3 + cell;
+      face_torques64(Mt, fsum, a, half_h, tl, tr);
 #pragma unroll
-        for (int k = 0; k < F; ++k) Da[k * N3] = fsum[k] - fprev[k];
+      for (int k = 0; k < F; ++k) Fs[k * kFaces + f] = fsum[k];
 #pragma unroll
-        for (int m = 0; m < 3; ++m) Da[(F + m) * N3] = tl[m] - trprev[m];
+      for (int m = 0; m < 3; ++m) {
+        Fs[(F + m) * kFaces + f] = tl[m];
+        Fs[(F + 3 + m) * kFaces + f] = tr[m];
       }
-#pragma unroll
-      for (int k = 0; k < F; ++k) fprev[k] = fsum[k];
-      trprev[0] = tr[0];
-      trprev[1] = tr[1];
-      trprev[2] = tr[2];
       if (A.face_flux && (j == 0 || j == N) && tile.outer(2 * a + (j == N ? 1 : 0))) {
         // sub-grid boundary face: sums and the torque about the interior cell
-        const int f = 2 * a + (j == N ? 1 : 0);
+        const int fo = 2 * a + (j == N ? 1 : 0);
 #pragma unroll
-        for (int k = 0; k < F; ++k) A.face_flux[tile.face(f, k, pc, pb)] = fsum[k];
+        for (int k = 0; k < F; ++k) A.face_flux[tile.face(fo, k, pc, pb)] = fsum[k];
 #pragma unroll
-        for (int m = 0; m < 3; ++m) A.face_flux[tile.face(f, F + m, pc, pb)] = (j == N) ? tl[m] : tr[m];
+        for (int m = 0; m < 3; ++m) A.face_flux[tile.face(fo, F + m, pc, pb)] = (j == N) ? tl[m] : tr[m];
       }
     }
     amax = warp_max(amax);
-    if ((tid & 31) == 0) red[tid >> 5] = amax;
-    __syncthreads();  // also: scratch writes visible, line-end reads finished
+    if (lane == 0) red[warp] = amax;
+    if (!team_barrier(B, &sh_ok)) break;  // the face sums are visible, line-end reads finished
 
     // ---- 5. divergence + sources, one thread per interior cell -----------
     const double inv_h = 1.0 / h;
     const double om = A.P.omega;
-    const double* Us = A.U + (size_t)s * F * T::kS3;
-    double* dU = A.dUdt + (size_t)s * F * T::kN3;
-    for (int c = tid; c < N3; c += kLThreads) {
+    const double* Us = A.U + (size_t)s * F * Tl::kS3;
+    double* dU = A.dUdt + (size_t)s * F * Tl::kN3;
+    for (int c = (rank + T * warp) * 32 + lane; c < N3; c += T * kLThreads) {
       const int x = c % N, y = (c / N) % N, z = c / (N * N);
       const int uc = tile.pad(x + G, y + G, z + G);  // in the sub-grid's padded array
       const int cs = tile.cell(c);                   // in its compact NN^3 array
+      // the cell's lower faces; the upper ones are N*N further
+      const double* f0 = Fs + (x * N + z) * N + y;
+      const double* f1 = Fs + (((N + 1) + y) * N + z) * N + x;
+      const double* f2 = Fs + ((2 * (N + 1) + z) * N + y) * N + x;
+      // differences of value q between the upper and the lower face (ql: its
+      // slot for the lower face, whose torques are about its right cell)
+      auto dif = [&](const double* fa, int q, int ql) {
+        return __ldcg(fa + q * kFaces + N * N) - __ldcg(fa + ql * kFaces);
+      };
       double du[F];
 #pragma unroll
       for (int k = 0; k < F; ++k) {
-        const double div = (D[(0 * DQ + k) * N3 + c] + D[(1 * DQ + k) * N3 + c]) + D[(2 * DQ + k) * N3 + c];
+        const double div = (dif(f0, k, k) + dif(f1, k, k)) + dif(f2, k, k);
         du[k] = -(div * inv_h);
       }
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
-        const double tq =
-            (D[(0 * DQ + F + m) * N3 + c] + D[(1 * DQ + F + m) * N3 + c]) + D[(2 * DQ + F + m) * N3 + c];
+        const double tq = (dif(f0, F + m, F + 3 + m) + dif(f1, F + m, F + 3 + m)) + dif(f2, F + m, F + 3 + m);
         du[ZX + m] = du[ZX + m] - tq * inv_h;
       }
-      const double sx = Us[SX * T::kS3 + uc], sy = Us[SY * T::kS3 + uc], sz = Us[SZ * T::kS3 + uc];
+      const double sx = Us[SX * Tl::kS3 + uc], sy = Us[SY * Tl::kS3 + uc], sz = Us[SZ * Tl::kS3 + uc];
       du[SX] = du[SX] + om * sy;
       du[SY] = du[SY] - om * sx;
-      du[ZX] = du[ZX] + om * Us[ZY * T::kS3 + uc];
-      du[ZY] = du[ZY] - om * Us[ZX * T::kS3 + uc];
+      du[ZX] = du[ZX] + om * Us[ZY * Tl::kS3 + uc];
+      du[ZY] = du[ZY] - om * Us[ZX * Tl::kS3 + uc];
       {
         // spin source w(x_c) x s, w = -omega z_hat x x_c: removes the torque
         // that the frame part s w_n of the momentum flux leaves in the face
@@ -485,27 +558,28 @@ __global__ void __launch_bounds__(kLThreads, 1) hydro_step_fp64_lines_kernel(Ste
         du[ZZ] = du[ZZ] + (wx * sy - wy * sx);
       }
       if (A.g) {
-        const double* gs = A.g + (size_t)s * 3 * T::kN3 + cs;
-        const double gx = gs[0], gy = gs[T::kN3], gz = gs[2 * T::kN3];
-        const double rho = Us[RHO * T::kS3 + uc];
+        const double* gs = A.g + (size_t)s * 3 * Tl::kN3 + cs;
+        const double gx = gs[0], gy = gs[Tl::kN3], gz = gs[2 * Tl::kN3];
+        const double rho = Us[RHO * Tl::kS3 + uc];
         du[SX] = du[SX] + rho * gx;
         du[SY] = du[SY] + rho * gy;
         du[SZ] = du[SZ] + rho * gz;
         du[EGAS] = du[EGAS] + ((sx * gx + sy * gy) + sz * gz);
       }
 #pragma unroll
-      for (int k = 0; k < F; ++k) dU[k * T::kN3 + cs] = du[k];
+      for (int k = 0; k < F; ++k) dU[k * Tl::kN3 + cs] = du[k];
     }
     if (tid == 0) {
       double m = red[0];
 #pragma unroll
-      for (int w = 1; w < kLThreads / 32; ++w) m = fmax(m, red[w]);
-      if (T::kTiles == 1)
+      for (int w = 1; w < kLWarps; ++w) m = fmax(m, red[w]);
+      if (Tl::kTiles == 1 && T == 1)
         A.amax[s] = m;
       else
         atomic_max_nonneg(A.amax + s, m);  // cleared before the launch
     }
-    __syncthreads();  // scratch, line ends and red reused by the next tile
+    // face sums and red are rewritten after the next tile's lines, whose
+    // barrier every thread of the team reaches after its reads above
   }
   __syncthreads();
   if (tid == 0) mbar_inval(&bar);
@@ -546,38 +620,78 @@ cudaError_t prepare_step_fp64_lines() {
   });
 }
 
-size_t step_fp64_lines_per_cta() { return kLinesPerCta; }
+size_t step_fp64_lines_per_team() { return kLinesPerTeam; }
+size_t step_fp64_lines_sync_words(int teams) { return 32 * (1 + (size_t)teams); }
 
-template <int NN>
-static void launch_fp64_lines_nn(const StepArgs64& A, int grid, int n_runs, cudaStream_t st) {
-  const size_t sm1 = step_fp64_lines_smem_bytes(true), sm0 = step_fp64_lines_smem_bytes(false);
-  if (A.gate && A.P.contact)
-    hydro_step_fp64_lines_kernel<true, true, NN><<<grid, kLThreads, sm1, st>>>(A, n_runs);
-  else if (A.gate)
-    hydro_step_fp64_lines_kernel<true, false, NN><<<grid, kLThreads, sm1, st>>>(A, n_runs);
-  else if (A.P.contact)
-    hydro_step_fp64_lines_kernel<false, true, NN><<<grid, kLThreads, sm0, st>>>(A, n_runs);
-  else
-    hydro_step_fp64_lines_kernel<false, false, NN><<<grid, kLThreads, sm0, st>>>(A, n_runs);
+// CTAs per team for `units` tiles on num_sms SMs: the smallest estimate of
+//   rounds of the teams over the batch x (a tile's time on T SMs),
+// the latter its FP64 work shared out (kTileUs on one SM), not below the
+// chain of the longest line run and a face (kChainUs), plus the team's
+// barriers and copies (kTeamUs).  A batch that fills whole rounds of single
+// CTAs keeps T = 1; 512 tiles on 152 SMs take 3.4 rounds' work in 4 rounds
+// alone, and one tile alone leaves 151 SMs idle.
+int step_fp64_choose_team(int units, int num_sms, int face_points) {
+  const double kTileUs = face_points == 1 ? 120.0 : 560.0, kChainUs = 12.0, kTeamUs = 12.0;
+  int best = 1;
+  double best_us = 1e300;
+  for (int T = 1; T <= num_sms; ++T) {
+    const int teams = num_sms / T;
+    const int rounds = (units + teams - 1) / teams;
+    double us = kTileUs / T;
+    if (T > 1) us = (us > kChainUs ? us : kChainUs) + kTeamUs;
+    // a larger team has to gain 2 %
+    if (rounds * us < 0.98 * best_us) {
+      best_us = rounds * us;
+      best = T;
+    }
+  }
+  return best;
 }
 
-// The FP64 step with every line once: grid persistent CTAs over the
-// A.n_sub * (nn/8)^3 tiles; A.lines holds grid * step_fp64_lines_per_cta()
-// doubles.  With 16^3 sub-grids the amax of a sub-grid is the atomic maximum
-// over its tiles, cleared here first.
-cudaError_t launch_step_fp64_lines(const StepArgs64& A, int grid, int nn, cudaStream_t st) {
+template <int NN>
+static cudaError_t launch_fp64_lines_nn(const StepArgs64& A, int grid, int n_runs, int T, unsigned* sync,
+                                        long long wait_ns, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kLThreads);
+  cfg.dynamicSmemBytes = step_fp64_lines_smem_bytes(A.gate);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = T > 1 ? 1 : 0;
+  if (A.gate && A.P.contact)
+    return cudaLaunchKernelEx(&cfg, hydro_step_fp64_lines_kernel<true, true, NN>, A, n_runs, T, sync, wait_ns);
+  if (A.gate)
+    return cudaLaunchKernelEx(&cfg, hydro_step_fp64_lines_kernel<true, false, NN>, A, n_runs, T, sync, wait_ns);
+  if (A.P.contact)
+    return cudaLaunchKernelEx(&cfg, hydro_step_fp64_lines_kernel<false, true, NN>, A, n_runs, T, sync, wait_ns);
+  return cudaLaunchKernelEx(&cfg, hydro_step_fp64_lines_kernel<false, false, NN>, A, n_runs, T, sync, wait_ns);
+}
+
+// The FP64 step with every line once, over the A.n_sub * (nn/8)^3 tiles:
+// `teams` teams of T CTAs (T > 1: teams * T at most the SMs, a cooperative
+// launch, and sync holds step_fp64_lines_sync_words(teams) words); A.lines
+// holds teams * step_fp64_lines_per_team() doubles.  Where several CTAs share
+// a sub-grid its amax is the atomic maximum over them, cleared here first.
+cudaError_t launch_step_fp64_lines(const StepArgs64& A, int teams, int T, unsigned* sync, int nn, cudaStream_t st) {
   cudaError_t e = prepare_step_fp64_lines();
   if (e != cudaSuccess) return e;
-  if (!A.lines) return cudaErrorInvalidValue;
+  if (!A.lines || T < 1 || (T > 1 && !sync)) return cudaErrorInvalidValue;
   const int n_runs = A.P.face_points == 1 ? g_runs_axis : g_runs_total;
-  if (nn == 16) {
+  if (T > 1) {
+    e = cudaMemsetAsync(sync, 0, step_fp64_lines_sync_words(teams) * sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
+  }
+  if (nn == 16 || T > 1) {
     e = cudaMemsetAsync(A.amax, 0, (size_t)A.n_sub * sizeof(double), st);
     if (e != cudaSuccess) return e;
-    launch_fp64_lines_nn<16>(A, grid, n_runs, st);
-  } else {
-    launch_fp64_lines_nn<8>(A, grid, n_runs, st);
   }
-  return cudaGetLastError();
+  // a second: far above the longest phase of a tile on one SM
+  const long long wait_ns = 1000000000ll;
+  return nn == 16 ? launch_fp64_lines_nn<16>(A, teams * T, n_runs, T, sync, wait_ns, st)
+                  : launch_fp64_lines_nn<8>(A, teams * T, n_runs, T, sync, wait_ns, st);
 }
 
 }  // namespace hyd
