@@ -131,6 +131,39 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 
+// ---- FP32 <-> FP64 on the integer pipes ----------------------------------------
+// The FP64 pipe takes a warp's conversion in 16 cycles, as long as the other
+// pipes take for some 60 instructions.  Numbers that are normal (or zero) in
+// FP32 convert by moving the exponent's bias and the significand; the others
+// (subnormals, overflows, infinities, NaNs) by the conversion instruction, in
+// a call: inlined, the compiler issues it predicated in every case, and a
+// predicated-off conversion holds the pipe like another.
+static __device__ __noinline__ double widen_call(float x) { return (double)x; }
+static __device__ __noinline__ float narrow_call(double x) { return (float)x; }
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  if ((m - 1u < 0x007fffffu) | (m >= 0x7f800000u)) return widen_call(x);
+  return __hiloint2double((int)(m == 0u ? b : ((m >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+}
+// To nearest, ties to even: the 29 bits cut off decide; a carry out of the
+// significand moves the exponent, to infinity at the top.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), mh = hi & 0x7fffffffu;
+  if (((mh | lo) != 0u) & (mh - 0x38100000u >= 0x0fe00000u)) return narrow_call(x);
+  const unsigned t = ((mh - 0x38000000u) << 3) | (lo >> 29);
+  const unsigned rest = (lo << 3) | (t & 1u);  // above half, or half with an odd result: > 0x80000000
+  const unsigned m = (mh | lo) == 0u ? 0u : t + (rest > 0x80000000u ? 1u : 0u);
+  return __uint_as_float(m | (hi & 0x80000000u));
+}
+
+// Whether eE > eta E (the dual-energy selections), from the FP32 values eEf of
+// eE and Ef of E where they differ by more than their rounding, else in FP64.
+static __device__ __noinline__ bool above_call(double eE, double eta, double E) { return eE > eta * E; }
+__device__ __forceinline__ bool above(double eE, float eEf, double eta, double E, float Ef) {
+  const float lim = 1.0001f * ((float)eta * Ef);
+  return (eEf > lim && lim > 1e-30f) ? true : above_call(eE, eta, E);
+}
+
 // ---- SSP-RK3 stage combination of one cell (Sec. IV-A.2) ----------------
 //   u <- alpha U0 + beta (U + dt dU/dt), (alpha, beta) = (0,1), (3/4,1/4), (1/3,2/3)
 //   then tau <- eps_E^(1/gamma) where eps_E = E - |s|^2/(2 rho) > eta2 E
@@ -143,22 +176,30 @@ __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a,
 template <bool kMixed>
 __device__ __forceinline__ void rk3_cell(const double U[F], const double U0[F], const double R[F], double dt,
                                          double alpha, double beta, double eta2, double inv_gamma, double u[F]) {
+  if (alpha == 0.0) {
+    // the first stage (beta = 1): U + dt R itself, without the factors' 20 or 30
+    // FP64 instructions
 #pragma unroll
-  for (int k = 0; k < F; ++k) {
-    if (kMixed) {
-      u[k] = fma(alpha, U0[k], beta * fma(dt, R[k], U[k]));
-    } else {
-      const double t = radd(U[k], rmul(dt, R[k]));
-      u[k] = radd(rmul(alpha, U0[k]), rmul(beta, t));
+    for (int k = 0; k < F; ++k) u[k] = kMixed ? fma(dt, R[k], U[k]) : radd(U[k], rmul(dt, R[k]));
+  } else {
+#pragma unroll
+    for (int k = 0; k < F; ++k) {
+      if (kMixed) {
+        u[k] = fma(alpha, U0[k], beta * fma(dt, R[k], U[k]));
+      } else {
+        const double t = radd(U[k], rmul(dt, R[k]));
+        u[k] = radd(rmul(alpha, U0[k]), rmul(beta, t));
+      }
     }
   }
   const double rho = u[RHO];
   if (kMixed) {
-    const double r0 = (double)__frcp_rn((float)rho);
+    const double r0 = widen(__frcp_rn(narrow(rho)));
     const double ri = r0 * fma(-rho, r0, 2.0);
     const double s2 = fma(u[SZ], u[SZ], fma(u[SY], u[SY], u[SX] * u[SX]));
     const double eE = u[EGAS] - 0.5 * s2 * ri;
-    if (eE > eta2 * u[EGAS]) u[TAU] = (double)__powf((float)eE, (float)inv_gamma);
+    const float eEf = narrow(eE);
+    if (above(eE, eEf, eta2, u[EGAS], narrow(u[EGAS]))) u[TAU] = widen(__powf(eEf, (float)inv_gamma));
   } else {
     const double vx = u[SX] / rho, vy = u[SY] / rho, vz = u[SZ] / rho;
     const double ek = rmul(rmul(0.5, rho), radd(radd(rmul(vx, vx), rmul(vy, vy)), rmul(vz, vz)));

@@ -67,16 +67,45 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 abs2(float2 a) { return f2(fabsf(a.x), fabsf(a.y)); }
 
-// slope32 on two lanes.
-__device__ __forceinline__ float2 slope32x2(float2 a, float2 b) {
-  const float2 t = mul2(f2(2.f), f2(fminf(fabsf(a.x), fabsf(b.x)), fminf(fabsf(a.y), fabsf(b.y))));
-  const float2 u = mul2(f2(0.5f), abs2(add2(a, b)));
-  const float2 ab = mul2(a, b);
-  return f2(ab.x <= 0.f ? 0.f : copysignf(fminf(t.x, u.x), b.x), ab.y <= 0.f ? 0.f : copysignf(fminf(t.y, u.y), b.y));
+// min(|a|, |b|) with the sign bit the exclusive or of a's and b's, in one
+// instruction.
+__device__ __forceinline__ float min_xorsign(float a, float b) {
+  float r;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
 }
 
-// ppm32 on two lanes (two fields of a line, or two lines); eta per lane.
-template <bool kSteep = false>
+// The MC slope on two lanes: w = min(|a|, |b|) signed by a b, so that w + |w| is
+// min(2|a|, 2|b|) where the differences agree in sign and 0 where they do not,
+// and its signed minimum with (a + b)/2 the slope: slope32's value (a zero may
+// carry a sign, and a product a b that underflows counts as positive).  Four
+// of its eight instructions run on the half-rate integer and comparison pipe,
+// of fourteen ten with the product's test, copysign and selects.
+__device__ __forceinline__ float2 slope32x2(float2 a, float2 b) {
+  const float wx = min_xorsign(a.x, b.x), wy = min_xorsign(a.y, b.y);
+  const float2 u = mul2(f2(0.5f), add2(a, b));
+  return f2(min_xorsign(__fadd_rn(wx, fabsf(wx)), u.x), min_xorsign(__fadd_rn(wy, fabsf(wy)), u.y));
+}
+
+// The fix-ups of one lane: p and m move to 3 s - 2 (the other one) where the
+// parabola overshoots, and to s at an extremum (e <= 0); s3 = 3 s.  Predicated
+// instructions on the values in place: a select costs a slot of the half-rate
+// pipe, and a move's value would be formed for every cell.
+__device__ __forceinline__ void ppm_fix(float e, float lhs, float rhs, float s, float s3, float& p, float& m) {
+  asm("{\n .reg .pred a, b, c;\n .reg .f32 n, q;\n"
+      " neg.f32 n, %4;\n mov.b32 q, %0;\n"
+      " setp.lt.f32 a, %3, n;\n setp.gt.f32 b, %3, %4;\n setp.le.f32 c, %2, 0f00000000;\n"
+      " @a fma.rn.f32 %0, %1, 0fC0000000, %6;\n"
+      " @b fma.rn.f32 %1, q, 0fC0000000, %6;\n"
+      " @c mov.b32 %0, %5;\n @c mov.b32 %1, %5;\n}"
+      : "+f"(p), "+f"(m)
+      : "f"(e), "f"(lhs), "f"(rhs), "f"(s), "f"(s3));
+}
+
+// ppm32 on two lanes (two fields of a line, or two lines).  kSteep: the
+// contact-steepening blend with eta in no lane (0), in both (1), or in the
+// x (2) or y (3) lane alone.
+template <int kSteep = 0>
 __device__ __forceinline__ void ppm32x2(float2 s0, float2 s1, float2 s2, float2 s3, float2 s4, float2& qp, float2& qm,
                                         float2 eta = make_float2(0.f, 0.f)) {
   const float2 msixth = f2(-(1.f / 6.f)), half = f2(0.5f);
@@ -84,21 +113,30 @@ __device__ __forceinline__ void ppm32x2(float2 s0, float2 s1, float2 s2, float2 
   const float2 D0 = slope32x2(d0, d1), D1 = slope32x2(d1, d2), D2 = slope32x2(d2, d3);
   float2 p = fma2(msixth, sub2(D2, D1), mul2(half, add2(s2, s3)));
   float2 m = fma2(msixth, sub2(D1, D0), mul2(half, add2(s1, s2)));
-  if (kSteep) {
+  if (kSteep == 1) {
     const float2 keep = sub2(f2(1.f), eta);
     p = fma2(eta, fma2(f2(-0.5f), D2, s3), mul2(keep, p));
     m = fma2(eta, fma2(half, D0, s1), mul2(keep, m));
+  }
+  if (kSteep == 2) {
+    const float keep = __fsub_rn(1.f, eta.x);
+    p.x = __fmaf_rn(eta.x, __fmaf_rn(-0.5f, D2.x, s3.x), __fmul_rn(keep, p.x));
+    m.x = __fmaf_rn(eta.x, __fmaf_rn(0.5f, D0.x, s1.x), __fmul_rn(keep, m.x));
+  }
+  if (kSteep == 3) {
+    const float keep = __fsub_rn(1.f, eta.y);
+    p.y = __fmaf_rn(eta.y, __fmaf_rn(-0.5f, D2.y, s3.y), __fmul_rn(keep, p.y));
+    m.y = __fmaf_rn(eta.y, __fmaf_rn(0.5f, D0.y, s1.y), __fmul_rn(keep, m.y));
   }
   const float2 e = mul2(sub2(p, s2), sub2(s2, m));
   const float2 dq = sub2(p, m);
   const float2 lhs = mul2(dq, fma2(f2(-0.5f), add2(p, m), s2));
   const float2 rhs = mul2(mul2(dq, dq), f2(1.f / 6.f));
   const float2 s2x3 = mul2(f2(3.f), s2);
-  const float2 mc = fma2(f2(-2.f), p, s2x3), pc = fma2(f2(-2.f), m, s2x3);
-  qp.x = e.x <= 0.f ? s2.x : (lhs.x < -rhs.x ? pc.x : p.x);
-  qp.y = e.y <= 0.f ? s2.y : (lhs.y < -rhs.y ? pc.y : p.y);
-  qm.x = e.x <= 0.f ? s2.x : (lhs.x > rhs.x ? mc.x : m.x);
-  qm.y = e.y <= 0.f ? s2.y : (lhs.y > rhs.y ? mc.y : m.y);
+  qp = p;
+  qm = m;
+  ppm_fix(e.x, lhs.x, rhs.x, s2.x, s2x3.x, qp.x, qm.x);
+  ppm_fix(e.y, lhs.y, rhs.y, s2.y, s2x3.y, qp.y, qm.y);
 }
 
 // The five samples of fields fa and fb along a line (stride st through cell
@@ -165,7 +203,7 @@ __device__ __forceinline__ void line10fc(const float* __restrict__ Q, int c, int
                                     contact_eta32(v.s[0].y, v.s[1].y, v.s[2].y, v.s[3].y, v.s[4].y))
                                : f2(0.f);
     float2 p, m;
-    ppm32x2<true>(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m, eta);
+    ppm32x2<1>(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m, eta);
     qp[RHO] = p.x;
     qp[SP0] = p.y;
     qm[RHO] = m.x;
@@ -234,11 +272,11 @@ __device__ __forceinline__ Side32x2 side32x2(const QA& qa, const QB& qb, int a, 
   s.p = mul2(f2(P.gm1), eps);
   const float2 gp = mul2(f2(P.gamma), s.p);
   const float2 c2 = f2(__fdividef(gp.x, s.rho.x), __fdividef(gp.y, s.rho.y));
-  const float2 c = mul2(c2, f2(rsqrtf(c2.x), rsqrtf(c2.y)));
   const float2 ux = fma2(f2(P.omega), yq, s.vx), uy = fma2(f2(-P.omega), xq, s.vy);
   s.un = (a == 0) ? ux : (a == 1) ? uy : s.vz;
   s.va = (a == 0) ? s.vx : (a == 1) ? s.vy : s.vz;
-  s.spd = add2(abs2(s.un), c);
+  // |u_n| + c with c = c^2 / c, in one rounding
+  s.spd = fma2(c2, f2(rsqrtf(c2.x), rsqrtf(c2.y)), abs2(s.un));
   return s;
 }
 
@@ -359,20 +397,24 @@ __device__ __forceinline__ void line10u(const float* __restrict__ Q, int c, int 
 // Returns false for a non-physical cell.
 __device__ __forceinline__ bool prims_mixed(const double u[F], double eta1, float gamma, float q[F]) {
   const double rho = u[RHO];
-  const double r0 = (double)__frcp_rn((float)rho);
+  const float rf = narrow(rho);
+  const double r0 = widen(__frcp_rn(rf));
   const double ri = r0 * fma(-rho, r0, 2.0);
   const double s2 = fma(u[SZ], u[SZ], fma(u[SY], u[SY], u[SX] * u[SX]));
   const double eE = u[EGAS] - 0.5 * s2 * ri;
-  const float rif = (float)ri;
-  const float eps = (eE > eta1 * u[EGAS]) ? (float)eE : __powf((float)u[TAU], gamma);
-  q[RHO] = (float)rho;
-  q[SX] = (float)u[SX] * rif;
-  q[SY] = (float)u[SY] * rif;
-  q[SZ] = (float)u[SZ] * rif;
+  const float rif = narrow(ri);
+  const float eEf = narrow(eE), tau = narrow(u[TAU]);
+  const float eps = above(eE, eEf, eta1, u[EGAS], narrow(u[EGAS])) ? eEf : __powf(tau, gamma);
+  q[RHO] = rf;
+  q[SX] = narrow(u[SX]) * rif;
+  q[SY] = narrow(u[SY]) * rif;
+  q[SZ] = narrow(u[SZ]) * rif;
   q[EGAS] = eps;
+  q[TAU] = tau;
 #pragma unroll
-  for (int k = TAU; k < F; ++k) q[k] = (float)u[k];
-  return (rho > 0.0) && (eps > 0.f);
+  for (int k = TAU + 1; k < F; ++k) q[k] = narrow(u[k]);
+  // rho > 0.0: from its FP32 value (false for NaN), or its bits where that is zero
+  return ((rf > 0.f) | ((rf == 0.f) & (__double_as_longlong(rho) > 0LL))) && (eps > 0.f);
 }
 
 // Indicator network: 54 -> 32 (ReLU) -> 32 (ReLU) -> 1 (logit).  Parameters

@@ -72,32 +72,31 @@ __device__ __forceinline__ RowMap row_map(int tid) {
 // padded index uc are the tile's; offx, offy: the tile's cell offsets in its
 // sub-grid): dU/dt from its per-axis differences of face sums,
 // D_a[q] = Fbar_a(i+1/2) - Fbar_a(i-1/2) for the F fluxes and the torque
-// differences for q >= F (FP64), summed as (D_x + D_y) + D_z: s01(q) gives
-// D_x + D_y, d2(q) gives D_z.  Then the rotating-frame, spin and gravity
-// sources, and io.store.  Every operation is explicitly rounded or fused,
+// differences for q >= F (FP64): sum(q) gives (D_x + D_y) + D_z.  Then the
+// rotating-frame, spin and gravity sources, and io.store.  Every operation is explicitly rounded or fused,
 // so that both sub-grid decompositions and every kernel give the same bits.
-template <class Io, class S01, class D2>
+template <class Io, class Sum>
 __device__ __forceinline__ void finish_cell(const StepArgs64& A, const Io& io, const typename Io::Sub& sub,
-                                            int offx, int offy, int x, int y, int z, const S01& s01, const D2& d2,
-                                            double hd, double inv_h, const double o[3]) {
+                                            int offx, int offy, int x, int y, int z, const Sum& sum, double hd,
+                                            double inv_h, const double o[3]) {
   const int c = (z * N + y) * N + x;
   const int uc = ((z + G) * S + (y + G)) * S + (x + G);
   const double om = A.P.omega;
   double du[F];
 #pragma unroll
-  for (int k = 0; k < F; ++k) du[k] = -__dmul_rn(__dadd_rn(s01(k), d2(k)), inv_h);
+  for (int k = 0; k < F; ++k) du[k] = -__dmul_rn(sum(k), inv_h);
 #pragma unroll
-  for (int m = 0; m < 3; ++m) du[ZX + m] = __dsub_rn(du[ZX + m], __dmul_rn(__dadd_rn(s01(F + m), d2(F + m)), inv_h));
+  for (int m = 0; m < 3; ++m) du[ZX + m] = __dsub_rn(du[ZX + m], __dmul_rn(sum(F + m), inv_h));
   // The sources' products and sums are written as explicit FMAs and
   // rounded operations, so that every kernel instance rounds them alike.
   double uin[F];
   io.own(sub, c, uc, uin);
   const double sx = uin[SX], sy = uin[SY], sz = uin[SZ];
-  du[SX] = fma(om, sy, du[SX]);
-  du[SY] = fma(-om, sx, du[SY]);
-  du[ZX] = fma(om, uin[ZY], du[ZX]);
-  du[ZY] = fma(-om, uin[ZX], du[ZY]);
-  {
+  if (om != 0.0) {  // (19 FP64 instructions that change nothing in an inertial frame)
+    du[SX] = fma(om, sy, du[SX]);
+    du[SY] = fma(-om, sx, du[SY]);
+    du[ZX] = fma(om, uin[ZY], du[ZX]);
+    du[ZY] = fma(-om, uin[ZX], du[ZY]);
     // spin source w(x_c) x s, w = -omega z_hat x x_c: removes the torque
     // that the frame part s w_n of the momentum flux leaves in the face
     // torques, so that sum (x_c x s + z)_z is conserved for omega != 0
@@ -295,9 +294,9 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
       float Str[3];
       right_torque32(a, h, Sf, Stl, Str);
 #pragma unroll
-      for (int k = 0; k < F; ++k) fd[k] = (double)Sf[k];
+      for (int k = 0; k < F; ++k) fd[k] = widen(Sf[k]);
 #pragma unroll
-      for (int m = 0; m < 3; ++m) tld[m] = (double)Stl[m];
+      for (int m = 0; m < 3; ++m) tld[m] = widen(Stl[m]);
       if (j >= 1) {
         const int cell = (axis_comp(2, a, b, j - 1, pb, pc) * N + axis_comp(1, a, b, j - 1, pb, pc)) * N +
                          axis_comp(0, a, b, j - 1, pb, pc);
@@ -310,7 +309,7 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
 #pragma unroll
       for (int k = 0; k < F; ++k) fprev[k] = fd[k];
 #pragma unroll
-      for (int m = 0; m < 3; ++m) trprev[m] = (double)Str[m];
+      for (int m = 0; m < 3; ++m) trprev[m] = widen(Str[m]);
       if (A.face_flux && (j == 0 || j == N)) {
         // tile boundary face: sums and the torque about the interior cell
         const int f = 2 * a + (j == N ? 1 : 0);
@@ -332,8 +331,10 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
     const int x = c % N, y = (c / N) % N, z = c / (N * N);
     finish_cell(
         A, io, sub, offx, offy, x, y, z,
-        [&](int q) { return __dadd_rn(D[(0 * DQ + q) * N3 + c], D[(1 * DQ + q) * N3 + c]); },
-        [&](int q) { return D[(2 * DQ + q) * N3 + c]; }, hd, inv_h, o);
+        [&](int q) {
+          return __dadd_rn(__dadd_rn(D[(0 * DQ + q) * N3 + c], D[(1 * DQ + q) * N3 + c]), D[(2 * DQ + q) * N3 + c]);
+        },
+        hd, inv_h, o);
   }
   if (tid == 0) {
     float m = red[0];

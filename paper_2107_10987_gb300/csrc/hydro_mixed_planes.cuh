@@ -126,7 +126,7 @@ __device__ __forceinline__ void plane_line(const float* __restrict__ ring, int i
     samples(fs, fs, v);
     const float eta = (kContact && contact) ? contact_eta32(v[0].x, v[1].x, v[2].x, v[3].x, v[4].x) : 0.f;
     if (kContact)
-      ppm32x2<true>(v[0], v[1], v[2], v[3], v[4], qp, qm, f2(eta));
+      ppm32x2<1>(v[0], v[1], v[2], v[3], v[4], qp, qm, f2(eta));
     else
       ppm32x2(v[0], v[1], v[2], v[3], v[4], qp, qm);
     put(fs, qp.x, qm.x);
@@ -208,8 +208,9 @@ __device__ __forceinline__ void mixed_subgrid_planes(const StepArgs64& A, const 
     const double* zu = zsum + (size_t)((p + 1) % 3) * 16 * N * N + c2;  // face p+1/2: upper face of p
     const double* zl = zsum + (size_t)(p % 3) * 16 * N * N + c2;        // face p-1/2: lower face of p
     finish_cell(
-        A, io, sub, offx, offy, c2 % N, c2 / N, p, [&](int q) { return a01[q * N * N]; },
-        [&](int q) { return __dsub_rn(zu[q * N * N], zl[(q < F ? q : q + 3) * N * N]); }, hd, inv_h, o);
+        A, io, sub, offx, offy, c2 % N, c2 / N, p,
+        [&](int q) { return __dadd_rn(a01[q * N * N], __dsub_rn(zu[q * N * N], zl[(q < F ? q : q + 3) * N * N])); },
+        hd, inv_h, o);
   };
 
   // ---- planes 0..4 of the padded sub-grid, straight into the ring --------
