@@ -160,9 +160,10 @@ int hydro_set_mode(hydro_ctx_t* ctx, const hydro_mode_t* mode);
  * (upper) of axis a; per face cell [c][b] (b < c the transverse axes) the F
  * face-averaged fluxes and the 3 components of the momentum-flux torque
  * about the adjacent interior cell.
- * Scratch (context-owned, allocated on first need and kept): per persistent
- * CTA 159,744 bytes of flux differences, and in FP64 mode 2,496,000 bytes of
- * line-end buffer (380 MB for one CTA per SM on a 152-SM GPU).
+ * Scratch (context-owned, allocated on first need and kept): in mixed
+ * precision 159,744 bytes of flux differences per persistent CTA; in FP64 mode
+ * 2,936,704 bytes of line ends, face sums and primitives per team of CTAs
+ * (446 MB for one CTA per SM on a 152-SM GPU).
  * Errors: EINVAL (NULL ctx/batch/pointers, n_sub < 0, misaligned U, dt < 0),
  * ENOMEM, ECUDA.
  * n_sub == 0 is a no-op. */
@@ -176,18 +177,22 @@ int hydro_step(hydro_ctx_t* ctx, const hydro_batch_t* B, double dt, double* dUdt
  *                        precision); the edge lines of a cell are
  *                        reconstructed in two axis sweeps and the vertex lines
  *                        in three (27 line evaluations per cell).  The
- *                        learned indicator uses it; the default.  The FP64
+ *                        learned indicator uses it.  The FP64
  *                        form (ROWS or AUTO; PLANES is mixed only) walks
  *                        each of the 13 lines once per cell along its own
- *                        direction into a per-CTA buffer, then sweeps the
- *                        faces by rows.
+ *                        direction into a buffer, then sums the faces; where
+ *                        the batch does not fill whole rounds of the SMs,
+ *                        teams of CTAs share a sub-grid.
  *   HYDRO_DECOMP_PLANES  mixed precision: the sub-grid swept plane by plane
- *                        along z by 768 threads (one CTA per SM), each of the
+ *                        along z by 640 threads (one CTA per SM), each of the
  *                        13 lines through a cell reconstructed once, the
- *                        primitives in a ring of six planes staged from
- *                        global memory one step ahead, the per-axis flux
- *                        differences kept on chip.
- *   HYDRO_DECOMP_AUTO    the autotuner's choice, else the default. */
+ *                        primitives in a ring of six planes that arrive
+ *                        one step ahead.
+ *   HYDRO_DECOMP_AUTO    the autotuner's choice, else by the number of 8^3
+ *                        tiles: the plane sweep where its rounds of one tile
+ *                        per SM take less than the row sweep's of two (at most
+ *                        one tile per SM, and just above whole rounds), else
+ *                        the row sweep. */
 #define HYDRO_DECOMP_AUTO 0
 #define HYDRO_DECOMP_ROWS 1
 #define HYDRO_DECOMP_PLANES 2
@@ -213,7 +218,8 @@ int hydro_autotune_step(hydro_ctx_t* ctx, const hydro_batch_t* B, double* dUdt, 
 int hydro_set_launch(hydro_ctx_t* ctx, int decomposition, int ctas);
 
 /* The launch shape the context's next step will use in its current
- * precision: *decomposition (ROWS or PLANES) and *ctas (either nullable). */
+ * precision over a large batch: *decomposition (ROWS or PLANES) and *ctas
+ * (either nullable). */
 int hydro_get_launch(const hydro_ctx_t* ctx, int* decomposition, int* ctas);
 
 /* SSP-RK3 stage update of the interior cells (ghosts are not touched):
@@ -361,8 +367,8 @@ typedef struct {
   /* Adaptive mesh (NULL: the uniform nbx x nby x nbz mesh above).  With a mesh
    * each stage runs hydro_fill_ghosts_amr, hydro_step with face_flux and
    * hydro_flux_correct_amr instead of the uniform ghost fill (nbx, nby, nbz
-   * and bc are then ignored).  In HYDRO_PREC_MIXED with 8^3 leaves and the
-   * row sweep (no contact steepening or spin feedback) the fill only
+   * and bc are then ignored).  In HYDRO_PREC_MIXED with 8^3 leaves
+   * (no contact steepening or spin feedback) the fill only
    * prolongs the ghost cells inside coarser leaves and the step reads the
    * others where they live: a same-level leaf's interior, or the mean of
    * the eight children in a finer leaf, from a restriction image of every

@@ -11,7 +11,7 @@
 #include "hydro_ctx.h"
 
 namespace hyd {
-cudaError_t launch_step_mixed_amr(const StepArgs64& A, const AMRArgs& M, int grid, cudaStream_t st);
+cudaError_t launch_step_mixed_amr(const StepArgs64& A, const AMRArgs& M, int grid, int planes, cudaStream_t st);
 cudaError_t launch_step_fp64_lines(const StepArgs64& A, int teams, int T, unsigned* sync, int nn, cudaStream_t st);
 cudaError_t prepare_step_fp64_lines();
 size_t step_fp64_lines_per_team();
@@ -94,20 +94,29 @@ static int ensure_buf(hydro_ctx* c, double** buf, size_t* have, size_t need, con
   return HYDRO_OK;
 }
 
-// The sub-grid decomposition a step of this context runs: the row sweep
-// unless the plane sweep was chosen (by hydro_set_launch or the autotuner;
-// mixed precision without the learned indicator only).
-static int eff_decomp(const hydro_ctx* c) {
+// The sub-grid decomposition a step of this context over `units` tiles runs
+// (mixed precision; FP64 and the learned indicator have the row sweep): what
+// hydro_set_launch or the autotuner chose, else the one whose rounds over the
+// SMs take less.  The plane sweep has one tile per SM at a time, 95 us each;
+// the row sweep two, 166 us for both, or 155 us where the last round leaves a
+// tile alone on its SM.  So planes up to one tile per SM and, on 152 SMs, from
+// 305 to 456 and from 609 to 760 tiles.
+static int eff_decomp(const hydro_ctx* c, int units) {
   if (c->mode.precision != HYDRO_PREC_MIXED || c->gate_on) return HYDRO_DECOMP_ROWS;
-  return c->decomp == HYDRO_DECOMP_PLANES ? HYDRO_DECOMP_PLANES : HYDRO_DECOMP_ROWS;
+  if (c->decomp != HYDRO_DECOMP_AUTO) return c->decomp;
+  const long sms = c->num_sms, full = units / (2 * sms), rest = units % (2 * sms);
+  const long planes_us = 95 * ((units + sms - 1) / sms);
+  const long rows_us = 166 * full + (rest == 0 ? 0 : rest <= sms ? 155 : 172);
+  return planes_us < rows_us ? HYDRO_DECOMP_PLANES : HYDRO_DECOMP_ROWS;
 }
 
-static int step_slots(const hydro_ctx* c, bool mixed) {
+static int step_slots(const hydro_ctx* c, int units) {
   // persistent CTAs: one per SM for FP64 (219 KB of shared memory each) and
-  // for the plane sweep (190 KB, 672 threads), two per SM for the mixed row
-  // sweep (110 KB each), unless the autotuner or the caller chose another
+  // for the plane sweep (230 KB), two per SM for the mixed row sweep (110 KB
+  // each), unless the autotuner or the caller chose another
+  const bool mixed = c->mode.precision == HYDRO_PREC_MIXED;
   if (c->slots_tuned[mixed ? 1 : 0] > 0) return c->slots_tuned[mixed ? 1 : 0];
-  if (!mixed || eff_decomp(c) == HYDRO_DECOMP_PLANES) return c->num_sms;
+  if (!mixed || eff_decomp(c, units) == HYDRO_DECOMP_PLANES) return c->num_sms;
   return 2 * c->num_sms;
 }
 
@@ -193,7 +202,7 @@ int hydro_rk3_fused_enqueue(hydro_ctx* c, const hydro_rk3_desc_t* d, int parity,
   cudaError_t e = hyd::launch_rk3_fused(S, Y, c->u2, reinterpret_cast<float*>(c->prims), d->dt,
                                         reinterpret_cast<unsigned*>(c->sync), d->nbx, d->nby,
                                         d->nbz, d->bc, cfl, c->mode.de_eta2, c->gamma, c->num_sms,
-                                        eff_decomp(c) == HYDRO_DECOMP_PLANES, c->N, st);
+                                        eff_decomp(c, step_units(c, d->a.n_sub)) == HYDRO_DECOMP_PLANES, c->N, st);
   if (e != cudaSuccess) return cuda_fail(e, "hydro_rk3_step (fused)");
   return HYDRO_OK;
 }
@@ -229,8 +238,7 @@ int hydro_ctx_prepare(hydro_ctx* c, int n_sub) {
 }
 
 bool hydro_amr_direct_ok(const hydro_ctx* c) {
-  return c->N == hyd::N && c->mode.precision == HYDRO_PREC_MIXED && !c->mode.contact && !c->mode.spin &&
-         eff_decomp(c) == HYDRO_DECOMP_ROWS;
+  return c->N == hyd::N && c->mode.precision == HYDRO_PREC_MIXED && !c->mode.contact && !c->mode.spin;
 }
 
 int hydro_ctx_prepare_amr(hydro_ctx* c, int n_sub) {
@@ -258,14 +266,14 @@ int hydro_step_amr_direct(hydro_ctx* c, const hydro_batch_t* B, const hydro_amr_
   if (!aligned16(B->U) || !aligned16(dUdt)) return HYDRO_EINVAL;
   int rc = hydro_ctx_prepare_amr(c, B->n_sub);
   if (rc) return rc;
-  const int slots = step_slots(c, true);
+  const int slots = step_slots(c, B->n_sub);
   const int grid = B->n_sub < slots ? B->n_sub : slots;
   rc = ensure_buf(c, &c->scratch, &c->scratch_bytes, (size_t)grid * hyd::kScratchPerSub * sizeof(double),
                   "cudaMalloc(step scratch)");
   if (rc) return rc;
   const hyd::StepArgs64 A = step_args(c, B, dUdt, amax, face_flux);
   const hyd::AMRArgs Am = hydro_amr_args(c, B, M);
-  const cudaError_t e = hyd::launch_step_mixed_amr(A, Am, grid, st);
+  const cudaError_t e = hyd::launch_step_mixed_amr(A, Am, grid, eff_decomp(c, B->n_sub) == HYDRO_DECOMP_PLANES, st);
   if (e != cudaSuccess) return cuda_fail(e, "hydro_step_amr_direct");
   return HYDRO_OK;
 }
@@ -331,13 +339,13 @@ int hydro_step(hydro_ctx_t* c, const hydro_batch_t* B, double dt, double* dUdt, 
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
   if (mixed) {
-    const int slots = step_slots(c, mixed);
+    const int slots = step_slots(c, units);
     const int grid = units < slots ? units : slots;
     rc = ensure_buf(c, &c->scratch, &c->scratch_bytes, (size_t)grid * hyd::kScratchPerSub * sizeof(double),
                     "cudaMalloc(step scratch)");
     if (rc) return rc;
-    e = hyd::launch_step_mixed(step_args(c, B, dUdt, amax, face_flux), grid, eff_decomp(c) == HYDRO_DECOMP_PLANES,
-                               c->N, st);
+    e = hyd::launch_step_mixed(step_args(c, B, dUdt, amax, face_flux), grid,
+                               eff_decomp(c, units) == HYDRO_DECOMP_PLANES, c->N, st);
   } else {
     rc = ensure_lines(c, units);
     if (rc) return rc;
@@ -423,7 +431,7 @@ int hydro_autotune_step(hydro_ctx_t* c, const hydro_batch_t* B, double* dUdt, do
     c->decomp = decomp0;
     c->slots_tuned[idx] = 0;
   }
-  if (slots_out) *slots_out = rc == HYDRO_OK ? step_slots(c, mixed) : 0;
+  if (slots_out) *slots_out = rc == HYDRO_OK ? step_slots(c, step_units(c, B->n_sub)) : 0;
   return rc;
 }
 
@@ -441,9 +449,9 @@ int hydro_set_launch(hydro_ctx_t* c, int decomposition, int ctas) {
 
 int hydro_get_launch(const hydro_ctx_t* c, int* decomposition, int* ctas) {
   if (!c) return HYDRO_EINVAL;
-  const bool mixed = c->mode.precision == HYDRO_PREC_MIXED;
-  if (decomposition) *decomposition = eff_decomp(c);
-  if (ctas) *ctas = step_slots(c, mixed);
+  const int many = 1 << 30;  // without a batch: a large one
+  if (decomposition) *decomposition = eff_decomp(c, many);
+  if (ctas) *ctas = step_slots(c, many);
   return HYDRO_OK;
 }
 

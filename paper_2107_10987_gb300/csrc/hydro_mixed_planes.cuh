@@ -1,37 +1,52 @@
 // hydro_mixed_planes.cuh -- one sub-grid of the mixed-precision hydro step as
-// a plane sweep: each of the 13 lines through a cell is reconstructed once.
+// a plane sweep: each of the 13 lines through a cell is reconstructed once,
+// and what a flux needs of a line's end is computed once with it.
 //
 // The row sweep (hydro_mixed_body.cuh) gives every thread one row of cells
 // along one axis and reconstructs, at each cell of the row, the 9 lines that
-// cross its faces of that axis: the edge lines of a cell are evaluated in two
-// axis sweeps and the vertex lines in three, 27 line evaluations per cell for
-// 13 distinct lines.  Here one CTA of kThreadsPl threads sweeps the sub-grid
-// plane by plane along z (k = -1 .. N), each step in three phases separated
-// by two barriers:
+// cross its faces of that axis: 27 line evaluations per cell for 13 distinct
+// lines, and the sound speed and energy of an edge's or corner's state once
+// per face at it, 54 per cell for 26.  Here one CTA of kThreadsPl threads per
+// SM sweeps the sub-grid plane by plane along z (k = -1 .. N), each step in
+// two phases:
 //   A  reconstruct plane k: the 13 lines of its interior cells, the 9 lines
 //      of the face-adjacent ghost cells around it (x = -1, N and y = -1, N)
 //      and, on the planes k = -1 and N, the 9 lines that cross the z-faces;
-//      both interface values of every line go to shared memory (R), the
-//      values towards +z into one of two z-buffers (Zp) that the next step
-//      reads;
+//      both ends of every line go to shared memory as records of 13 floats
+//      (rho v | E tau p c^2 | z species | 1/c), the ends towards +z into one of
+//      two z-buffers that the next step reads;
 //   B  the fluxes of the x- and y-faces of plane k and of the z-faces between
-//      planes k-1 and k, three threads per face (the face's three groups
-//      of points, combined by warp shuffles in the fixed order), into face-sum
-//      buffers (converted to FP64 once per face); meanwhile the primitives of
-//      plane k+3 are converted from the FP64 staging buffer that phase A
-//      filled from global memory, and two of the warps that have no face
-//      finish plane k-2: its z-differences, the divergence and the sources,
-//      and its dU/dt is stored (finish_cell);
-//   C  per cell of plane k, the FP64 x- and y-differences of face sums.
-// The primitives live in a ring of six FP32 planes (the five planes a line
-// of plane k reaches, and the one being converted), so the CTA holds about
-// 190 KB of shared memory instead of the whole padded sub-grid and runs 21
-// warps on its SM; the per-axis flux differences never leave the SM.
+//      planes k-1 and k, one thread per group of a face's points (the groups
+//      of its summation order, listed group by group so that a warp's threads
+//      have equal work), into group sums in shared memory; meanwhile the next
+//      primitive plane arrives;
+//   C  (in the interval of phase A of the next step) per cell and quantity, the
+//      FP64 differences of the face sums: x plus y of plane k, and z of plane
+//      k - 1, whose total goes to the CTA's scratch in global memory; two steps
+//      later two warps finish the plane from there (divergence, sources and
+//      update: finish_cell).
+// The FP64 pipe takes 16 cycles for a warp's instruction, so its work (C, the
+// finish, the conversion of the next plane's state) is spread over the steps,
+// beside the lines' FP32 work of other warps, and C's operands are widened on
+// the integer pipes.
+//
+// What bounds it: the latency of its intervals with 20 warps and one tile per
+// SM (phase A alone 25 us of a tile's 95, the face fluxes 14, phase C 15, the
+// conversion of a padded FP64 state 14, the first planes and the last finish
+// 25; measured with the others left out).  A row sweep with two tiles on the
+// SM overlaps them and takes 83 us a tile, but 160 for one alone, so the
+// dispatch gives this sweep the batches of at most one tile per SM (77 leaves
+// with contact steepening and spin: 173 -> 101 us).  Two fields of a line share
+// each packed instruction in phase A, and two fields of a point in phase B:
+// the records' float4 quarters are register pairs as they are loaded.  The
+// primitives live in a ring of six FP32 planes (the five planes a line of
+// plane k reaches, and the one arriving), so the CTA holds 225 KB of shared
+// memory.
 //
 // The arithmetic is the row sweep's own: the same ppm32x2 on the same samples
 // (exactly symmetric under reversal of a line, so the orientation in which a
 // line is evaluated does not matter; each lane rounds alike whichever field
-// or line shares its instruction), the same point_pair32 on the same pairs
+// or line shares its instruction), the same point flux on the same pairs
 // in the same order, the same grouping of
 // each face sum, the same FP64 differences and finish_cell.  The two
 // decompositions therefore give the same bits.
@@ -42,138 +57,224 @@
 
 namespace hyd {
 
-// 24 warps, one CTA per SM.  (The register file is shared out per scheduler:
-// 21 warps would be charged as 24, at the same 80 registers a thread.)
-constexpr int kThreadsPl = 768;
+// 20 warps, one CTA per SM, at 96 registers a thread: phase A's 35 warps of
+// lines are two rounds, with phase C's second items on the warps that have one
+// line; phase B's 21 warps of face groups go one to a warp, the last beside
+// another of two points.
+constexpr int kThreadsPl = 640;
 constexpr int kWarpsPl = kThreadsPl / 32;
 constexpr int kPl = S * S;                // 196 cells of a padded plane
 constexpr int kRing = 6;                  // primitive planes held
-constexpr int kRowR = N * N + 1;          // interior cells of a plane, padded for the banks
-constexpr int kRowB = N + 1;              // face-adjacent ghost cells along a side, padded
+constexpr int kNN = N * N;                // 64 cells of an interior plane
 constexpr int kNFaceXY = 2 * (N + 1) * N; // x- and y-faces of a plane (144)
-// Phase B: 10 faces per warp, the 208 faces of a plane on warps 0 .. 20;
-// warps 21 and 22 finish an earlier plane meanwhile.
-constexpr int kFinishT0 = 21 * 32;
-static_assert((kNFaceXY + N * N + 9) / 10 <= kFinishT0 / 32 && kFinishT0 + N * N <= kThreadsPl, "phase B warps");
+constexpr int kNFace = kNFaceXY + kNN;    // and the z-faces below it (208)
+constexpr int kFaceWarps = (kNFace + 31) / 32;  // 7
+constexpr int kSlots = 36;                // line-end slots of a plane's cells (r_slot)
+// A slot holds the records of one direction's ends at the 64 cells of a plane
+// (kBndB: at the 8 ghost cells along a side): three float4 quarters, then 1/c.
+constexpr int kSlotB = 52 * kNN, kBndB = 52 * N;
 
 // Shared-memory layout of one CTA (offsets in bytes).
 struct PlaneSmem {
-  static constexpr size_t stage = 0;                                            // double [F][kPl]
-  static constexpr size_t s01 = stage + sizeof(double) * F * kPl;               // double [2][DQ][64]
-  static constexpr size_t ring = s01 + sizeof(double) * 2 * DQ * N * N;         // float [kRing][F][kPl]
-  static constexpr size_t rint = ring + sizeof(float) * kRing * F * kPl;        // float [17][F][kRowR]
-  static constexpr size_t zp = rint + sizeof(float) * 17 * F * kRowR;           // float [2][9][F][kRowR]
-  static constexpr size_t rbnd = zp + sizeof(float) * 2 * 9 * F * kRowR;        // float [4][9][F][kRowB]
-  static constexpr size_t fs = rbnd + sizeof(float) * 4 * 9 * F * kRowB;        // double [16][kNFaceXY]
-  static constexpr size_t zs = fs + sizeof(double) * 16 * kNFaceXY;             // double [3][16][64]
-  static constexpr size_t coord = zs + sizeof(double) * 3 * 16 * N * N;         // float [2][N + 2]
-  static constexpr size_t red = coord + sizeof(float) * 2 * (N + 2);            // float [kWarpsPl]
-  static constexpr size_t total = red + sizeof(float) * kWarpsPl;
+  static constexpr int ring = 0;                                    // float2 [kRing][5][kPl]
+  static constexpr int ends = ring + 8 * kRing * 5 * kPl;           // [kSlots] of kSlotB bytes
+  static constexpr int bnd = ends + kSlots * kSlotB;                // [4][9] of kBndB bytes
+  static constexpr int sums = bnd + 4 * 9 * kBndB;                  // float [3][F + 3][kNFace]
+  static constexpr int coord = sums + 4 * 3 * (F + 3) * kNFace;     // float [2][N + 2]
+  static constexpr int red = coord + 4 * 2 * (N + 2);               // float [kWarpsPl]
+  static constexpr int stage = (red + 4 * kWarpsPl + 15) / 16 * 16; // double [F][kPl] (Io without primitives)
+  static constexpr int total = stage + 8 * F * kPl;
 };
 constexpr size_t kPlaneSmemBytes = PlaneSmem::total;
 static_assert(kPlaneSmemBytes <= 227 * 1024, "plane sweep shared memory");
 
 // Direction code of d in {-1,0,1}^3: (dz+1)*9 + (dy+1)*3 + (dx+1); 13 is 0.
-__device__ __forceinline__ int dcode(int dx, int dy, int dz) { return (dz + 1) * 9 + (dy + 1) * 3 + (dx + 1); }
+// The ends of a plane's interior cells lie in slot `code`, those towards +z
+// (code >= 18) in slot code or code + 9 by the parity of the plane.
+__device__ __forceinline__ int r_slot(int code, int k) { return code + (code >= 18 ? 9 * (k & 1) : 0); }
+// Ghost cells: side sd (0: x = -1, 1: x = N, 2: y = -1, 3: y = N), the side's
+// 9 directions into the sub-grid bi = (u2+1)*3 + (u1+1) ((+-1, u1, u2) for x
+// sides, (u1, +-1, u2) for y sides), position pos along the side.
+__device__ __forceinline__ int bnd_off(int sd, int bi, int pos) { return (sd * 9 + bi) * kBndB + 16 * pos; }
 
-// Where R[d] of interior cell `cell` (y*8 + x) of plane k lives: directions
-// towards +z (code >= 18) in the z-buffer of the plane's parity, the other
-// 17 in rint.  Returns the address of field 0; fields are kRowR apart.
-__device__ __forceinline__ float* r_int_slot(float* rint, float* zp, int code, int k, int cell) {
-  if (code >= 18) return zp + ((size_t)((k & 1) * 9 + code - 18) * F) * kRowR + cell;
-  return rint + ((size_t)(code < 13 ? code : code - 1) * F) * kRowR + cell;
-}
-// R[d] of a face-adjacent ghost cell of side sd (0: x = -1, 1: x = N, 2:
-// y = -1, 3: y = N) at position pos along the side; the side's 9 directions
-// point into the sub-grid: (+-1, u1, u2) for x sides, (u1, +-1, u2) for y
-// sides, bi = (u2+1)*3 + (u1+1).
-__device__ __forceinline__ float* r_bnd_slot(float* rbnd, int sd, int bi, int pos) {
-  return rbnd + ((size_t)(sd * 9 + bi) * F) * kRowB + pos;
+// Lane l of a warp that covers half of an 8 x 8 plane (half hf): x runs
+// fastest and the two rows a half-warp reads as 8-byte pairs are four rows
+// (448 bytes of the ring) apart, on the other half of the banks.
+__device__ __forceinline__ int half_cell(int l, int hf) {
+  const int y = ((l >> 3) & 1) * 4 + (l >> 4) + 2 * hf;
+  return y * N + (l & 7);
 }
 
-// Reconstruct one line of the cell at padded plane coordinates (ix, iy) of
-// padded plane zp along (dx, dy, dz), for the five fields f0 .. f0 + 4 (f0 =
-// 0 or 5): both interface values of each, to dp (towards +d) and dm (towards
-// -d; nullptr: not needed), field stride fst (dp, dm address field 0).
-// Samples from the primitive ring.  kContact as line10fc.
+// One work item of phase A: the line of the cell at padded plane coordinates
+// (ix, iy) along (dx, dy, dz); zo: the ring offsets of the planes k-2 .. k+2.
+// dp, dm: the records of the ends towards +d and -d (dm null: not needed), of
+// position pos among cnt (the slot's cells).  kContact as line10fc: the
+// density and species lines (lane x of pair 0, lane y of pair 4) are
+// steepened.
 template <bool kContact, bool kSpin>
-__device__ __forceinline__ void plane_line(const float* __restrict__ ring, int ix, int iy, int zp, int dx, int dy,
-                                           int dz, int f0, float* dp, float* dm, int fst, const StepParamsF& PF) {
-  int off[5];
+__device__ __forceinline__ void plane_line(const float2* __restrict__ ring, int ix, int iy, const int zo[5], int dx,
+                                           int dy, int dz, unsigned char* dp, unsigned char* dm, int pos, int cnt,
+                                           const StepParamsF& PF) {
+  const float2* v[5];
+  const int c = iy * S + ix, cd = dy * S + dx;
 #pragma unroll
-  for (int m = 0; m < 5; ++m)
-    off[m] = ((zp + (m - 2) * dz) % kRing) * (F * kPl) + (iy + (m - 2) * dy) * S + (ix + (m - 2) * dx);
+  for (int m = 0; m < 5; ++m) v[m] = ring + ((dz == 0 ? zo[2] : dz > 0 ? zo[m] : zo[4 - m]) + c + (m - 2) * cd);
   bool contact = false;
   if (kContact)
-    contact = contact_line32(ring[off[1] + RHO * kPl], ring[off[3] + RHO * kPl],
-                             __fmul_rn(PF.gm1, ring[off[1] + EGAS * kPl]),
-                             __fmul_rn(PF.gm1, ring[off[3] + EGAS * kPl]), __fmul_rn(PF.gamma, 0.1f));
-  // the five samples of fields fa and fb as pairs
-  auto samples = [&](int fa, int fb, float2 v[5]) {
-#pragma unroll
-    for (int m = 0; m < 5; ++m) v[m] = f2(ring[off[m] + fa * kPl], ring[off[m] + fb * kPl]);
-  };
-  auto put = [&](int f, float qp, float qm) {
-    dp[f * fst] = qp;
-    if (dm) dm[f * fst] = qm;
-  };
-  // fields 0 .. 4: the density alone (the steepened field), then (1, 2) and
-  // (3, 4); fields 5 .. 9: (5, 6), (7, 8), then the species alone
-  static_assert(RHO == 0 && SP0 == F - 1 && F == 10, "field split of a half line");
-  const int fs = f0 == 0 ? RHO : SP0;
-  {
-    float2 v[5], qp, qm;
-    samples(fs, fs, v);
-    const float eta = (kContact && contact) ? contact_eta32(v[0].x, v[1].x, v[2].x, v[3].x, v[4].x) : 0.f;
-    if (kContact)
-      ppm32x2<1>(v[0], v[1], v[2], v[3], v[4], qp, qm, f2(eta));
-    else
-      ppm32x2(v[0], v[1], v[2], v[3], v[4], qp, qm);
-    put(fs, qp.x, qm.x);
-  }
-  // the cell's spin fed back into the velocity at both ends (spin_dv32; the
-  // row sweep's values, bit for bit)
-  float dv[3] = {0.f, 0.f, 0.f};
-  const bool spin = kSpin && f0 == 0;
-  if (spin)
-    spin_dv32(ring[off[2] + RHO * kPl], ring[off[2] + EGAS * kPl], ring[off[2] + ZX * kPl], ring[off[2] + ZY * kPl],
-              ring[off[2] + ZZ * kPl], PF.k3h, __fmul_rn(PF.gamma, PF.gm1), dx, dy, dz, dv);
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int fa = (f0 == 0 ? 1 : 5) + 2 * i;
-    float2 v[5], qp, qm;
-    samples(fa, fa + 1, v);
-    ppm32x2(v[0], v[1], v[2], v[3], v[4], qp, qm);
-    if (spin) {
-      // fields 1, 2 (i = 0) and 3 (i = 1) are the velocity
-      qp.x = __fadd_rn(qp.x, dv[2 * i]);
-      qm.x = __fsub_rn(qm.x, dv[2 * i]);
-      if (i == 0) {
-        qp.y = __fadd_rn(qp.y, dv[1]);
-        qm.y = __fsub_rn(qm.y, dv[1]);
-      }
+    contact = contact_line32(v[1][0].x, v[3][0].x, __fmul_rn(PF.gm1, v[1][2 * kPl].x),
+                             __fmul_rn(PF.gm1, v[3][2 * kPl].x), __fmul_rn(PF.gamma, 0.1f));
+  // pair f (fields 2f, 2f + 1)
+  auto pair = [&](auto fc, float2& qp, float2& qm) {
+    constexpr int f = decltype(fc)::value;
+    const float2 s0 = v[0][f * kPl], s1 = v[1][f * kPl], s2 = v[2][f * kPl], s3 = v[3][f * kPl], s4 = v[4][f * kPl];
+    if constexpr (kContact && (f == 0 || f == 4)) {
+      const float eta = !contact ? 0.f
+                        : f == 0 ? contact_eta32(s0.x, s1.x, s2.x, s3.x, s4.x)
+                                 : contact_eta32(s0.y, s1.y, s2.y, s3.y, s4.y);
+      ppm32x2<f == 0 ? 2 : 3>(s0, s1, s2, s3, s4, qp, qm, f2(eta));
+    } else {
+      ppm32x2(s0, s1, s2, s3, s4, qp, qm);
     }
-    put(fa, qp.x, qm.x);
-    put(fa + 1, qp.y, qm.y);
+  };
+  using std::integral_constant;
+  auto quarter = [&](unsigned char* d, int i, float2 a, float2 b) {
+    *reinterpret_cast<float4*>(d + i * 16 * cnt) = make_float4(a.x, a.y, b.x, b.y);
+  };
+  float2 p0, m0, p1, m1, p2, m2;
+  pair(integral_constant<int, 3>{}, p0, m0);
+  pair(integral_constant<int, 4>{}, p1, m1);
+  quarter(dp, 2, p0, p1);
+  if (dm) quarter(dm, 2, m0, m1);
+  pair(integral_constant<int, 0>{}, p0, m0);
+  pair(integral_constant<int, 1>{}, p1, m1);
+  if constexpr (kSpin) {
+    // the cell's spin fed back into the velocity at both ends (spin_dv32;
+    // the row sweep's values, bit for bit)
+    float dv[3];
+    spin_dv32(v[2][0].x, v[2][2 * kPl].x, v[2][3 * kPl].x, v[2][3 * kPl].y, v[2][4 * kPl].x, PF.k3h,
+              __fmul_rn(PF.gamma, PF.gm1), dx, dy, dz, dv);
+    p0.y = __fadd_rn(p0.y, dv[0]);
+    m0.y = __fsub_rn(m0.y, dv[0]);
+    p1.x = __fadd_rn(p1.x, dv[1]);
+    m1.x = __fsub_rn(m1.x, dv[1]);
+    p1.y = __fadd_rn(p1.y, dv[2]);
+    m1.y = __fsub_rn(m1.y, dv[2]);
   }
+  quarter(dp, 0, p0, p1);
+  if (dm) quarter(dm, 0, m0, m1);
+  pair(integral_constant<int, 2>{}, p2, m2);
+  // E, p, c^2 and 1/c of an end (side32x2's operations)
+  auto end = [&](unsigned char* d, float2 q0, float2 q1, float2 q2) {
+    const float v2 = __fmaf_rn(q1.y, q1.y, __fmaf_rn(q1.x, q1.x, __fmul_rn(q0.y, q0.y)));
+    const float E = __fmaf_rn(__fmul_rn(0.5f, q0.x), v2, q2.x);
+    const float p = __fmul_rn(PF.gm1, q2.x);
+    const float c2 = __fdividef(__fmul_rn(PF.gamma, p), q0.x);
+    quarter(d, 1, f2(E, q2.y), f2(p, c2));
+    *reinterpret_cast<float*>(d + 48 * cnt - 12 * pos) = rsqrtf(c2);
+  };
+  end(dp, p0, p1, p2);
+  if (dm) end(dm, m0, m1, m2);
 }
 
+// One face side of a thread's points: where the record of point (u1, u2)
+// lies, base + u1 s1 + u2 s2 + (u2 == 1 ? s3 : 0) bytes, quarters qst bytes
+// apart, its 1/c at dr.
+struct SideRef {
+  const unsigned char* base;
+  int s1, s2, s3, qst, dr;
+  template <int u1, int u2>
+  __device__ __forceinline__ void load(float4 q[3], float& rs) const {
+    const unsigned char* p = base + u1 * s1 + u2 * s2 + (u2 == 1 ? s3 : 0);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) q[i] = *reinterpret_cast<const float4*>(p + i * qst);
+    rs = *reinterpret_cast<const float*>(p + dr);
+  }
+};
+
+// One quadrature point of a face (point_pair32's operations on one point,
+// two fields in the two lanes), added to a group's sums G (field pairs) and
+// the torque about the left cell TL.  w: the point's weight.
+template <int u1, int u2>
+__device__ __forceinline__ void plane_point(const SideRef& sl, const SideRef& sr, int a, float om, float r,
+                                            float half_h, float w, float2 G[5], float TL[3], float& amax) {
+  float4 L[3], R[3];
+  float rsL, rsR;
+  sl.load<u1, u2>(L, rsL);
+  sr.load<u1, u2>(R, rsR);
+  const float hw = 0.5f * w, hq = 0.5f * __fmul_rn(w, half_h);
+  const float vaL = a == 0 ? L[0].y : a == 1 ? L[0].z : L[0].w, vaR = a == 0 ? R[0].y : a == 1 ? R[0].z : R[0].w;
+  const float unL = __fmaf_rn(om, r, vaL), unR = __fmaf_rn(om, r, vaR);
+  const float aq = fmaxf(__fmaf_rn(L[1].w, rsL, fabsf(unL)), __fmaf_rn(R[1].w, rsR, fabsf(unR)));
+  amax = fmaxf(amax, aq);
+  const float2 uL2 = f2(unL), uR2 = f2(unR), na2 = f2(-aq), hw2 = f2(hw);
+  const float pp = __fadd_rn(L[1].z, R[1].z);
+  const float pw = __fmaf_rn(L[1].z, vaL, __fmul_rn(R[1].z, vaR));
+  // 2 F_q of two fields with conserved values cL, cR and the pressure term x
+  auto flux = [&](float2 cL, float2 cR, float2 x) {
+    const float2 sum = fma2(cL, uL2, fma2(cR, uR2, x));
+    return fma2(na2, sub2(cR, cL), sum);
+  };
+  auto flux0 = [&](float2 cL, float2 cR) {
+    const float2 sum = fma2(cL, uL2, mul2(cR, uR2));
+    return fma2(na2, sub2(cR, cL), sum);
+  };
+  const float2 f01 = flux(f2(L[0].x, __fmul_rn(L[0].x, L[0].y)), f2(R[0].x, __fmul_rn(R[0].x, R[0].y)),
+                          f2(0.f, a == 0 ? pp : 0.f));
+  const float2 f23 = flux(mul2(f2(L[0].x), f2(L[0].z, L[0].w)), mul2(f2(R[0].x), f2(R[0].z, R[0].w)),
+                          f2(a == 1 ? pp : 0.f, a == 2 ? pp : 0.f));
+  const float2 f45 = flux(f2(L[1].x, L[1].y), f2(R[1].x, R[1].y), f2(pw, 0.f));
+  const float2 f67 = flux0(f2(L[2].x, L[2].y), f2(R[2].x, R[2].y));
+  const float2 f89 = flux0(f2(L[2].z, L[2].w), f2(R[2].z, R[2].w));
+  G[0] = fma2(hw2, f01, G[0]);
+  G[1] = fma2(hw2, f23, G[1]);
+  G[2] = fma2(hw2, f45, G[2]);
+  G[3] = fma2(hw2, f67, G[3]);
+  G[4] = fma2(hw2, f89, G[4]);
+  const float d0 = a == 0 ? 1.f : (float)u1, d1 = a == 1 ? 1.f : (a == 0 ? (float)u1 : (float)u2),
+              d2 = a == 2 ? 1.f : (float)u2;
+  const float fx = f01.y, fy = f23.x, fz = f23.y;
+  TL[0] = __fmaf_rn(hq, __fmaf_rn(d1, fz, __fmul_rn(-d2, fy)), TL[0]);
+  TL[1] = __fmaf_rn(hq, __fmaf_rn(d2, fx, __fmul_rn(-d0, fz)), TL[1]);
+  TL[2] = __fmaf_rn(hq, __fmaf_rn(d0, fy, __fmul_rn(-d1, fx)), TL[2]);
+}
+
+// Phase C's item j (0 or 1) of a thread: the second ones go to the last warps.
+__device__ __forceinline__ int phase_c_item(int tid, int j) {
+  constexpr int kFirst2 = 2 * kThreadsPl - (F + 3) * kNN;  // the first thread with a second item
+  static_assert(kFirst2 >= 0 && kFirst2 % 32 == 0, "phase C items");
+  return j == 0 ? tid : tid >= kFirst2 ? kThreadsPl + tid - kFirst2 : (F + 3) * kNN;
+}
+
+// cp.async of 8 or 16 bytes to shared memory, and the wait for all of the
+// thread's copies.
+template <int kBytes>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+  if constexpr (kBytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(kBytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // One 8^3 tile (work unit s) as a plane sweep; Io as for mixed_subgrid, plus
-//   io.load_fields(sub, c, f0, nf, u)   fields f0 .. f0+nf-1 of padded cell c
-// (nf <= 5).  sm: the CTA's dynamic shared memory (kPlaneSmemBytes).  Ends
-// with a barrier.  Must be called by all kThreadsPl threads.
+//   Io::kPrims: io.prim_pairs(sub, c) the five primitive pairs of padded cell
+//     c (float2, io.kPairStride apart);
+//   else, Io::kRows: io.row(sub, k, z, y) the row of field k of the padded
+//     state (14 doubles, 16-byte aligned);
+//   else io.load_fields(sub, c, f0, nf, u), fields f0 .. f0+nf-1 of cell c.
+// sm: the CTA's dynamic shared memory (kPlaneSmemBytes); D: its scratch
+// (kScratchPerSub doubles).  Ends with a barrier.  Must be called by all
+// kThreadsPl threads.
 template <bool kContact, bool kSpin, class Io>
-__device__ __forceinline__ void mixed_subgrid_planes(const StepArgs64& A, const Io& io, int s, unsigned char* sm) {
-  double* stage = reinterpret_cast<double*>(sm + PlaneSmem::stage);
-  double* s01 = reinterpret_cast<double*>(sm + PlaneSmem::s01);
-  float* ring = reinterpret_cast<float*>(sm + PlaneSmem::ring);
-  float* rint = reinterpret_cast<float*>(sm + PlaneSmem::rint);
-  float* zp = reinterpret_cast<float*>(sm + PlaneSmem::zp);
-  float* rbnd = reinterpret_cast<float*>(sm + PlaneSmem::rbnd);
-  double* fsum = reinterpret_cast<double*>(sm + PlaneSmem::fs);
-  double* zsum = reinterpret_cast<double*>(sm + PlaneSmem::zs);
+__device__ __forceinline__ void mixed_subgrid_planes(const StepArgs64& A, const Io& io, int s, unsigned char* sm,
+                                                     double* __restrict__ D) {
+  float2* ring = reinterpret_cast<float2*>(sm + PlaneSmem::ring);
+  unsigned char* ends = sm + PlaneSmem::ends;
+  unsigned char* bnd = sm + PlaneSmem::bnd;
+  float* sums = reinterpret_cast<float*>(sm + PlaneSmem::sums);
   float* coord = reinterpret_cast<float*>(sm + PlaneSmem::coord);
   float* red = reinterpret_cast<float*>(sm + PlaneSmem::red);
+  double* stage = reinterpret_cast<double*>(sm + PlaneSmem::stage);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const typename Io::Sub sub = io.begin(s);
   const int si = io.sidx(sub), offx = io.offx(sub), offy = io.offy(sub);
@@ -181,8 +282,6 @@ __device__ __forceinline__ void mixed_subgrid_planes(const StepArgs64& A, const 
   const StepParamsF PF{(float)A.P.gamma, (float)A.P.gm1, (float)A.P.omega, kSpin ? 1 : 0,
                        kSpin ? (float)(3.0 / hd) : 0.f};
   const float h = (float)hd, half_h = 0.5f * h;
-  const double o[3] = {A.origin[3 * si + 0], A.origin[3 * si + 1], A.origin[3 * si + 2]};
-  const double inv_h = 1.0 / hd;
   const int npt = A.P.face_points;
   float amax = 0.f;
   bool bad = false;
@@ -191,292 +290,334 @@ __device__ __forceinline__ void mixed_subgrid_planes(const StepArgs64& A, const 
   auto convert = [&](const double* u, int z, int q) {
     float pq[F];
     bad |= !prims_mixed(u, A.P.eta1, PF.gamma, pq);
-    float* dst = ring + (size_t)(z % kRing) * F * kPl + q;
+    float2* dst = ring + (z % kRing) * (5 * kPl) + q;
 #pragma unroll
-    for (int f = 0; f < F; ++f) dst[f * kPl] = pq[f];
+    for (int f = 0; f < 5; ++f) dst[f * kPl] = f2(pq[2 * f], pq[2 * f + 1]);
+  };
+  // the asynchronous copies of cell q of padded plane z's primitives
+  auto copy_prims = [&](int z, int q) {
+    if constexpr (Io::kPrims) {
+      const float2* src = io.prim_pairs(sub, z * kPl + q);
+      float2* dst = ring + (z % kRing) * (5 * kPl) + q;
+#pragma unroll
+      for (int f = 0; f < 5; ++f) cp_async<8>(dst + f * kPl, src + (size_t)f * Io::kPairStride);
+    }
   };
 
-  sub_coords(coord, hd, o[0], o[1], offx, offy);
-
-  // dU/dt of plane p (its z-differences from the face sums of p - 1/2 and
-  // p + 1/2, the x- plus y-differences from phase C, finish_cell), on the
-  // 64 threads t0 .. t0 + 63
-  auto finish_plane = [&](int p, int t0) {
-    const int c2 = tid - t0;
-    if (c2 < 0 || c2 >= N * N) return;
-    const double* a01 = s01 + (size_t)(p & 1) * DQ * N * N + c2;
-    const double* zu = zsum + (size_t)((p + 1) % 3) * 16 * N * N + c2;  // face p+1/2: upper face of p
-    const double* zl = zsum + (size_t)(p % 3) * 16 * N * N + c2;        // face p-1/2: lower face of p
-    finish_cell(
-        A, io, sub, offx, offy, c2 % N, c2 / N, p,
-        [&](int q) { return __dadd_rn(a01[q * N * N], __dsub_rn(zu[q * N * N], zl[(q < F ? q : q + 3) * N * N])); },
-        hd, inv_h, o);
-  };
+  {
+    const double ox = A.origin[3 * si + 0], oy = A.origin[3 * si + 1];
+    sub_coords(coord, hd, ox, oy, offx, offy);
+  }
 
   // ---- planes 0..4 of the padded sub-grid, straight into the ring --------
   for (int e = tid; e < 5 * kPl; e += kThreadsPl) {
-    double u[F];
-    io.load_fields(sub, e, 0, 5, u);
-    io.load_fields(sub, e, 5, 5, u + 5);
-    convert(u, e / kPl, e % kPl);
+    if constexpr (Io::kPrims) {
+      copy_prims(e / kPl, e % kPl);
+    } else {
+      double u[F];
+      io.load_fields(sub, e, 0, 5, u);
+      io.load_fields(sub, e, 5, 5, u + 5);
+      convert(u, e / kPl, e % kPl);
+    }
   }
+  if constexpr (Io::kPrims) cp_async_wait();
   __syncthreads();
 
-  // this thread's share of the prefetch of the next padded plane: 5 fields
-  // of one cell
-  const bool pf_on = tid < 2 * kPl;
-  const int pf_q = tid % kPl, pf_f0 = (tid / kPl) * 5;
+  // phase C's items: quantity q (the F fluxes, then the torque's components)
+  // of one cell of the plane; each carries the x plus y difference of the
+  // plane before and the z-face sum below the plane after
+  constexpr int kItems = 2;
+  double d01[kItems];
+  float zlo[kItems];
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    d01[j] = 0.0;
+    zlo[j] = 0.f;
+  }
+  auto phase_c = [&](int k) {
+    // the face's sum (G0 + G1) + G2 of value q (the centre alone with one point)
+    auto total = [&](int q, int face) {
+      const float* g = sums + q * kNFace + face;
+      constexpr int kG = (F + 3) * kNFace;
+      return npt == 1 ? g[2 * kG] : __fadd_rn(__fadd_rn(g[0], g[kG]), g[2 * kG]);
+    };
+    // component m of the torque about the right cell (right_torque32)
+    auto right = [&](int m, int a, int face) {
+      const float tl = total(F + m, face);
+      if (m == a) return tl;
+      const bool plus = m == (a == 2 ? 0 : a + 1);
+      return __fmaf_rn(plus ? h : -h, total(SX + 3 - a - m, face), tl);
+    };
+#pragma unroll
+    for (int j = 0; j < kItems; ++j) {
+      const int i = phase_c_item(tid, j);
+      if (i < (F + 3) * kNN) {
+        const int q = i / kNN, cell = i % kNN, x = cell % N, y = cell / N;
+        auto lower = [&](int a, int face) { return q < F ? total(q, face) : right(q - F, a, face); };
+        const float zu = total(q, kNFaceXY + cell), zl = lower(2, kNFaceXY + cell);
+        if (k >= 1)
+          D[(size_t)q * N3 + (k - 1) * kNN + cell] = __dadd_rn(d01[j], __dsub_rn(widen(zu), widen(zlo[j])));
+        zlo[j] = zl;
+        float xu = 0.f, xl = 0.f, yu = 0.f, yl = 0.f;
+        if (k < N) {
+          const int fx = y * (N + 1) + x, fy = N * (N + 1) + cell;  // the lower faces
+          xu = total(q, fx + 1);
+          xl = lower(0, fx);
+          yu = total(q, fy + N);
+          yl = lower(1, fy);
+          d01[j] = __dadd_rn(__dsub_rn(widen(xu), widen(xl)), __dsub_rn(widen(yu), widen(yl)));
+        }
+        if (A.face_flux) {
+          // sub-grid boundary faces: sums and the torque about the interior cell
+          if (k < N) {
+            if (x == 0) io.face(sub, 0, q, k, y, widen(xl));
+            if (x == N - 1) io.face(sub, 1, q, k, y, widen(xu));
+            if (y == 0) io.face(sub, 2, q, k, x, widen(yl));
+            if (y == N - 1) io.face(sub, 3, q, k, x, widen(yu));
+          }
+          if (k == 0) io.face(sub, 4, q, y, x, widen(zl));
+          if (k == N) io.face(sub, 5, q, y, x, widen(zu));
+        }
+      }
+    }
+  };
 
+  // the copies of padded plane z's state into the stage (Io without
+  // primitives): rows asynchronously, else through this thread's registers
+  double pf[5];
+  const int pf_q = tid % kPl, pf_f0 = (tid / kPl) * 5;
+  auto stage_issue = [&](int z) {
+    if constexpr (Io::kRows) {
+      // 14 rows of 7 16-byte pieces per field
+      for (int i = tid; i < F * kPl / 2; i += kThreadsPl) {
+        const int f = i / (kPl / 2), r = i % (kPl / 2), y = r / (S / 2), x2 = r % (S / 2);
+        cp_async<16>(stage + f * kPl + 2 * r, io.row(sub, f, z, y) + 2 * x2);
+      }
+    } else if constexpr (!Io::kPrims) {
+      if (tid < 2 * kPl) io.load_fields(sub, z * kPl + pf_q, pf_f0, 5, pf);
+    }
+  };
+  auto stage_arrive = [&]() {
+    if constexpr (Io::kRows || Io::kPrims) {
+      cp_async_wait();
+    } else {
+      if (tid < 2 * kPl) {
+#pragma unroll
+        for (int f = 0; f < 5; ++f) stage[(pf_f0 + f) * kPl + pf_q] = pf[f];
+      }
+    }
+  };
+  // the finish of plane p, by the 64 threads t0 .. t0 + 63
+  const double inv_h = 1.0 / hd;
+  auto finish_plane = [&](int p, int t0) {
+    const int c2 = tid - t0, c = p * kNN + c2;
+    if (c2 < 0 || c2 >= kNN) return;
+    const double o[3] = {A.origin[3 * si + 0], A.origin[3 * si + 1], A.origin[3 * si + 2]};
+    finish_cell(A, io, sub, offx, offy, c2 % N, c2 / N, p, [&](int q) { return D[(size_t)q * N3 + c]; }, hd, inv_h, o);
+  };
+  // warps with one line item (the last five) finish a plane (two of them) and
+  // convert the staged one (the others)
+  constexpr int kOneLine = 35 - kWarpsPl;  // 15: the first warp with one item
+  constexpr int kConvT0 = (kOneLine + 2) * 32;
+
+  if constexpr (!Io::kPrims) {
+    stage_issue(5);
+    stage_arrive();
+    __syncthreads();
+  }
 #pragma unroll 1
   for (int k = -1; k <= N; ++k) {
     const int zpk = k + G;  // padded index of plane k
-    double pf[5];
-    const bool pf_do = pf_on && k + 6 < S;  // padded plane k + 6 = plane k + 3
-    if (pf_do) io.load_fields(sub, (k + 6) * kPl + pf_q, pf_f0, 5, pf);
+    // the next padded plane, k + 6 (its ring slot is plane k's own padded
+    // index, which phase A no longer reads)
+    const int znew = k + 6;
+    if constexpr (Io::kPrims) {
+      if (znew < S && tid < kPl) copy_prims(znew, tid);
+    }
 
-    // ---- A: reconstruct plane k ------------------------------------------
-    // work items: a line of one cell for five of its fields (f0 = 0 or 5)
-    if (k >= 0 && k < N) {
-      constexpr int kLines = 13 * N * N + 4 * 9 * N;  // 1120
-      for (int i = tid; i < 2 * kLines; i += kThreadsPl) {
-        const int f0 = i < kLines ? 0 : 5, li = i < kLines ? i : i - kLines;
-        if (li < 13 * N * N) {
-          // line L of interior cell (x, y): canonical direction code 14 + L
-          const int L = li / (N * N), cell = li % (N * N), x = cell % N, y = cell / N;
-          const int code = 14 + L, dx = code % 3 - 1, dy = (code / 3) % 3 - 1, dz = code / 9 - 1;
-          float* dp = r_int_slot(rint, zp, code, k, cell);
-          float* dm = r_int_slot(rint, zp, 26 - code, k, cell);
-          plane_line<kContact, kSpin>(ring, x + G, y + G, zpk, dx, dy, dz, f0, dp, dm, kRowR, PF);
-        } else {
-          // face-adjacent ghost cell: the 9 lines into the sub-grid
-          const int j = li - 13 * N * N, sd = j / (9 * N), bi = (j % (9 * N)) / N, pos = j % N;
-          const int u1 = bi % 3 - 1, u2 = bi / 3 - 1;
-          int x, y, dx, dy;
-          if (sd < 2) {
-            x = sd == 0 ? -1 : N;
-            y = pos;
-            dx = sd == 0 ? 1 : -1;
-            dy = u1;
-          } else {
-            x = pos;
-            y = sd == 2 ? -1 : N;
-            dx = u1;
-            dy = sd == 2 ? 1 : -1;
-          }
-          plane_line<kContact, kSpin>(ring, x + G, y + G, zpk, dx, dy, u2, f0, r_bnd_slot(rbnd, sd, bi, pos), nullptr,
-                               kRowB, PF);
+    // ---- A: reconstruct plane k; C of the step before; the finish of plane
+    // k - 3; the conversion of padded plane k + 6.  The FP64 pipe serves C, the
+    // finish and the conversion while the lines run: even warps take C first.
+    const bool c_first = (warp & 1) == 0;
+    if (k >= 1 && c_first) phase_c(k - 1);
+    const bool inner = k >= 0 && k < N;
+    const int n_int = inner ? (npt == 1 ? 6 : 26) : (npt == 1 ? 2 : 18);     // halves of planes of cells
+    const int n_bnd = inner ? (npt == 1 ? 1 : 9) : 0;                        // 32 ghost-cell lines each
+    int zo[5];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) zo[m] = ((zpk + m - 2) % kRing) * (5 * kPl);
+#pragma unroll 1
+    for (int i = warp; i < n_int + n_bnd; i += kWarpsPl) {
+      int ix, iy, dx, dy, dz, pos, cnt;
+      unsigned char *dp, *dm;
+      if (i < n_int) {
+        const int cell = half_cell(lane, i & 1), L = i >> 1;
+        int code;
+        if (inner)
+          code = npt == 1 ? (L == 0 ? 14 : L == 1 ? 16 : 22) : 14 + L;  // the lines with d's code above 13
+        else
+          code = (k < 0 ? 18 : 0) + (npt == 1 ? 4 : L);  // towards +z from k = -1, towards -z from k = N
+        dx = code % 3 - 1;
+        dy = (code / 3) % 3 - 1;
+        dz = code / 9 - 1;
+        ix = cell % N + G;
+        iy = cell / N + G;
+        pos = cell;
+        cnt = kNN;
+        dp = ends + r_slot(code, k) * kSlotB + 16 * cell;
+        dm = inner ? ends + r_slot(26 - code, k) * kSlotB + 16 * cell : nullptr;
+      } else {
+        // face-adjacent ghost cells: the 9 lines into the sub-grid (the middle
+        // one alone with one point)
+        const int j = (i - n_int) * 32 + lane;
+        const int sd = npt == 1 ? j / N : j / (9 * N), bi = npt == 1 ? 4 : (j / N) % 9;
+        const int u1 = bi % 3 - 1, in = (sd & 1) ? -1 : 1, out = (sd & 1) ? N : -1;
+        pos = j % N;
+        cnt = N;
+        dz = bi / 3 - 1;
+        dx = sd < 2 ? in : u1;
+        dy = sd < 2 ? u1 : in;
+        ix = (sd < 2 ? out : pos) + G;
+        iy = (sd < 2 ? pos : out) + G;
+        dp = bnd + bnd_off(sd, bi, pos);
+        dm = nullptr;
+      }
+      plane_line<kContact, kSpin>(ring, ix, iy, zo, dx, dy, dz, dp, dm, pos, cnt, PF);
+    }
+    if (k >= 1 && !c_first) phase_c(k - 1);
+    if (k >= 3) finish_plane(k - 3, kOneLine * 32);
+    if constexpr (!Io::kPrims) {
+      if (znew < S && tid >= kConvT0) {
+#pragma unroll 1
+        for (int q = tid - kConvT0; q < kPl; q += kThreadsPl - kConvT0) {
+          double u[F];
+#pragma unroll
+          for (int f = 0; f < F; ++f) u[f] = stage[f * kPl + q];
+          convert(u, znew, q);
         }
       }
-    } else {
-      // k = -1: the lines towards +z; k = N: towards -z (interior columns)
-      constexpr int kLines = 9 * N * N;
-      for (int i = tid; i < 2 * kLines; i += kThreadsPl) {
-        const int f0 = i < kLines ? 0 : 5, li = i < kLines ? i : i - kLines;
-        const int zi = li / (N * N), cell = li % (N * N), x = cell % N, y = cell / N;
-        const int dx = zi % 3 - 1, dy = zi / 3 - 1, dz = k < 0 ? 1 : -1;
-        float* dp = r_int_slot(rint, zp, dcode(dx, dy, dz), k, cell);
-        plane_line<kContact, kSpin>(ring, x + G, y + G, zpk, dx, dy, dz, f0, dp, nullptr, kRowR, PF);
-      }
-    }
-    if (pf_do) {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) stage[(pf_f0 + f) * kPl + pf_q] = pf[f];
     }
     __syncthreads();
 
-    // ---- B: face fluxes; conversion of padded plane k + 6 ------------------
+    // ---- B: face fluxes; the copies of the next padded plane --------------------
+    if constexpr (!Io::kPrims) {
+      if (znew + 1 < S) stage_issue(znew + 1);
+    }
     if (k >= 0) {
-      const int slot = warp * 10 + lane / 3, g = lane % 3;
-      // x- and y-faces of plane k (k < N), z-faces between k-1 and k
-      const bool zface = slot >= kNFaceXY;
-      const bool active = lane < 30 && slot < kNFaceXY + N * N && (k < N || zface);
-      float Gf[F], Gtl[3];
-#pragma unroll
-      for (int q = 0; q < F; ++q) Gf[q] = 0.f;
-#pragma unroll
-      for (int m = 0; m < 3; ++m) Gtl[m] = 0.f;
-      int a = 0, fx = 0, fy = 0;  // face axis; the left cell's (x, y) in plane k (or k-1 for z-faces)
-      if (active) {
+      // items: face `slot` for group 0 (points 0-3), 2 (points 6-8), 1 (4, 5);
+      // with one point per face the centre (group 2) alone
+      const int n_faces = k < N ? kNFace : kNN, fw = k < N ? kFaceWarps : kNN / 32;
+      // (a 21st item goes to a warp of the smallest group, of two points)
+      static_assert(3 * kFaceWarps == kWarpsPl + 1, "phase B items");
+#pragma unroll 1
+      for (int wi = warp; wi < (npt == 1 ? fw : 3 * fw);
+           wi = (wi == 2 * kFaceWarps && fw == kFaceWarps) ? 3 * kFaceWarps - 1 : 3 * kFaceWarps) {
+        const int part = npt == 1 ? 1 : wi / fw;  // 0, 1, 2: groups 0, 2, 1
+        const int f = (npt == 1 ? wi : wi % fw) * 32 + lane;
+        if (f >= n_faces) continue;
+        const int slot = k < N ? f : kNFaceXY + f;
+        // the face's axis and its left cell (fx, fy) in plane k (k - 1 for z)
+        int a, fx, fy;
         if (slot < N * (N + 1)) {
           a = 0;
           fy = slot / (N + 1);
           fx = slot % (N + 1) - 1;
-        } else if (!zface) {
+        } else if (slot < kNFaceXY) {
           a = 1;
-          const int t = slot - N * (N + 1);
-          fx = t / (N + 1);
-          fy = t % (N + 1) - 1;
+          const int t = slot - N * (N + 1);  // x fastest: neighbouring lanes read neighbouring cells
+          fx = t % N;
+          fy = t / N - 1;
         } else {
           a = 2;
-          const int t = slot - kNFaceXY;
-          fx = t % N;
-          fy = t / N;
+          fx = (slot - kNFaceXY) % N;
+          fy = (slot - kNFaceXY) / N;
         }
-        // left-cell centre in FP32 (the row sweep's values)
-        const float xc = coord[fx + 1], yc = coord[(N + 2) + fy + 1];
-        // point n of the face: its directions dL, dR (as small integers) and
-        // where its left value R_left[dL] and right value R_right[dR] live
-        struct Pt {
-          const float* pl;
-          const float* pr;
-          int sl, sr, dl[3], dr[3], u1, u2;
-        };
-        auto geom = [&](int n) {
-          Pt t;
-          t.u1 = face_u1(n);
-          t.u2 = face_u2(n);
-          const int u1 = t.u1, u2 = t.u2;
-          // d along (a, b, c) = (1, u1, u2), b < c the transverse axes
-          t.dl[0] = a == 0 ? 1 : u1;
-          t.dl[1] = a == 1 ? 1 : (a == 0 ? u1 : u2);
-          t.dl[2] = a == 2 ? 1 : u2;
-#pragma unroll
-          for (int m = 0; m < 3; ++m) t.dr[m] = m == a ? -1 : t.dl[m];
-          const int cl = dcode(t.dl[0], t.dl[1], t.dl[2]), cr = dcode(t.dr[0], t.dr[1], t.dr[2]);
-          t.sl = t.sr = kRowR;
-          if (a == 0) {
-            const int bi = (u2 + 1) * 3 + (u1 + 1);
-            if (fx < 0) {
-              t.pl = r_bnd_slot(rbnd, 0, bi, fy);
-              t.sl = kRowB;
-            } else {
-              t.pl = r_int_slot(rint, zp, cl, k, fy * N + fx);
-            }
-            if (fx + 1 >= N) {
-              t.pr = r_bnd_slot(rbnd, 1, bi, fy);
-              t.sr = kRowB;
-            } else {
-              t.pr = r_int_slot(rint, zp, cr, k, fy * N + fx + 1);
-            }
-          } else if (a == 1) {
-            const int bi = (u2 + 1) * 3 + (u1 + 1);
-            if (fy < 0) {
-              t.pl = r_bnd_slot(rbnd, 2, bi, fx);
-              t.sl = kRowB;
-            } else {
-              t.pl = r_int_slot(rint, zp, cl, k, fy * N + fx);
-            }
-            if (fy + 1 >= N) {
-              t.pr = r_bnd_slot(rbnd, 3, bi, fx);
-              t.sr = kRowB;
-            } else {
-              t.pr = r_int_slot(rint, zp, cr, k, (fy + 1) * N + fx);
-            }
-          } else {
-            t.pl = r_int_slot(rint, zp, cl, k - 1, fy * N + fx);
-            t.pr = r_int_slot(rint, zp, cr, k, fy * N + fx);
+        // interior records: code of (1, u1, u2) along (a, b, c), b < c
+        const int par = 9 * (k & 1) * kSlotB, parl = 9 * ((k - 1) & 1) * kSlotB;
+        const int cb = a == 0 ? 3 : 1, cc = a == 2 ? 3 : 9, ca = a == 0 ? 1 : a == 1 ? 3 : 9;
+        const int cell = fy * N + fx;
+        SideRef sl, sr;
+        sl.base = ends + (13 + ca) * kSlotB + 16 * cell + (a == 2 ? parl : 0);
+        sr.base = ends + (13 - ca) * kSlotB + 16 * (cell + (a == 0 ? 1 : a == 1 ? N : 0));
+        sl.s1 = sr.s1 = cb * kSlotB;
+        sl.s2 = sr.s2 = cc * kSlotB;
+        sl.s3 = sr.s3 = a == 2 ? 0 : par;
+        sl.qst = sr.qst = 16 * kNN;
+        sl.dr = 48 * kNN - 12 * cell;
+        sr.dr = 48 * kNN - 12 * (cell + (a == 0 ? 1 : a == 1 ? N : 0));
+        if (a < 2) {
+          const int fa = a == 0 ? fx : fy, pos = a == 0 ? fy : fx;
+          if (fa < 0) {
+            sl.base = bnd + bnd_off(2 * a, 4, pos);
+            sl.s1 = bnd_off(0, 1, 0);
+            sl.s2 = bnd_off(0, 3, 0);
+            sl.s3 = 0;
+            sl.qst = 16 * N;
+            sl.dr = 48 * N - 12 * pos;
           }
-          return t;
-        };
-        // the lane's group (face_group_ends): g = 0 the pairs (0, 1) and (2,
-        // 3), g = 1 the pair (4, 5), g = 2 the pair (6, 7) and the centre 8 in
-        // both lanes (with one flux point per face only the centre)
-        // points n and n + 1 in the two lanes (kTwo), or n alone
-        auto points = [&](auto two, int n) {
-          constexpr bool kTwo = decltype(two)::value;
-          const Pt tA = geom(n), tB = kTwo ? geom(n + 1) : tA;
-          float2 dL[3];
-#pragma unroll
-          for (int m = 0; m < 3; ++m) dL[m] = f2((float)tA.dl[m], (float)tB.dl[m]);
-          const float2 xq = fma2(f2(half_h), dL[0], f2(xc)), yq = fma2(f2(half_h), dL[1], f2(yc));
-          const float wA = face_w(tA.u1, tA.u2, npt), wB = face_w(tB.u1, tB.u2, npt);
-          point_pair32<kTwo>([&](int q) { return tA.pl[q * tA.sl]; }, [&](int q) { return tA.pr[q * tA.sr]; },
-                             [&](int q) { return tB.pl[q * tB.sl]; }, [&](int q) { return tB.pr[q * tB.sr]; }, a,
-                             xq, yq, dL, PF, 0.5f * wA, 0.5f * __fmul_rn(wA, half_h), 0.5f * wB,
-                             0.5f * __fmul_rn(wB, half_h), Gf, Gtl, amax);
-        };
-        // the lane's group (face_group_ends): g = 0 the pairs (0, 1) and (2,
-        // 3), g = 1 the pair (4, 5), g = 2 the pair (6, 7) and the centre 8
-        // (with one flux point per face only the centre)
-        static_assert(face_group_ends(3) && face_group_ends(5) && face_group_ends(8), "lane groups");
-        using Two = std::integral_constant<bool, true>;
-        using One = std::integral_constant<bool, false>;
-        if (npt != 1) points(Two{}, g == 0 ? 0 : 2 * g + 2);  // 0, 4, 6
-        if (npt != 1 && g == 0) points(Two{}, 2);
-        if (g == 2) points(One{}, 8);
-      }
-      // the face's three groups, (G0 + G1) + G2, on the lane of group 0
-      float out[16];
-#pragma unroll
-      for (int q = 0; q < F + 3; ++q) {
-        const float v = q < F ? Gf[q] : Gtl[q - F];
-        const float v1 = __shfl_down_sync(0xffffffffu, v, 1), v2 = __shfl_down_sync(0xffffffffu, v, 2);
-        out[q] = npt == 1 ? v2 : __fadd_rn(__fadd_rn(v, v1), v2);
-      }
-      // the torque about the right cell centre from the face's sums
-      right_torque32(a, h, out, out + F, out + F + 3);
-      if (active && g == 0) {
-        double* dst = zface ? zsum + (size_t)(k % 3) * 16 * N * N + (slot - kNFaceXY) : fsum + slot;
-        const int dstride = zface ? N * N : kNFaceXY;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) dst[q * dstride] = (double)out[q];
-        if (A.face_flux) {
-          // sub-grid boundary faces: sums and the torque about the interior cell
-          int f = -1, pc = 0, pb = 0;
-          bool upper = false;
-          if (a == 0 && (fx < 0 || fx + 1 >= N)) {
-            f = fx < 0 ? 0 : 1;
-            upper = fx >= 0;
-            pc = k;
-            pb = fy;
-          } else if (a == 1 && (fy < 0 || fy + 1 >= N)) {
-            f = fy < 0 ? 2 : 3;
-            upper = fy >= 0;
-            pc = k;
-            pb = fx;
-          } else if (a == 2 && (k == 0 || k == N)) {
-            f = k == 0 ? 4 : 5;
-            upper = k == N;
-            pc = fy;
-            pb = fx;
-          }
-          if (f >= 0) {
-#pragma unroll
-            for (int q = 0; q < F; ++q) io.face(sub, f, q, pc, pb, dst[q * dstride]);
-#pragma unroll
-            for (int m = 0; m < 3; ++m) io.face(sub, f, F + m, pc, pb, dst[(upper ? F + m : F + 3 + m) * dstride]);
+          if (fa + 1 >= N) {
+            sr.base = bnd + bnd_off(2 * a + 1, 4, pos);
+            sr.s1 = bnd_off(0, 1, 0);
+            sr.s2 = bnd_off(0, 3, 0);
+            sr.s3 = 0;
+            sr.qst = 16 * N;
+            sr.dr = 48 * N - 12 * pos;
           }
         }
-      }
-    }
-    // plane k - 2 is complete (its upper z-face was summed in the last
-    // step): two warps that have no face finish it
-    if (k >= 2) finish_plane(k - 2, kFinishT0);
-    if (k + 6 < S) {
-      // the staged padded plane k + 6 into the ring
-      for (int q = tid; q < kPl; q += kThreadsPl) {
-        double u[F];
+        // the coordinate that the frame velocity's normal component takes (y_q
+        // for x-faces, x_q for y-faces; none for z) by the offset along b
+        const float om = a == 0 ? PF.omega : a == 1 ? -PF.omega : 0.f;
+        const float cen = a == 0 ? coord[(N + 2) + fy + 1] : coord[fx + 1];
+        const float rp = __fmaf_rn(half_h, 1.f, cen), rm = __fmaf_rn(half_h, -1.f, cen);
+        constexpr float w1 = 1.f / 36.f, w4 = 4.f / 36.f, w16 = 16.f / 36.f;
+        float2 Gs[5];
+        float TL[3] = {0.f, 0.f, 0.f};
 #pragma unroll
-        for (int f = 0; f < F; ++f) u[f] = stage[f * kPl + q];
-        convert(u, k + 6, q);
+        for (int q = 0; q < 5; ++q) Gs[q] = f2(0.f);
+        int g;
+        // the points of the groups in the face's order (face_u1, face_u2)
+        if (part == 0) {
+          g = 0;
+          plane_point<1, 1>(sl, sr, a, om, rp, half_h, w1, Gs, TL, amax);
+          plane_point<-1, -1>(sl, sr, a, om, rm, half_h, w1, Gs, TL, amax);
+          plane_point<1, 0>(sl, sr, a, om, rp, half_h, w4, Gs, TL, amax);
+          plane_point<-1, 0>(sl, sr, a, om, rm, half_h, w4, Gs, TL, amax);
+        } else if (part == 1) {
+          g = 2;
+          if (npt != 1) {
+            plane_point<0, 1>(sl, sr, a, om, cen, half_h, w4, Gs, TL, amax);
+            plane_point<0, -1>(sl, sr, a, om, cen, half_h, w4, Gs, TL, amax);
+          }
+          plane_point<0, 0>(sl, sr, a, om, cen, half_h, npt == 1 ? 1.f : w16, Gs, TL, amax);
+        } else {
+          g = 1;
+          plane_point<1, -1>(sl, sr, a, om, rp, half_h, w1, Gs, TL, amax);
+          plane_point<-1, 1>(sl, sr, a, om, rm, half_h, w1, Gs, TL, amax);
+        }
+        float* out = sums + g * (F + 3) * kNFace + slot;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          out[(2 * q) * kNFace] = Gs[q].x;
+          out[(2 * q + 1) * kNFace] = Gs[q].y;
+        }
+#pragma unroll
+        for (int m = 0; m < 3; ++m) out[(F + m) * kNFace] = TL[m];
       }
     }
+    if (Io::kPrims || znew + 1 < S) stage_arrive();
     __syncthreads();
-
-    // ---- C: the x- plus y-differences of face sums of plane k -------------
-    if (k >= 0 && k < N) {
-      for (int t = tid; t < DQ * N * N; t += kThreadsPl) {
-        const int q = t / (N * N), cell = t % (N * N), x = cell % N, y = cell / N;
-        // upper face: its fluxes and left-cell torques (q); lower face: its
-        // fluxes and right-cell torques (ql)
-        const int ql = q < F ? q : q + 3;
-        const int xl = y * (N + 1) + x, yl = N * (N + 1) + x * (N + 1) + y;  // lower x- and y-face slots
-        const double d0 = __dsub_rn(fsum[q * kNFaceXY + xl + 1], fsum[ql * kNFaceXY + xl]);
-        const double d1 = __dsub_rn(fsum[q * kNFaceXY + yl + 1], fsum[ql * kNFaceXY + yl]);
-        s01[(size_t)(k & 1) * DQ * N * N + q * N * N + cell] = __dadd_rn(d0, d1);
-      }
-    }
   }
-  // the last plane, after the last z-faces
-  finish_plane(N - 1, 0);
-
+  phase_c(N);
   // ---- amax and the status ------------------------------------------------
 #pragma unroll
   for (int o2 = 16; o2 > 0; o2 >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o2));
   if (lane == 0) red[warp] = amax;
   if (bad) atomicOr(A.status, 1u);
   __syncthreads();
-  if (tid == 0) {
+  // the last two planes
+  finish_plane(N - 2, 0);
+  finish_plane(N - 1, 2 * 32);
+  if (tid == kThreadsPl - 1) {
     float m = red[0];
 #pragma unroll
     for (int w = 1; w < kWarpsPl; ++w) m = fmaxf(m, red[w]);

@@ -61,9 +61,9 @@ struct FusedArgs {
   double cfl, eta2, inv_gamma;
   double alpha[3], beta[3];  // the stage coefficients of the update kernel
   long long wait_ns;    // bound of every wait
-  float* P[2];          // FP32 primitives of the stage inputs, [n][F][NN^3] each (row
-                        // sweep only; NULL otherwise): P[0] holds X's, then U2's;
-                        // P[1] holds U1's
+  float2* P[2];         // FP32 primitives of the stage inputs, pairs of fields
+                        // [n][F/2][NN^3] each: P[0] holds X's, then U2's; P[1]
+                        // holds U1's
 };
 constexpr int kSyncHead = 4;
 
@@ -72,21 +72,22 @@ constexpr int kSyncHead = 4;
 // The FP32 primitives of one cell's state u (prims_mixed) into P at
 // compact cell ci of sub-grid s (NN^3 = n3 cells); a non-physical cell sets
 // the status bit.
-__device__ __forceinline__ void store_prims(const FusedArgs& A, float* P, int s, int ci, const double u[F], int n3) {
+__device__ __forceinline__ void store_prims(const FusedArgs& A, float2* P, int s, int ci, const double u[F], int n3) {
   float q[F];
   if (!prims_mixed(u, A.S.P.eta1, (float)A.S.P.gamma, q)) atomicOr(A.S.status, 1u);
-  float* p = P + (size_t)s * F * n3 + ci;
+  float2* p = P + (size_t)s * (F / 2) * n3 + ci;
 #pragma unroll
-  for (int k = 0; k < F; ++k) p[(size_t)k * n3] = q[k];
+  for (int k = 0; k < F / 2; ++k) p[(size_t)k * n3] = make_float2(q[2 * k], q[2 * k + 1]);
 }
 
-// kPrims: the row sweep reads the FP32 primitives of its window from P
-// (recovered once per cell by the tile that produced the state) instead of
-// recovering them from the FP64 state of every padded cell.
-template <int NN, bool kPrimsIn = false>
+// Both sweeps read the FP32 primitives of their windows from P (recovered
+// once per cell by the tile that produced the state) instead of recovering
+// them from the FP64 state of every padded cell.
+template <int NN>
 struct FusedIo {
   using T = Tile<NN>;
-  static constexpr bool kPrims = kPrimsIn;
+  static constexpr bool kPrims = true, kRows = false;
+  static constexpr int kPairStride = T::kN3;
   const FusedArgs& A;
   int stage;
   double dt;
@@ -126,30 +127,25 @@ struct FusedIo {
       for (int k = 0; k < nf; ++k) u[k] = __ldcg(q + (size_t)(f0 + k) * T::kN3);
     }
   }
-  // Padded cell c of the tile: its source sub-grid and cell under the
-  // uniform mesh's boundary map, fields f0 .. f0 + nf - 1.
-  __device__ __forceinline__ void load_fields(const Sub& q, int c, int f0, int nf, double* u) const {
+  // The primitive pairs of padded cell c of the tile, kPairStride apart: in
+  // the stage input's primitive buffer, at the source cell of the boundary map.
+  __device__ __forceinline__ const float2* prim_pairs(const Sub& q, int c) const {
     const int nx = A.nbx * NN, ny = A.nby * NN, nz = A.nbz * NN;
     const int gx = bc_map(q.kx * NN + q.t.o[0] + c % S - G, nx, A.bc);
     const int gy = bc_map(q.ky * NN + q.t.o[1] + (c / S) % S - G, ny, A.bc);
     const int gz = bc_map(q.kz * NN + q.t.o[2] + c / (S * S) - G, nz, A.bc);
     const int os = ((gz / NN) * A.nby + (gy / NN)) * A.nbx + (gx / NN);
     const int ix = gx & (NN - 1), iy = gy & (NN - 1), iz = gz & (NN - 1);
-    state(os, (iz * NN + iy) * NN + ix, ((iz + G) * T::kS + (iy + G)) * T::kS + (ix + G), u, f0, nf);
+    return A.P[stage == 1 ? 1 : 0] + (size_t)os * (F / 2) * T::kN3 + (iz * NN + iy) * NN + ix;
   }
-  __device__ __forceinline__ void load(const Sub& q, int c, double u[F]) const { load_fields(q, c, 0, F, u); }
-  // The primitives of padded cell c of the tile (kPrims): from the stage
-  // input's primitive buffer, at the source cell of the boundary map.
   __device__ __forceinline__ void load_prims(const Sub& q, int c, float* u) const {
-    const int nx = A.nbx * NN, ny = A.nby * NN, nz = A.nbz * NN;
-    const int gx = bc_map(q.kx * NN + q.t.o[0] + c % S - G, nx, A.bc);
-    const int gy = bc_map(q.ky * NN + q.t.o[1] + (c / S) % S - G, ny, A.bc);
-    const int gz = bc_map(q.kz * NN + q.t.o[2] + c / (S * S) - G, nz, A.bc);
-    const int os = ((gz / NN) * A.nby + (gy / NN)) * A.nbx + (gx / NN);
-    const int ix = gx & (NN - 1), iy = gy & (NN - 1), iz = gz & (NN - 1);
-    const float* p = A.P[stage == 1 ? 1 : 0] + (size_t)os * F * T::kN3 + (iz * NN + iy) * NN + ix;
+    const float2* p = prim_pairs(q, c);
 #pragma unroll
-    for (int k = 0; k < F; ++k) u[k] = __ldcg(p + (size_t)k * T::kN3);
+    for (int k = 0; k < F / 2; ++k) {
+      const float2 v = __ldcg(p + (size_t)k * T::kN3);
+      u[2 * k] = v.x;
+      u[2 * k + 1] = v.y;
+    }
   }
   __device__ __forceinline__ void own(const Sub& q, int c, int uc, double u[F]) const {
     state(q.t.s, q.t.cell(c), q.t.pad(uc), u);
@@ -171,7 +167,7 @@ struct FusedIo {
       double* o = A.U2 + (size_t)s * F * T::kN3 + ci;
 #pragma unroll
       for (int k = 0; k < F; ++k) o[(size_t)k * T::kN3] = un[k];
-      if (kPrims) store_prims(A, A.P[0], s, ci, un, T::kN3);  // U2's, for stage 2
+      store_prims(A, A.P[0], s, ci, un, T::kN3);  // U2's, for stage 2
     } else {
       double* o = A.Y + (size_t)s * F * T::kS3 + pi;
 #pragma unroll
@@ -225,7 +221,6 @@ static __device__ bool wait_neighbours(const FusedArgs& A, const unsigned* flags
 template <bool kGate, bool kContact, bool kSpin = false>
 struct RowBody {
   static constexpr int kThreads = kThreadsMx, kMinBlocks = 2;
-  static constexpr bool kPrims = true;  // reads its windows' primitives from FusedArgs::P
   static constexpr size_t kRed = (kMixedSmemBytes + 15) / 16 * 16;
   static constexpr size_t kSmem = kRed + sizeof(float) * (kThreadsMx / 32);
   RowMap R;
@@ -243,13 +238,14 @@ struct RowBody {
 template <bool kContact, bool kSpin = false>
 struct PlaneBody {
   static constexpr int kThreads = kThreadsPl, kMinBlocks = 1;
-  static constexpr bool kPrims = false;
   static constexpr size_t kSmem = kPlaneSmemBytes;
   unsigned char* sm;
-  __device__ PlaneBody(const StepArgs64&, unsigned char* p) : sm(p) {}
+  double* D;
+  __device__ PlaneBody(const StepArgs64& S, unsigned char* p)
+      : sm(p), D(S.scratch + (size_t)blockIdx.x * kScratchPerSub) {}
   template <class Io>
   __device__ __forceinline__ void run(const StepArgs64& S, const Io& io, int s) const {
-    mixed_subgrid_planes<kContact, kSpin>(S, io, s, sm);
+    mixed_subgrid_planes<kContact, kSpin>(S, io, s, sm, D);
   }
 };
 
@@ -269,7 +265,7 @@ __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fu
   unsigned* published = A.sync + kSyncHead;    // U2 tiles done, per sub-grid
   unsigned* published1 = published + n;        // U1 tiles done, per sub-grid
 
-  using Io = FusedIo<NN, Body::kPrims>;
+  using Io = FusedIo<NN>;
   // grid-wide barrier number k (1, 2, ...): every CTA arrives once per barrier
   auto grid_sync = [&](unsigned k) {
     if (tid == 0) {
@@ -287,8 +283,8 @@ __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fu
   };
   unsigned barriers = 0;
 
-  // ---- the primitives of X's interiors (row sweep), once per cell --------
-  if (Body::kPrims) {
+  // ---- the primitives of X's interiors, once per cell ---------------------
+  {
     for (int u = blockIdx.x; u < units; u += gridDim.x) {
       const T t(u);
       const double* __restrict__ x = A.S.U + (size_t)t.s * F * T::kS3;
@@ -341,7 +337,7 @@ __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fu
       rk3_cell<true>(xv, xv, rv, dt, A.alpha[0], A.beta[0], A.eta2, A.inv_gamma, u1);
 #pragma unroll
       for (int k = 0; k < F; ++k) y[(size_t)k * T::kS3 + uc] = u1[k];
-      if (Body::kPrims) store_prims(A, A.P[1], t.s, ci, u1, T::kN3);
+      store_prims(A, A.P[1], t.s, ci, u1, T::kN3);
     }
     __syncthreads();
     if (tid == 0) {
@@ -455,8 +451,8 @@ static cudaError_t launch_fused_nn(const StepArgs64& S, double* Y, double* U2, f
   A.S = S;
   A.Y = Y;
   A.U2 = U2;
-  A.P[0] = prims;
-  A.P[1] = prims + (size_t)S.n_sub * F * Tile<NN>::kN3;
+  A.P[0] = reinterpret_cast<float2*>(prims);
+  A.P[1] = A.P[0] + (size_t)S.n_sub * (F / 2) * Tile<NN>::kN3;
   A.dt_out = dt_out;
   A.sync = sync;
   A.nbx = nbx;

@@ -16,9 +16,13 @@ namespace hyd {
 template <int NN>
 struct StepIo {
   using T = Tile<NN>;
-  static constexpr bool kPrims = false;
+  static constexpr bool kPrims = false, kRows = true;
   const StepArgs64& A;
   using Sub = T;
+  // row y of plane z of the tile's padded window, field k
+  __device__ __forceinline__ const double* row(const Sub& q, int k, int z, int y) const {
+    return A.U + ((size_t)q.s * F + k) * T::kS3 + q.pad(0, y, z);
+  }
   __device__ __forceinline__ Sub begin(int u) const { return T(u); }
   __device__ __forceinline__ int sidx(const Sub& q) const { return q.s; }
   __device__ __forceinline__ int offx(const Sub& q) const { return q.o[0]; }
@@ -76,9 +80,10 @@ __global__ void __launch_bounds__(kThreadsMx, 2) hydro_step_mixed_kernel(StepArg
 template <bool kContact, int NN = N, bool kSpin = false>
 __global__ void __launch_bounds__(kThreadsPl, 1) hydro_step_mixed_planes_kernel(StepArgs64 A) {
   extern __shared__ __align__(128) unsigned char sm[];
+  double* __restrict__ D = A.scratch + (size_t)blockIdx.x * kScratchPerSub;
   const StepIo<NN> io{A};
   const int units = A.n_sub * Tile<NN>::kTiles;
-  for (int u = blockIdx.x; u < units; u += gridDim.x) mixed_subgrid_planes<kContact, kSpin>(A, io, u, sm);
+  for (int u = blockIdx.x; u < units; u += gridDim.x) mixed_subgrid_planes<kContact, kSpin>(A, io, u, sm, D);
 }
 
 

@@ -1,4 +1,4 @@
-// hydro_step_mixed_amr.cu -- the mixed-precision row sweep over the leaves of
+// hydro_step_mixed_amr.cu -- the mixed-precision sweeps over the leaves of
 // an adaptive mesh (8^3 leaves) with a tile loader that reads each ghost cell
 // where it lives, so that the ghost fill need not copy or restrict
 // (hydro_fill_ghosts_amr_lean):
@@ -19,7 +19,7 @@ namespace hyd {
 
 struct AmrStepIo {
   using T = Tile<N>;
-  static constexpr bool kPrims = false;
+  static constexpr bool kPrims = false, kRows = false;
   const StepArgs64& A;
   const AMRArgs& M;
   struct Sub {
@@ -92,21 +92,35 @@ __global__ void __launch_bounds__(kThreadsMx, 2) hydro_step_mixed_amr_kernel(Ste
   }
 }
 
+// The plane sweep (no indicator): one CTA per SM.
+__global__ void __launch_bounds__(kThreadsPl, 1) hydro_step_mixed_amr_planes_kernel(StepArgs64 A, AMRArgs M) {
+  extern __shared__ __align__(128) unsigned char sm[];
+  double* __restrict__ D = A.scratch + (size_t)blockIdx.x * kScratchPerSub;
+  const AmrStepIo io{A, M};
+  for (int u = blockIdx.x; u < A.n_sub; u += gridDim.x) {
+    const int s = leaf_at(M, u);  // the same for the whole CTA
+    if (s >= 0) mixed_subgrid_planes<false, false>(A, io, s, sm, D);
+  }
+}
+
 cudaError_t prepare_step_mixed_amr() {
   static unsigned long long done = 0;
   return once_per_device(&done, [] {
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(hydro_step_mixed_amr_kernel<false>, at, (int)kMixedSmemBytes);
-    return e == cudaSuccess ? cudaFuncSetAttribute(hydro_step_mixed_amr_kernel<true>, at, (int)kMixedSmemBytes) : e;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(hydro_step_mixed_amr_kernel<true>, at, (int)kMixedSmemBytes);
+    return e == cudaSuccess ? cudaFuncSetAttribute(hydro_step_mixed_amr_planes_kernel, at, (int)kPlaneSmemBytes) : e;
   });
 }
 
-// grid: persistent CTAs (two per SM by default, as the row sweep of
-// hydro_step); the leaves' dU/dt, amax and boundary faces (A.face_flux).
-cudaError_t launch_step_mixed_amr(const StepArgs64& A, const AMRArgs& M, int grid, cudaStream_t st) {
+// grid: persistent CTAs (as for hydro_step in the decomposition); the leaves'
+// dU/dt, amax and boundary faces (A.face_flux).
+cudaError_t launch_step_mixed_amr(const StepArgs64& A, const AMRArgs& M, int grid, int planes, cudaStream_t st) {
   cudaError_t e = prepare_step_mixed_amr();
   if (e != cudaSuccess) return e;
-  if (A.gate)
+  if (planes && !A.gate)
+    hydro_step_mixed_amr_planes_kernel<<<grid, kThreadsPl, kPlaneSmemBytes, st>>>(A, M);
+  else if (A.gate)
     hydro_step_mixed_amr_kernel<true><<<grid, kThreadsMx, kMixedSmemBytes, st>>>(A, M);
   else
     hydro_step_mixed_amr_kernel<false><<<grid, kThreadsMx, kMixedSmemBytes, st>>>(A, M);
