@@ -82,12 +82,16 @@ __device__ __forceinline__ double slope64(double a, double b) {
   return sign64(min64(twice_mag(lo), half_mag(mag64(radd(a, b)))), b);
 }
 
-// The unlimited PPM interface value between samples sa and sb (in the line's
-// order) from their limited slopes Da, Db: (sa + sb)/2 - (Db - Da)/6.  The
-// +d value of a cell and the -d value of its +d neighbour are the same
-// number, so a sweep along the line may compute it once for both.
-__device__ __forceinline__ double ppm_iface64(double sa, double sb, double Da, double Db) {
-  return fma(-1.0 / 6.0, rsub(Db, Da), half64(radd(sa, sb)));
+// PPM's interface value between two neighbouring samples of a line, taken from
+// both sides: with dl = s_b - s_a and the limited slopes Da, Db,
+//   u = value - s_a = dl/2 - (Db - Da)/6,  w = s_b - value = dl/2 + (Db - Da)/6.
+// The +d side of a cell and the -d side of its +d neighbour share the slopes'
+// difference and dl, so a sweep along the line forms both in three FP64
+// instructions (exactly mirrored on the reversed line).
+__device__ __forceinline__ void ppm_sides64(double dl, double Da, double Db, double& u, double& w) {
+  const double t = rsub(Db, Da), hd = half64(dl);
+  u = fma(-1.0 / 6.0, t, hd);
+  w = fma(1.0 / 6.0, t, hd);
 }
 
 // Contact steepening of the interface values p (+d) and m (-d) of the
@@ -100,33 +104,30 @@ __device__ __forceinline__ void ppm_steep64(double s1, double s3, double D0, dou
   m = radd(rmul(keep, m), rmul(eta, radd(s1, half64(D0))));
 }
 
-// The monotonicity fix-ups of PPM on the interface values p (+d) and m (-d)
-// of the cell value s2: a local extremum flattens the cell, an interface
-// value that would put the parabola's extremum inside the cell is moved to
-// 3 s2 - 2 (the other one).  With u = p - s2 and w = s2 - m, an extremum is
-// u w <= 0, and of one sign the parabola test (p - m)(s2 - (p + m)/2) against
-// +-(p - m)^2/6 reads |w| > 2|u| (m moves to s2 - 2u) and |u| > 2|w| (p moves
-// to s2 + 2w): sign bits and comparisons of bit patterns, so two FP64
-// instructions and one in a cell that moves, instead of nine and three.  The
-// limited values are continuous where the tests switch.
-__device__ __forceinline__ void ppm_limit64(double s2, double& p, double& m) {
-  const double u = rsub(p, s2), w = rsub(s2, m);
+// The same on u = p - s2 and w = s2 - m.
+__device__ __forceinline__ void ppm_steep_sides64(double s1, double s2, double s3, double D0, double D2, double eta,
+                                                  double& u, double& w) {
+  double p = radd(s2, u), m = rsub(s2, w);
+  ppm_steep64(s1, s3, D0, D2, eta, p, m);
+  u = rsub(p, s2);
+  w = rsub(s2, m);
+}
+
+// The monotonicity fix-ups of PPM on the interface values s2 + u (+d) and
+// s2 - w (-d) of the cell value s2, giving p and m: a local extremum flattens
+// the cell, an interface value that would put the parabola's extremum inside
+// the cell is moved to 3 s2 - 2 (the other one).  An extremum is u w <= 0, and
+// with one sign the parabola test (p - m)(s2 - (p + m)/2) against +-(p - m)^2/6
+// reads |w| > 2|u| (m moves to s2 - 2u) and |u| > 2|w| (p moves to s2 + 2w):
+// magnitudes cut to twice the other's, on the bit patterns, and two FP64
+// additions where the tests and moves took twelve.  The limited values are
+// continuous where the tests switch.
+__device__ __forceinline__ void ppm_limit64(double s2, double u, double w, double& p, double& m) {
   const long long au = mag64(u), aw = mag64(w);
-  if (signs_differ(u, w) || min64(au, aw) == 0LL) {
-    p = s2;
-    m = s2;
-    return;
-  }
-  const long long au2 = twice_mag(au), aw2 = twice_mag(aw);
-  const bool mm = aw > au2, mp = au > aw2;
-  if (mm || mp) {
-    // s2 - 2u or s2 + 2w (w has u's sign)
-    const double r = radd(s2, sign64(mm ? au2 : aw2, u, mm));
-    if (mm)
-      m = r;
-    else
-      p = r;
-  }
+  const bool flat = signs_differ(u, w);
+  const long long lu = flat ? 0LL : min64(au, twice_mag(aw)), lw = flat ? 0LL : min64(aw, twice_mag(au));
+  p = radd(s2, sign64(lu, u));
+  m = rsub(s2, sign64(lw, w));
 }
 
 // PPM on the five samples s0..s4 of one line: qp = value at the +d end of the
@@ -139,12 +140,11 @@ __device__ __forceinline__ void ppm64(double s0, double s1, double s2, double s3
                                       double& qm, double eta = 0.0) {
   const double d0 = rsub(s1, s0), d1 = rsub(s2, s1), d2 = rsub(s3, s2), d3 = rsub(s4, s3);
   const double D0 = slope64(d0, d1), D1 = slope64(d1, d2), D2 = slope64(d2, d3);
-  double p = ppm_iface64(s2, s3, D1, D2);
-  double m = ppm_iface64(s1, s2, D0, D1);
-  if (kSteep && eta > 0.0) ppm_steep64(s1, s3, D0, D2, eta, p, m);
-  ppm_limit64(s2, p, m);
-  qp = p;
-  qm = m;
+  double u, w, x;
+  ppm_sides64(d2, D1, D2, u, x);
+  ppm_sides64(d1, D0, D1, x, w);
+  if (kSteep && eta > 0.0) ppm_steep_sides64(s1, s2, s3, D0, D2, eta, u, w);
+  ppm_limit64(s2, u, w, qp, qm);
 }
 
 // All ten primitives along the line through smem cell index c with stride st.
@@ -223,6 +223,41 @@ __device__ __forceinline__ void line10u(const double* __restrict__ Q, int c, int
   }
 }
 
+// 1 / sqrt(x) for x > 0 to about an ulp: the FP32 value y refined by one step of
+// Halley's third-order iteration, y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the
+// FP32 value's error of 2^-22 leaves 2^-63), five FP64 instructions.  Outside
+// FP32's normal range the library's function, in a call.
+static __device__ __noinline__ double rsqrt_call(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rsqrt64(double x) {
+  if ((unsigned)__double2hiint(x) - 0x38100000u >= 0x0fd00000u) return rsqrt_call(x);
+  const double y = widen(rsqrtf(narrow(x)));
+  const double e = fma(-rmul(x, y), y, 1.0);
+  return fma(rmul(e, y), fma(0.375, e, 0.5), y);
+}
+
+// The primitives of one cell from its conserved rho, s, E in u (v and eps in
+// place) and the tracer; false for a non-physical cell.  The three quotients
+// by rho from one reciprocal, each with Markstein's correction (the remainder
+// s - q rho, exact in a fused step, times 1/rho), which rounds them correctly.
+__device__ __forceinline__ bool prims64(double u[EGAS + 1], double tau, const StepParams& P) {
+  const double rho = u[RHO];
+  const double ri = __drcp_rn(rho);
+  double v[3];
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    const double q = rmul(u[SX + m], ri);
+    v[m] = fma(fma(-q, rho, u[SX + m]), ri, q);
+  }
+  const double E = u[EGAS];
+  const double ek = rmul(half64(rho), radd(radd(rmul(v[0], v[0]), rmul(v[1], v[1])), rmul(v[2], v[2])));
+  const double eE = rsub(E, ek);
+  const double eps = (eE > rmul(P.eta1, E)) ? eE : pow(tau, P.gamma);
+#pragma unroll
+  for (int m = 0; m < 3; ++m) u[SX + m] = v[m];
+  u[EGAS] = eps;
+  return (rho > 0.0) && (eps > 0.0);
+}
+
 // What the flux needs of a reconstructed state besides its fields: the
 // pressure p, the energy E = eps + rho |v|^2 / 2 and the sound speed.
 // c = sqrt(gamma p / rho) = gamma p / sqrt(gamma p rho): one reciprocal square
@@ -238,7 +273,7 @@ __device__ __forceinline__ End64 end64(double rho, double vx, double vy, double 
   e.p = rmul(P.gm1, eps);
   e.E = fma(half64(rho), fma(vz, vz, fma(vy, vy, rmul(vx, vx))), eps);
   const double gp = rmul(P.gamma, e.p);
-  e.c = (__double_as_longlong(gp) <= 0LL) ? 0.0 : rmul(gp, rsqrt(rmul(gp, rho)));
+  e.c = (__double_as_longlong(gp) <= 0LL) ? 0.0 : rmul(gp, rsqrt64(rmul(gp, rho)));
   return e;
 }
 

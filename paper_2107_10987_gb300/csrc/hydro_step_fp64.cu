@@ -109,17 +109,12 @@ __global__ void __launch_bounds__(kThreads64, 1) hydro_step_fp64_kernel(StepArgs
     // ---- 2. primitives in place ----------------------------------------
     bool bad = false;
     for (int c = tid; c < S3; c += kThreads64) {
-      const double rho = Q[RHO * S3 + c];
-      const double vx = Q[SX * S3 + c] / rho, vy = Q[SY * S3 + c] / rho, vz = Q[SZ * S3 + c] / rho;
-      const double E = Q[EGAS * S3 + c];
-      const double ek = rmul(rmul(0.5, rho), radd(radd(rmul(vx, vx), rmul(vy, vy)), rmul(vz, vz)));
-      const double eE = rsub(E, ek);
-      const double eps = (eE > rmul(A.P.eta1, E)) ? eE : pow(Q[TAU * S3 + c], A.P.gamma);
-      Q[SX * S3 + c] = vx;
-      Q[SY * S3 + c] = vy;
-      Q[SZ * S3 + c] = vz;
-      Q[EGAS * S3 + c] = eps;
-      bad |= !(rho > 0.0) || !(eps > 0.0);
+      double w[EGAS + 1];
+#pragma unroll
+      for (int k = 0; k <= EGAS; ++k) w[k] = Q[k * S3 + c];
+      bad |= !prims64(w, Q[TAU * S3 + c], A.P);
+#pragma unroll
+      for (int k = SX; k <= EGAS; ++k) Q[k * S3 + c] = w[k];
     }
     if (bad) atomicOr(A.status, 1u);
     __syncthreads();

@@ -44,12 +44,13 @@
 // What bounds it: the FP64 pipe, which issues a warp's instruction every 16
 // cycles per SM.  12 warps keep it busy without prefetching (6 warps held it
 // at 83 %), and the work is cut to the pipe's: decisions on bit patterns,
-// masks instead of |x| and -x, line ends' sound speeds shared and the flux in
-// two fused steps per field.  A tile of random data takes a CTA 0.726 ms
-// (about 1.09 before); the RK3 step of a 512-sub-grid blast 12.96 -> 7.73 ms.
+// masks instead of |x| and -x, an interface value from both its sides at once,
+// line ends' sound speeds shared, unread ends of ghost cells left out, and the
+// flux in two fused steps per field.  A tile of random data takes a CTA 0.664
+// ms (about 1.09 before); the RK3 step of a 512-sub-grid blast 13.0 -> 7.0 ms.
 // Teams serve the batches that do not fill whole rounds of the SMs
-// (step_fp64_choose_team): 512 tiles take pairs of CTAs 2.69 ms and single
-// ones 2.90, one tile takes the whole chip 0.09 ms and one CTA 0.73.
+// (step_fp64_choose_team): 512 tiles take pairs of CTAs 2.45 ms and single
+// ones 2.65, one tile takes the whole chip 0.08 ms and one CTA 0.66.
 #include <algorithm>
 #include <vector>
 
@@ -164,10 +165,10 @@ __device__ __forceinline__ void ld_sector(const double* p, double& a, double& b,
 
 // One work item of phase 3: fields k0 .. k0 + NG - 1 along run word e.  The
 // window holds, per field, the samples S(i-2..i+2) of cell i of the run, the
-// differences and MC slopes around it and the interface value Q(i - 1/2);
-// each step loads one sample per field and forms one difference, one slope
-// and one interface value (ppm64's operations on the same operands), then
-// the cell's fix-ups, and stores the group's sectors of both records of the
+// differences and MC slopes around it and w = S(i) - Q(i - 1/2) of the
+// interface value Q; each step loads one sample per field and forms one
+// difference, one slope and one interface value from both its sides (ppm64's
+// operations on the same operands), then the cell's fix-ups, and stores the group's sectors of both records of the
 // cell: fields 0 .. 5 with end64's values the first two, fields 6 .. 9 the
 // last.
 template <bool kGate, bool kContact, int NG>
@@ -181,10 +182,18 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
   static_assert(NG == 6 || NG == 4, "field groups 0 .. 5 and 6 .. 9");
   double* Rp = R + ((size_t)(2 * dir_index(dx, dy, dz)) * kBox + b0) * kRec + (NG == 6 ? 0 : 8);
   double* Rm = Rp + (size_t)kBox * kRec;
+  // A ghost cell (the first or the last of a run) has only the end at its face
+  // read: towards +d where d points into the tile from it, else towards -d.
+  auto outward = [&](int i) {  // bit 0: the +d end is not read, bit 1: the -d end
+    const int x = b0 % (N + 2) + i * dx, y = (b0 / (N + 2)) % (N + 2) + i * dy, z = b0 / ((N + 2) * (N + 2)) + i * dz;
+    const int in = x == 0 ? dx : x == N + 1 ? -dx : y == 0 ? dy : y == N + 1 ? -dy : z == 0 ? dz : z == N + 1 ? -dz : 0;
+    return in == 0 ? 0 : in > 0 ? 2 : 1;
+  };
+  const int out0 = outward(0), outn = outward(n - 1);
   const double* q = Q + k0 * S3 + c0;
   // the group's steepened field: rho in the first, the species in the second
   const bool steep_group = kContact;
-  double sm2[NG], sm1[NG], s0[NG], s1[NG], dr[NG], Dm[NG], Dc[NG], qm[NG];
+  double sm2[NG], sm1[NG], s0[NG], s1[NG], dr[NG], Dm[NG], Dc[NG], wl[NG];
 #pragma unroll
   for (int f = 0; f < NG; ++f) {
     const double* qf = q + f * S3;
@@ -196,7 +205,8 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
     Dm[f] = slope64(rsub(sm1[f], sm2[f]), dl);  // slope at cell i - 1
     dr[f] = rsub(s1[f], s0[f]);
     Dc[f] = slope64(dl, dr[f]);  // slope at cell i
-    qm[f] = ppm_iface64(sm1[f], s0[f], Dm[f], Dc[f]);  // interface value at i - 1/2
+    double u;
+    ppm_sides64(dl, Dm[f], Dc[f], u, wl[f]);  // interface value at i - 1/2
   }
 #pragma unroll 1
   for (int i = 0; i < n; ++i) {
@@ -210,9 +220,8 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
       const double s2 = q[f * S3 + (i + 2) * sv];
       const double d2 = rsub(s2, s1[f]);
       const double Dp = slope64(dr[f], d2);  // slope at cell i + 1
-      const double qp = ppm_iface64(s0[f], s1[f], Dc[f], Dp);
-      p[f] = qp;
-      m[f] = qm[f];
+      double up, wn;
+      ppm_sides64(dr[f], Dc[f], Dp, up, wn);
       if (kGate && smooth_i && !(k == ZX || k == ZY || k == ZZ)) {
         // the indicator's unlimited 4-point values (line10u)
         const double c7 = 7.0 / 12.0, c1 = 1.0 / 12.0;
@@ -221,9 +230,9 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
       } else {
         if (kContact && contact && (k == RHO || k == SP0)) {
           const double eta = contact_eta64(sm2[f], sm1[f], s0[f], s1[f], s2);
-          if (eta > 0.0) ppm_steep64(sm1[f], s1[f], Dm[f], Dp, eta, p[f], m[f]);
+          if (eta > 0.0) ppm_steep_sides64(sm1[f], s0[f], s1[f], Dm[f], Dp, eta, up, wl[f]);
         }
-        ppm_limit64(s0[f], p[f], m[f]);
+        ppm_limit64(s0[f], up, wl[f], p[f], m[f]);
       }
       sm2[f] = sm1[f];
       sm1[f] = s0[f];
@@ -232,7 +241,7 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
       dr[f] = d2;
       Dm[f] = Dc[f];
       Dc[f] = Dp;
-      qm[f] = qp;
+      wl[f] = wn;
     }
     if (NG == 6 && P.spin) {
       // the cell's spin fed back into the velocity at both ends (spin_dv64)
@@ -245,36 +254,17 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
         m[(1 + m3) % NG] = rsub(m[(1 + m3) % NG], dv[m3]);
       }
     }
-    double* wp = Rp + i * bv;
-    double* wm = Rm + i * bv;
-    if (NG == 6) {
-      const End64 ep = end64(p[0], p[1], p[2], p[3], p[NG > 4 ? 4 : 0], P);
-      const End64 em = end64(m[0], m[1], m[2], m[3], m[NG > 4 ? 4 : 0], P);
-      st_sector(wp, p[0], p[1], p[2], p[3]);
-      st_sector(wm, m[0], m[1], m[2], m[3]);
-      st_sector(wp + 4, ep.p, ep.E, ep.c, p[NG > 5 ? 5 : 0]);
-      st_sector(wm + 4, em.p, em.E, em.c, m[NG > 5 ? 5 : 0]);
-    } else {
-      st_sector(wp, p[0], p[1], p[2], p[3]);
-      st_sector(wm, m[0], m[1], m[2], m[3]);
-    }
+    const int out = (i == 0 ? out0 : 0) | (i == n - 1 ? outn : 0);
+    auto put = [&](double* d, const double(&q)[NG]) {
+      st_sector(d, q[0], q[1], q[2], q[3]);
+      if (NG == 6) {
+        const End64 e = end64(q[0], q[1], q[2], q[3], q[NG > 4 ? 4 : 0], P);
+        st_sector(d + 4, e.p, e.E, e.c, q[NG > 5 ? 5 : 0]);
+      }
+    };
+    if (!(out & 1)) put(Rp + i * bv, p);
+    if (!(out & 2)) put(Rm + i * bv, m);
   }
-}
-
-// The primitives of one padded cell in place of its conserved state
-// (hydro_step_fp64_kernel's arithmetic); false for a non-physical cell.
-__device__ __forceinline__ bool prims64(double u[EGAS + 1], double tau, const StepParams& P) {
-  const double rho = u[RHO];
-  const double vx = u[SX] / rho, vy = u[SY] / rho, vz = u[SZ] / rho;
-  const double E = u[EGAS];
-  const double ek = rmul(rmul(0.5, rho), radd(radd(rmul(vx, vx), rmul(vy, vy)), rmul(vz, vz)));
-  const double eE = rsub(E, ek);
-  const double eps = (eE > rmul(P.eta1, E)) ? eE : pow(tau, P.gamma);
-  u[SX] = vx;
-  u[SY] = vy;
-  u[SZ] = vz;
-  u[EGAS] = eps;
-  return (rho > 0.0) && (eps > 0.0);
 }
 
 // Barrier of a team (T = 1: of the CTA): every thread's earlier writes are
