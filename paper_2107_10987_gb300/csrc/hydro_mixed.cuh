@@ -370,25 +370,39 @@ __device__ __forceinline__ float face_w(int u1, int u2, int face_points) {
   return face_points == 1 ? 1.f : (u1 == 0 && u2 == 0) ? (16.f / 36.f) : (u1 == 0 || u2 == 0) ? (4.f / 36.f) : (1.f / 36.f);
 }
 
-// Unlimited interface value towards +d (the 4-point formula the PPM
-// interface value reduces to when no limiter acts): used on cells the
-// learned indicator marks smooth.
-__device__ __forceinline__ void unlimited32(float s0, float s1, float s2, float s3, float s4, float& qp, float& qm) {
-  const float a = 7.f / 12.f, b = 1.f / 12.f;
-  qp = __fmaf_rn(a, __fadd_rn(s2, s3), -__fmul_rn(b, __fadd_rn(s1, s4)));
-  qm = __fmaf_rn(a, __fadd_rn(s1, s2), -__fmul_rn(b, __fadd_rn(s0, s3)));
+// Unlimited interface values (the 4-point formula the PPM interface value
+// reduces to when no limiter acts) on two lanes: used on cells the learned
+// indicator marks smooth.
+__device__ __forceinline__ void unlimited32x2(const float2 s[5], float2& qp, float2& qm) {
+  const float2 a = f2(7.f / 12.f), b = f2(-(1.f / 12.f));
+  qp = fma2(a, add2(s[2], s[3]), mul2(b, add2(s[1], s[4])));
+  qm = fma2(a, add2(s[1], s[2]), mul2(b, add2(s[0], s[3])));
 }
 
 // Lines of a cell the indicator marks smooth: the unlimited formula for all
-// fields but the spin, which stays limited.
+// fields but the spin, which stays limited.  Two fields per packed
+// instruction, as line10f: about 200 instructions against its 330 (287 a field
+// at a time).
 __device__ __forceinline__ void line10u(const float* __restrict__ Q, int c, int st, float qp[F], float qm[F]) {
+  static_assert(ZX == 6 && ZZ == 8 && SP0 == 9, "pairs of fields");
 #pragma unroll
-  for (int k = 0; k < F; ++k) {
-    const float* q = Q + k * S3 + c;
-    if (k == ZX || k == ZY || k == ZZ)
-      ppm32(q[-2 * st], q[-st], q[0], q[st], q[2 * st], qp[k], qm[k]);
+  for (int k = 0; k < F; k += 2) {
+    const Samples2 v = samples2(Q, c, st, k, k + 1);
+    float2 p, m;
+    if (k < ZX)
+      unlimited32x2(v.s, p, m);
     else
-      unlimited32(q[-2 * st], q[-st], q[0], q[st], q[2 * st], qp[k], qm[k]);
+      ppm32x2(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m);
+    if (k == ZZ) {  // the species, in the spin's other lane
+      float2 pu, mu;
+      unlimited32x2(v.s, pu, mu);
+      p.y = pu.y;
+      m.y = mu.y;
+    }
+    qp[k] = p.x;
+    qp[k + 1] = p.y;
+    qm[k] = m.x;
+    qm[k + 1] = m.y;
   }
 }
 
