@@ -96,18 +96,15 @@ static int ensure_buf(hydro_ctx* c, double** buf, size_t* have, size_t need, con
 
 // The sub-grid decomposition a step of this context over `units` tiles runs
 // (mixed precision; FP64 and the learned indicator have the row sweep): what
-// hydro_set_launch or the autotuner chose, else the one whose rounds over the
-// SMs take less.  The plane sweep has one tile per SM at a time, 95 us each;
-// the row sweep two, 166 us for both, or 155 us where the last round leaves a
-// tile alone on its SM.  So planes up to one tile per SM and, on 152 SMs, from
-// 305 to 456 and from 609 to 760 tiles.
+// hydro_set_launch or the autotuner chose, else the plane sweep for a batch
+// of at most one tile per SM, the row sweep for more.  A tile alone on an SM
+// takes the plane sweep 95 us and the row sweep 155; two row-sweep tiles share
+// an SM in 166 (304 tiles 0.176 ms; 400 tiles 0.278 against 0.272 for planes,
+// 700 tiles 0.42 against 0.45).
 static int eff_decomp(const hydro_ctx* c, int units) {
   if (c->mode.precision != HYDRO_PREC_MIXED || c->gate_on) return HYDRO_DECOMP_ROWS;
   if (c->decomp != HYDRO_DECOMP_AUTO) return c->decomp;
-  const long sms = c->num_sms, full = units / (2 * sms), rest = units % (2 * sms);
-  const long planes_us = 95 * ((units + sms - 1) / sms);
-  const long rows_us = 166 * full + (rest == 0 ? 0 : rest <= sms ? 155 : 172);
-  return planes_us < rows_us ? HYDRO_DECOMP_PLANES : HYDRO_DECOMP_ROWS;
+  return units <= c->num_sms ? HYDRO_DECOMP_PLANES : HYDRO_DECOMP_ROWS;
 }
 
 static int step_slots(const hydro_ctx* c, int units) {
