@@ -139,24 +139,24 @@ __device__ __forceinline__ void ppm32x2(float2 s0, float2 s1, float2 s2, float2 
   ppm_fix(e.y, lhs.y, rhs.y, s2.y, s2x3.y, qp.y, qm.y);
 }
 
-// The five samples of fields fa and fb along a line (stride st through cell
-// c of the padded FP32 array Q), as pairs.
+// The row sweep's FP32 primitives of a padded tile are pairs of fields,
+// [F/2][S3] float2: pair f holds fields 2f and 2f + 1, one 8-byte load for both
+// lanes of the packed arithmetic.
 struct Samples2 {
   float2 s[5];
 };
-__device__ __forceinline__ Samples2 samples2(const float* __restrict__ Q, int c, int st, int fa, int fb) {
-  const float* qa = Q + fa * S3 + c;
-  const float* qb = Q + fb * S3 + c;
+// The five samples of pair f along a line (stride st through cell c).
+__device__ __forceinline__ Samples2 samples2(const float2* __restrict__ Q, int c, int st, int f) {
   Samples2 r;
 #pragma unroll
-  for (int m = 0; m < 5; ++m) r.s[m] = f2(qa[(m - 2) * st], qb[(m - 2) * st]);
+  for (int m = 0; m < 5; ++m) r.s[m] = Q[f * S3 + c + (m - 2) * st];
   return r;
 }
 
-__device__ __forceinline__ void line10f(const float* __restrict__ Q, int c, int st, float qp[F], float qm[F]) {
+__device__ __forceinline__ void line10f(const float2* __restrict__ Q, int c, int st, float qp[F], float qm[F]) {
 #pragma unroll
   for (int k = 0; k < F; k += 2) {
-    const Samples2 v = samples2(Q, c, st, k, k + 1);
+    const Samples2 v = samples2(Q, c, st, k / 2);
     float2 p, m;
     ppm32x2(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m);
     qp[k] = p.x;
@@ -190,30 +190,24 @@ __device__ __forceinline__ bool contact_line32(float r0, float r1, float p0, flo
 // line10f with contact steepening of the density and species lines (the
 // gas-dynamics contact test of line10c over the two neighbours; gamma_k0 =
 // gamma K0, gm1 = gamma - 1).
-__device__ __forceinline__ void line10fc(const float* __restrict__ Q, int c, int st, float gamma_k0, float gm1,
+__device__ __forceinline__ void line10fc(const float2* __restrict__ Q, int c, int st, float gamma_k0, float gm1,
                                          float qp[F], float qm[F]) {
-  static_assert(RHO == 0 && SP0 == F - 1, "the steepened fields are the first and the last");
-  const bool contact = contact_line32(Q[RHO * S3 + c - st], Q[RHO * S3 + c + st],
-                                      __fmul_rn(gm1, Q[EGAS * S3 + c - st]), __fmul_rn(gm1, Q[EGAS * S3 + c + st]),
-                                      gamma_k0);
-  {
-    // density and species, steepened, as one pair
-    const Samples2 v = samples2(Q, c, st, RHO, SP0);
-    const float2 eta = contact ? f2(contact_eta32(v.s[0].x, v.s[1].x, v.s[2].x, v.s[3].x, v.s[4].x),
-                                    contact_eta32(v.s[0].y, v.s[1].y, v.s[2].y, v.s[3].y, v.s[4].y))
-                               : f2(0.f);
-    float2 p, m;
-    ppm32x2<1>(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m, eta);
-    qp[RHO] = p.x;
-    qp[SP0] = p.y;
-    qm[RHO] = m.x;
-    qm[SP0] = m.y;
-  }
+  static_assert(RHO == 0 && EGAS == 4 && SP0 == F - 1, "the steepened fields are the first and the last");
+  const bool contact =
+      contact_line32(Q[c - st].x, Q[c + st].x, __fmul_rn(gm1, Q[2 * S3 + c - st].x),
+                     __fmul_rn(gm1, Q[2 * S3 + c + st].x), gamma_k0);
 #pragma unroll
-  for (int k = 1; k < F - 1; k += 2) {
-    const Samples2 v = samples2(Q, c, st, k, k + 1);
+  for (int k = 0; k < F; k += 2) {
+    const Samples2 v = samples2(Q, c, st, k / 2);
     float2 p, m;
-    ppm32x2(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m);
+    if (k == 0)
+      ppm32x2<2>(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m,
+                 f2(contact ? contact_eta32(v.s[0].x, v.s[1].x, v.s[2].x, v.s[3].x, v.s[4].x) : 0.f));
+    else if (k == F - 2)
+      ppm32x2<3>(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m,
+                 f2(contact ? contact_eta32(v.s[0].y, v.s[1].y, v.s[2].y, v.s[3].y, v.s[4].y) : 0.f));
+    else
+      ppm32x2(v.s[0], v.s[1], v.s[2], v.s[3], v.s[4], p, m);
     qp[k] = p.x;
     qp[k + 1] = p.y;
     qm[k] = m.x;
@@ -383,11 +377,11 @@ __device__ __forceinline__ void unlimited32x2(const float2 s[5], float2& qp, flo
 // fields but the spin, which stays limited.  Two fields per packed
 // instruction, as line10f: about 200 instructions against its 330 (287 a field
 // at a time).
-__device__ __forceinline__ void line10u(const float* __restrict__ Q, int c, int st, float qp[F], float qm[F]) {
+__device__ __forceinline__ void line10u(const float2* __restrict__ Q, int c, int st, float qp[F], float qm[F]) {
   static_assert(ZX == 6 && ZZ == 8 && SP0 == 9, "pairs of fields");
 #pragma unroll
   for (int k = 0; k < F; k += 2) {
-    const Samples2 v = samples2(Q, c, st, k, k + 1);
+    const Samples2 v = samples2(Q, c, st, k / 2);
     float2 p, m;
     if (k < ZX)
       unlimited32x2(v.s, p, m);
@@ -562,12 +556,26 @@ __host__ __device__ constexpr GateOffsets make_gate_offsets() {
 }
 __constant__ const GateOffsets c_gate_off = make_gate_offsets();
 
+// Density and internal energy of a cell in the two layouts the indicator
+// reads: FP64 [F][S3], and the row sweep's FP32 pairs (both the first of their
+// pair).  neighbour: feature j's neighbour of cell c, in the feature's field.
+__device__ __forceinline__ double gate_rho(const double* Q, int c) { return Q[RHO * S3 + c]; }
+__device__ __forceinline__ double gate_eps(const double* Q, int c) { return Q[EGAS * S3 + c]; }
+__device__ __forceinline__ double gate_neighbour(const double* Q, int c, int j) {
+  return Q[RHO * S3 + c + c_gate_off.off[j]];
+}
+__device__ __forceinline__ float gate_rho(const float2* Q, int c) { return Q[RHO / 2 * S3 + c].x; }
+__device__ __forceinline__ float gate_eps(const float2* Q, int c) { return Q[EGAS / 2 * S3 + c].x; }
+__device__ __forceinline__ float gate_neighbour(const float2* Q, int c, int j) {
+  return Q[RHO / 2 * S3 + c + c_gate_off.off[j] - (j < 27 ? 0 : (EGAS - EGAS / 2) * S3)].x;
+}
+
 // One indicator feature (index j of 54) of the cell at padded index c:
 // (q(c + k_j) - q(c)) / (|q(c + k_j)| + |q(c)|), q = density (j < 27) or
 // pressure (gm1 * eps), k_j the j-th neighbour in (z, y, x) order.
 template <class T>
 __device__ __forceinline__ float gate_feature(const T* __restrict__ Q, int c, float rc, float pc, float gm1, int j) {
-  const float v = (float)Q[RHO * S3 + c + c_gate_off.off[j]];
+  const float v = (float)gate_neighbour(Q, c, j);
   const float qk = j < 27 ? v : gm1 * v;
   const float qc = j < 27 ? rc : pc;
   return __fdividef(qk - qc, fabsf(qk) + fabsf(qc));
@@ -582,8 +590,8 @@ __device__ __forceinline__ void gate_tile_mma(const T* __restrict__ Q, float gm1
                                               const GateFrags& f, int lane, float& logit0, float& logit1,
                                               bool& zero0, bool& zero1) {
   const int t = lane & 3;
-  const float r0 = (float)Q[RHO * S3 + c0], p0 = gm1 * (float)Q[EGAS * S3 + c0];
-  const float r1 = (float)Q[RHO * S3 + c1], p1 = gm1 * (float)Q[EGAS * S3 + c1];
+  const float r0 = (float)gate_rho(Q, c0), p0 = gm1 * (float)gate_eps(Q, c0);
+  const float r1 = (float)gate_rho(Q, c1), p1 = gm1 * (float)gate_eps(Q, c1);
   uint32_t a[4][4];
   bool nz0 = false, nz1 = false;
 #pragma unroll
@@ -661,9 +669,9 @@ template <class T, int kThreads>
 __device__ __forceinline__ void gate_phase(const T* __restrict__ Q, float gm1, const float* __restrict__ gate_w,
                                            float logit_thr, int zero_smooth, uint8_t* smooth, uint8_t* pred) {
   const int tid = threadIdx.x;
-  const T r0 = Q[RHO * S3], e0 = Q[EGAS * S3];
+  const auto r0 = gate_rho(Q, 0), e0 = gate_eps(Q, 0);
   bool same = true;
-  for (int c = tid; c < S3; c += kThreads) same &= (Q[RHO * S3 + c] == r0) & (Q[EGAS * S3 + c] == e0);
+  for (int c = tid; c < S3; c += kThreads) same &= (gate_rho(Q, c) == r0) & (gate_eps(Q, c) == e0);
   if (__syncthreads_and(same)) {
     for (int c = tid; c < S3; c += kThreads) smooth[c] = (uint8_t)zero_smooth;
     __syncthreads();

@@ -26,7 +26,7 @@ namespace hyd {
 
 constexpr int kThreadsMx = NROW;  // 192
 
-// Dynamic shared memory of one CTA: FP32 primitives [F][S3], then two
+// Dynamic shared memory of one CTA: FP32 primitives [F/2][S3][2], then two
 // [S3] byte arrays of smooth flags (learned indicator), then the FP32 cell-
 // centre coordinates x_c, y_c of the reconstructed cells (sub_coords).
 constexpr size_t kMixedSmemBytes = (size_t)F * S3 * sizeof(float) + 2 * S3 + 2 * (N + 2) * sizeof(float);
@@ -140,9 +140,9 @@ __device__ __forceinline__ void finish_cell(const StepArgs64& A, const Io& io, c
 // a barrier, so the next sub-grid may reuse all of them.
 // kContact: contact steepening of the density and species lines (line10fc).
 template <bool kGate, bool kContact = false, bool kSpin = false, class Io>
-__device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io, int s, const RowMap& R, float* Qf,
+__device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io, int s, const RowMap& R, float2* Qf,
                                               float* red, double* __restrict__ D) {
-  uint8_t* smooth = reinterpret_cast<uint8_t*>(Qf + F * S3);
+  uint8_t* smooth = reinterpret_cast<uint8_t*>(Qf + F / 2 * S3);
   float* coord = reinterpret_cast<float*>(smooth + 2 * S3);
   const int tid = threadIdx.x;
   const int a = R.a, b = R.b, pb = R.pb, pc = R.pc, sa = R.sa, sb = R.sb, sc = R.sc;
@@ -168,14 +168,14 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
       bad |= !prims_mixed(u, A.P.eta1, PF.gamma, q);
     }
 #pragma unroll
-    for (int k = 0; k < F; ++k) Qf[k * S3 + c] = q[k];
+    for (int k = 0; k < F / 2; ++k) Qf[k * S3 + c] = f2(q[2 * k], q[2 * k + 1]);
   }
   if (bad) atomicOr(A.status, 1u);
   __syncthreads();
 
   // ---- 2b. learned smoothness indicator (gate_phase) ---------------------
   if (kGate)
-    gate_phase<float, kThreadsMx>(Qf, PF.gm1, A.gate_w, A.gate_logit_thr, A.gate_zero_smooth, smooth, smooth + S3);
+    gate_phase<float2, kThreadsMx>(Qf, PF.gm1, A.gate_w, A.gate_logit_thr, A.gate_zero_smooth, smooth, smooth + S3);
 
   // ---- 3. row sweep in FP32 --------------------------------------------
   const float h = (float)hd, half_h = 0.5f * h;
@@ -226,8 +226,8 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
       if constexpr (kSpin) {
         // the cell's spin fed back into the velocity at both ends of both
         // lines (spin_dv32; the plane sweep's values, bit for bit)
-        const float rc = Qf[RHO * S3 + cj], ec = Qf[EGAS * S3 + cj], zx = Qf[ZX * S3 + cj],
-                    zy = Qf[ZY * S3 + cj], zz = Qf[ZZ * S3 + cj], gg1 = __fmul_rn(PF.gamma, PF.gm1);
+        const float rc = Qf[cj].x, ec = Qf[2 * S3 + cj].x, zx = Qf[3 * S3 + cj].x, zy = Qf[3 * S3 + cj].y,
+                    zz = Qf[4 * S3 + cj].x, gg1 = __fmul_rn(PF.gamma, PF.gm1);
         float dv[3];
         spin_dv32(rc, ec, zx, zy, zz, PF.k3h, gg1, axis_comp(0, a, b, 1, t1, t2), axis_comp(1, a, b, 1, t1, t2),
                   axis_comp(2, a, b, 1, t1, t2), dv);

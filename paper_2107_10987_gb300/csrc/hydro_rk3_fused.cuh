@@ -224,11 +224,11 @@ struct RowBody {
   static constexpr size_t kRed = (kMixedSmemBytes + 15) / 16 * 16;
   static constexpr size_t kSmem = kRed + sizeof(float) * (kThreadsMx / 32);
   RowMap R;
-  float* Qf;
+  float2* Qf;
   float* red;
   double* D;
   __device__ RowBody(const StepArgs64& S, unsigned char* sm)
-      : R(row_map(threadIdx.x)), Qf(reinterpret_cast<float*>(sm)), red(reinterpret_cast<float*>(sm + kRed)),
+      : R(row_map(threadIdx.x)), Qf(reinterpret_cast<float2*>(sm)), red(reinterpret_cast<float*>(sm + kRed)),
         D(S.scratch + (size_t)blockIdx.x * kScratchPerSub) {}
   template <class Io>
   __device__ __forceinline__ void run(const StepArgs64& S, const Io& io, int s) const {

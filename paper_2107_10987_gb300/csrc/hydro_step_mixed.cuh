@@ -67,7 +67,7 @@ struct StepIo {
 // other instances carry none of.
 template <bool kGate, bool kContact = false, int NN = N, bool kSpin = false>
 __global__ void __launch_bounds__(kThreadsMx, 2) hydro_step_mixed_kernel(StepArgs64 A) {
-  extern __shared__ __align__(128) float Qf[];  // [F][S3] FP32 primitives, then [2][S3] smooth flags
+  extern __shared__ __align__(128) float2 Qf[];  // [F/2][S3] FP32 primitive pairs, then [2][S3] smooth flags
   __shared__ float red[kThreadsMx / 32];
   double* __restrict__ D = A.scratch + (size_t)blockIdx.x * kScratchPerSub;
   const RowMap R = row_map(threadIdx.x);
