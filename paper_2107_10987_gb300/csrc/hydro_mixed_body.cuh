@@ -247,21 +247,18 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
         }
       }
       if (j >= 0) {
-        // the pair's two points (n = 2p, 2p + 1) in the two lanes; the centre
-        // in both
+        // the pair's points n = 2p and 2p + 1, or the centre
         const int nA = 2 * p, nB = kTwo ? nA + 1 : nA;
-        const int u1A = face_u1(nA), u2A = face_u2(nA), u1B = face_u1(nB), u2B = face_u2(nB);
-        const int ptA = (u1A + 1) * 3 + (u2A + 1), ptB = (u1B + 1) * 3 + (u2B + 1);
-        float2 dL[3];
-#pragma unroll
-        for (int m = 0; m < 3; ++m)
-          dL[m] = f2((float)axis_comp(m, a, b, 1, u1A, u2A), (float)axis_comp(m, a, b, 1, u1B, u2B));
-        const float2 xq = fma2(f2(half_h), dL[0], f2(xc)), yq = fma2(f2(half_h), dL[1], f2(yc));
-        const float wA = face_w(u1A, u2A, npt), wB = face_w(u1B, u2B, npt);
-        point_pair32<kTwo>([&](int k) { return plus[ptA][k]; }, [&](int k) { return qmA[k]; },
-                           [&](int k) { return plus[ptB][k]; }, [&](int k) { return kTwo ? qmB[k] : qmA[k]; }, a,
-                           xq, yq, dL, PF, 0.5f * wA, 0.5f * __fmul_rn(wA, half_h), 0.5f * wB,
-                           0.5f * __fmul_rn(wB, half_h), Gf, Gtl, amax);
+        auto point = [&](int n, const float* qR) {
+          const int u1 = face_u1(n), u2 = face_u2(n);
+          const float w = face_w(u1, u2, npt);
+          const float e1 = u1 == 0 ? 0.f : u1 > 0 ? 1.f : -1.f, e2 = u2 == 0 ? 0.f : u2 > 0 ? 1.f : -1.f;
+          point32(plus[(u1 + 1) * 3 + (u2 + 1)], qR, a, a == 0 ? PF.omega : a == 1 ? -PF.omega : 0.f,
+                  __fmaf_rn(half_h, e1, a == 0 ? yc : xc), a == 0 ? 1.f : e1, a == 1 ? 1.f : a == 0 ? e1 : e2,
+                  a == 2 ? 1.f : e2, PF, 0.5f * w, 0.5f * __fmul_rn(w, half_h), Gf, Gtl, amax);
+        };
+        point(nA, qmA);
+        if (kTwo) point(nB, qmB);
         // a group is complete after points 3, 5 and 8 (face_group_ends, never
         // inside a pair): S = G0, then (S + G1), then (S + G2)
         if (face_group_ends(nB)) {

@@ -163,7 +163,7 @@ __device__ __forceinline__ void plane_line(const float2* __restrict__ ring, int 
   quarter(dp, 0, p0, p1);
   if (dm) quarter(dm, 0, m0, m1);
   pair(integral_constant<int, 2>{}, p2, m2);
-  // E, p, c^2 and 1/c of an end (side32x2's operations)
+  // E, p, c^2 and 1/c of an end (point32's operations)
   auto end = [&](unsigned char* d, float2 q0, float2 q1, float2 q2) {
     const float v2 = __fmaf_rn(q1.y, q1.y, __fmaf_rn(q1.x, q1.x, __fmul_rn(q0.y, q0.y)));
     const float E = __fmaf_rn(__fmul_rn(0.5f, q0.x), v2, q2.x);
@@ -191,7 +191,7 @@ struct SideRef {
   }
 };
 
-// One quadrature point of a face (point_pair32's operations on one point,
+// One quadrature point of a face (point32's operations,
 // two fields in the two lanes), added to a group's sums G (field pairs) and
 // the torque about the left cell TL.  w: the point's weight.
 template <int u1, int u2>
