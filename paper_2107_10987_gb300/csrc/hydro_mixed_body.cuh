@@ -21,6 +21,7 @@
 #pragma once
 #include <type_traits>
 #include "hydro_mixed.cuh"
+#include "hydro_tmem.cuh"
 
 namespace hyd {
 
@@ -136,12 +137,13 @@ __device__ __forceinline__ void finish_cell(const StepArgs64& A, const Io& io, c
 //   io.face(sub, f, q, pc, pb, v)  boundary-face value (tile face f)
 //   io.amax(sub, m)           the tile's maximum signal speed (thread 0)
 // Qf: the CTA's dynamic shared memory; red: [kThreadsMx / 32] floats of
-// shared memory; D: the CTA's scratch (kScratchPerSub doubles).  Ends with
-// a barrier, so the next sub-grid may reuse all of them.
+// shared memory; D: the CTA's scratch (kScratchPerSub doubles); tm: the
+// thread's tensor memory (tmem_alloc).  Ends with a barrier, so the next
+// sub-grid may reuse all of them.
 // kContact: contact steepening of the density and species lines (line10fc).
 template <bool kGate, bool kContact = false, bool kSpin = false, class Io>
 __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io, int s, const RowMap& R, float2* Qf,
-                                              float* red, double* __restrict__ D) {
+                                              float* red, double* __restrict__ D, uint32_t tm) {
   uint8_t* smooth = reinterpret_cast<uint8_t*>(Qf + F / 2 * S3);
   float* coord = reinterpret_cast<float*>(smooth + 2 * S3);
   const int tid = threadIdx.x;
@@ -180,7 +182,6 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
   // ---- 3. row sweep in FP32 --------------------------------------------
   const float h = (float)hd, half_h = 0.5f * h;
   float amax = 0.f;
-  float plus[9][F];
   // the previous face's sums and right-cell torques, converted to FP64 once
   // (exact conversions of the FP32 sums)
   double fprev[F], trprev[3];
@@ -190,6 +191,7 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
 #pragma unroll 1
   for (int j = -1; j <= N; ++j) {
     const int cj = c0 + j * sa;
+    tmem_wait_st();  // cell j - 1's plus-states
     // face j-1/2: completed groups S (fluxes, left-cell torques) and the
     // group being summed, G
     float Sf[F], Stl[3], Gf[F], Gtl[3];
@@ -212,7 +214,7 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
       constexpr bool kTwo = decltype(two)::value;
       const int t1 = p / 3 - 1, t2 = p % 3 - 1;
       float qpA[F], qmA[F], qpB[F], qmB[F];
-      if (kGate && smooth[cj]) {
+      if (kGate && smooth[cj]) {  // (per thread)
         line10u(Qf, cj, sa + t1 * sb + t2 * sc, qpA, qmA);
         if (kTwo) line10u(Qf, cj, sa - t1 * sb - t2 * sc, qpB, qmB);
       } else if (kContact) {
@@ -223,6 +225,7 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
         line10f(Qf, cj, sa + t1 * sb + t2 * sc, qpA, qmA);
         if (kTwo) line10f(Qf, cj, sa - t1 * sb - t2 * sc, qpB, qmB);
       }
+      if (kGate) __syncwarp();
       if constexpr (kSpin) {
         // the cell's spin fed back into the velocity at both ends of both
         // lines (spin_dv32; the plane sweep's values, bit for bit)
@@ -253,7 +256,9 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
           const int u1 = face_u1(n), u2 = face_u2(n);
           const float w = face_w(u1, u2, npt);
           const float e1 = u1 == 0 ? 0.f : u1 > 0 ? 1.f : -1.f, e2 = u2 == 0 ? 0.f : u2 > 0 ? 1.f : -1.f;
-          point32(plus[(u1 + 1) * 3 + (u2 + 1)], qR, a, a == 0 ? PF.omega : a == 1 ? -PF.omega : 0.f,
+          float qL[F];
+          tmem_ld(tm, (u1 + 1) * 3 + (u2 + 1), qL);
+          point32(qL, qR, a, a == 0 ? PF.omega : a == 1 ? -PF.omega : 0.f,
                   __fmaf_rn(half_h, e1, a == 0 ? yc : xc), a == 0 ? 1.f : e1, a == 1 ? 1.f : a == 0 ? e1 : e2,
                   a == 2 ? 1.f : e2, PF, 0.5f * w, 0.5f * __fmul_rn(w, half_h), Gf, Gtl, amax);
         };
@@ -275,11 +280,8 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
           first = false;
         }
       }
-#pragma unroll
-      for (int k = 0; k < F; ++k) {
-        plus[p][k] = qpA[k];
-        if (kTwo) plus[8 - p][k] = qpB[k];
-      }
+      tmem_st(tm, p, qpA);
+      if (kTwo) tmem_st(tm, 8 - p, qpB);
     };
 #pragma unroll 1
     for (int p = npt == 1 ? 4 : 0; p < 4; ++p) pair_step(p, std::integral_constant<bool, true>{});

@@ -73,7 +73,11 @@ __global__ void __launch_bounds__(kThreadsMx, 2) hydro_step_mixed_kernel(StepArg
   const RowMap R = row_map(threadIdx.x);
   const StepIo<NN> io{A};
   const int units = A.n_sub * Tile<NN>::kTiles;
-  for (int u = blockIdx.x; u < units; u += gridDim.x) mixed_subgrid<kGate, kContact, kSpin>(A, io, u, R, Qf, red, D);
+  __shared__ uint32_t sh_tm;
+  const uint32_t tm = tmem_alloc(&sh_tm);
+  for (int u = blockIdx.x; u < units; u += gridDim.x)
+    mixed_subgrid<kGate, kContact, kSpin>(A, io, u, R, Qf, red, D, tm);
+  tmem_free(tm);
 }
 
 // The plane sweep: one CTA of kThreadsPl threads per SM (no indicator).

@@ -85,11 +85,14 @@ __global__ void __launch_bounds__(kThreadsMx, 2) hydro_step_mixed_amr_kernel(Ste
   __shared__ float red[kThreadsMx / 32];
   double* __restrict__ D = A.scratch + (size_t)blockIdx.x * kScratchPerSub;
   const RowMap R = row_map(threadIdx.x);
+  __shared__ uint32_t sh_tm;
+  const uint32_t tm = tmem_alloc(&sh_tm);
   const AmrStepIo io{A, M};
   for (int u = blockIdx.x; u < A.n_sub; u += gridDim.x) {
     const int s = leaf_at(M, u);  // the same for the whole CTA
-    if (s >= 0) mixed_subgrid<kGate>(A, io, s, R, Qf, red, D);
+    if (s >= 0) mixed_subgrid<kGate>(A, io, s, R, Qf, red, D, tm);
   }
+  tmem_free(tm);
 }
 
 // The plane sweep (no indicator): one CTA per SM.
