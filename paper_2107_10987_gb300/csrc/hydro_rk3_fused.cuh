@@ -227,17 +227,13 @@ struct RowBody {
   float2* Qf;
   float* red;
   double* D;
-  uint32_t tm;  // held until the kernel returns, from wherever
   __device__ RowBody(const StepArgs64& S, unsigned char* sm)
       : R(row_map(threadIdx.x)), Qf(reinterpret_cast<float2*>(sm)), red(reinterpret_cast<float*>(sm + kRed)),
-        D(S.scratch + (size_t)blockIdx.x * kScratchPerSub) {
-    __shared__ uint32_t sh_tm;
-    tm = tmem_alloc(&sh_tm);
-  }
-  __device__ ~RowBody() { tmem_free(tm); }
+        D(S.scratch + (size_t)blockIdx.x * kScratchPerSub) {}
   template <class Io>
   __device__ __forceinline__ void run(const StepArgs64& S, const Io& io, int s) const {
-    mixed_subgrid<kGate, kContact, kSpin>(S, io, s, R, Qf, red, D, tm);
+    RowPlusLocal plus;  // (not in tensor memory: hydro_tmem.cuh)
+    mixed_subgrid<kGate, kContact, kSpin>(S, io, s, R, Qf, red, D, plus);
   }
 };
 template <bool kContact, bool kSpin = false>

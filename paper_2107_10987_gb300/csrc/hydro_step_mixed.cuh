@@ -74,10 +74,10 @@ __global__ void __launch_bounds__(kThreadsMx, 2) hydro_step_mixed_kernel(StepArg
   const StepIo<NN> io{A};
   const int units = A.n_sub * Tile<NN>::kTiles;
   __shared__ uint32_t sh_tm;
-  const uint32_t tm = tmem_alloc(&sh_tm);
+  RowPlusTmem plus{tmem_alloc(&sh_tm)};
   for (int u = blockIdx.x; u < units; u += gridDim.x)
-    mixed_subgrid<kGate, kContact, kSpin>(A, io, u, R, Qf, red, D, tm);
-  tmem_free(tm);
+    mixed_subgrid<kGate, kContact, kSpin>(A, io, u, R, Qf, red, D, plus);
+  tmem_free(plus.t);
 }
 
 // The plane sweep: one CTA of kThreadsPl threads per SM (no indicator).

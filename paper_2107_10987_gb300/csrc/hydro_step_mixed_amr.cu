@@ -86,13 +86,13 @@ __global__ void __launch_bounds__(kThreadsMx, 2) hydro_step_mixed_amr_kernel(Ste
   double* __restrict__ D = A.scratch + (size_t)blockIdx.x * kScratchPerSub;
   const RowMap R = row_map(threadIdx.x);
   __shared__ uint32_t sh_tm;
-  const uint32_t tm = tmem_alloc(&sh_tm);
+  RowPlusTmem plus{tmem_alloc(&sh_tm)};
   const AmrStepIo io{A, M};
   for (int u = blockIdx.x; u < A.n_sub; u += gridDim.x) {
     const int s = leaf_at(M, u);  // the same for the whole CTA
-    if (s >= 0) mixed_subgrid<kGate>(A, io, s, R, Qf, red, D, tm);
+    if (s >= 0) mixed_subgrid<kGate>(A, io, s, R, Qf, red, D, plus);
   }
-  tmem_free(tm);
+  tmem_free(plus.t);
 }
 
 // The plane sweep (no indicator): one CTA per SM.
