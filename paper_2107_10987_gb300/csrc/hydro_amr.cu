@@ -321,15 +321,27 @@ __global__ void __launch_bounds__(256) hydro_ghost_amr_prolong_kernel(AMRArgs A)
       // additions, in the same order, as prolonging child by child
       const int need_x = ((mask & 0x55) ? 1 : 0) | ((mask & 0xaa) ? 2 : 0);  // children with x offset -, +
       double* dst0 = dstb + ((2 * C[2] - b[2] + G) * LS + (2 * C[1] - b[1] + G)) * LS + (2 * C[0] - b[0] + G);
+      // the next field's seven values load while this one's children form
+      double cn, qpn[3], qmn[3];
+      auto fetch = [&](int k) {
+        cn = Cp[(size_t)k * LS3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          qpn[d] = nbp[2 * d + 1][(size_t)k * nbs[2 * d + 1]];
+          qmn[d] = nbp[2 * d][(size_t)k * nbs[2 * d]];
+        }
+      };
+      fetch(0);
 #pragma unroll 1
       for (int k = 0; k < F; ++k) {
-        const double c = Cp[(size_t)k * LS3];
+        const double c = cn;
         double qp[3], qm[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          qp[d] = nbp[2 * d + 1][(size_t)k * nbs[2 * d + 1]];
-          qm[d] = nbp[2 * d][(size_t)k * nbs[2 * d]];
+          qp[d] = qpn[d];
+          qm[d] = qmn[d];
         }
+        if (k + 1 < F) fetch(k + 1);
         // A coarse cell whose six neighbours have its bits (finite, not -0:
         // a uniform region) has the slopes c - c = +0, and every child is
         // ((c -+ 0) -+ 0) -+ 0 = c exactly: stored without the FP64 work.
@@ -714,12 +726,16 @@ int hydro_fill_ghosts_amr(hydro_ctx_t* c, const hydro_batch_t* B, const hydro_am
   const int cap = c->num_sms * 8;
   const int grid = B->n_sub < cap ? B->n_sub : cap;
   cudaStream_t st = (cudaStream_t)stream;
+  // (the prolongation and the flux correction have work in few leaves: a block
+  // per leaf, handed out as blocks end, where persistent blocks of up to four
+  // leaves each waited for the unluckiest; with the prefetch the mixed step of
+  // 4,040 leaves went from 7.71 to 7.64 ms)
   if (c->N == 16) {
     hyd::hydro_ghost_amr_kernel<16><<<grid, 256, 0, st>>>(A);
-    hyd::hydro_ghost_amr_prolong_kernel<16, false><<<grid, 256, 0, st>>>(A);
+    hyd::hydro_ghost_amr_prolong_kernel<16, false><<<B->n_sub, 256, 0, st>>>(A);
   } else {
     hyd::hydro_ghost_amr_kernel<8><<<grid, 256, 0, st>>>(A);
-    hyd::hydro_ghost_amr_prolong_kernel<8, false><<<grid, 256, 0, st>>>(A);
+    hyd::hydro_ghost_amr_prolong_kernel<8, false><<<B->n_sub, 256, 0, st>>>(A);
   }
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
 }
@@ -732,12 +748,10 @@ int hydro_flux_correct_amr(hydro_ctx_t* c, const hydro_batch_t* B, const hydro_a
   int rc = hydro_ctx_prepare(c, 0);
   if (rc) return rc;
   hyd::AMRArgs A = hydro_amr_args(c, B, M);
-  const int cap = c->num_sms * 8;
-  const int grid = B->n_sub < cap ? B->n_sub : cap;
   if (c->N == 16)
-    hyd::hydro_flux_correct_kernel<16, false><<<grid, 256, 0, (cudaStream_t)stream>>>(A, B->h, face_flux, dUdt);
+    hyd::hydro_flux_correct_kernel<16, false><<<B->n_sub, 256, 0, (cudaStream_t)stream>>>(A, B->h, face_flux, dUdt);
   else
-    hyd::hydro_flux_correct_kernel<8, false><<<grid, 256, 0, (cudaStream_t)stream>>>(A, B->h, face_flux, dUdt);
+    hyd::hydro_flux_correct_kernel<8, false><<<B->n_sub, 256, 0, (cudaStream_t)stream>>>(A, B->h, face_flux, dUdt);
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
 }
 
@@ -764,7 +778,7 @@ int hydro_fill_ghosts_amr_lean(hydro_ctx_t* c, const hydro_batch_t* B, const hyd
     hyd::hydro_amr_restrict_kernel<8><<<grid, 256, 0, st>>>(B->U, c->amr_img, B->n_sub);
     hyd::hydro_amr_finer_kernel<8><<<(8 * B->n_sub + 255) / 256, 256, 0, st>>>(A);
   }
-  hyd::hydro_ghost_amr_prolong_kernel<8, true><<<grid, 256, 0, st>>>(A);
+  hyd::hydro_ghost_amr_prolong_kernel<8, true><<<B->n_sub, 256, 0, st>>>(A);
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
 }
 
@@ -792,7 +806,7 @@ int hydro_update_amr_lean(hydro_ctx_t* c, const hydro_batch_t* B, const hydro_am
   const bool mixed = c->mode.precision == HYDRO_PREC_MIXED;
   const double eta2 = c->mode.de_eta2, ig = 1.0 / c->gamma;
   const double al = alpha[stage], be = beta[stage];
-  hyd::hydro_flux_correct_kernel<8, true><<<grid, 256, 0, st>>>(A, B->h, face_flux, dUdt);
+  hyd::hydro_flux_correct_kernel<8, true><<<B->n_sub, 256, 0, st>>>(A, B->h, face_flux, dUdt);
   if (mixed && image)
     hyd::hydro_update_amr_kernel<true, true><<<grid, 256, 0, st>>>(A, dUdt, U0, Uout, dt_dev, al, be, eta2, ig);
   else if (mixed)
