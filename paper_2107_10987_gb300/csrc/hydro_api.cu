@@ -98,9 +98,9 @@ static int ensure_buf(hydro_ctx* c, double** buf, size_t* have, size_t need, con
 // (mixed precision; FP64 and the learned indicator have the row sweep): what
 // hydro_set_launch or the autotuner chose, else the plane sweep for a batch
 // of at most one tile per SM, the row sweep for more.  A tile alone on an SM
-// takes the plane sweep 95 us and the row sweep 155; two row-sweep tiles share
-// an SM in 166 (304 tiles 0.176 ms; 400 tiles 0.278 against 0.272 for planes,
-// 700 tiles 0.42 against 0.45).
+// takes the plane sweep 94 us and the row sweep 109; two row-sweep tiles share
+// an SM in 150 (planes: 182 for the two; 200 tiles 147 against 181, 400 tiles
+// 240 against 273, 700 tiles 363 against 449).
 static int eff_decomp(const hydro_ctx* c, int units) {
   if (c->mode.precision != HYDRO_PREC_MIXED || c->gate_on) return HYDRO_DECOMP_ROWS;
   if (c->decomp != HYDRO_DECOMP_AUTO) return c->decomp;
