@@ -34,7 +34,7 @@
 // SM (phase A alone 25 us of a tile's 95, the face fluxes 14, phase C 15, the
 // conversion of a padded FP64 state 14, the first planes and the last finish
 // 25; measured with the others left out).  A row sweep with two tiles on the
-// SM overlaps them and takes 83 us a tile, but 160 for one alone, so the
+// SM overlaps them and takes 68 us a tile, but 109 for one alone, so the
 // dispatch gives this sweep the batches of at most one tile per SM (77 leaves
 // with contact steepening and spin: 173 -> 101 us).  Two fields of a line share
 // each packed instruction in phase A, and two fields of a point in phase B:
@@ -46,9 +46,8 @@
 // The arithmetic is the row sweep's own: the same ppm32x2 on the same samples
 // (exactly symmetric under reversal of a line, so the orientation in which a
 // line is evaluated does not matter; each lane rounds alike whichever field
-// or line shares its instruction), the same point flux on the same pairs
-// in the same order, the same grouping of
-// each face sum, the same FP64 differences and finish_cell.  The two
+// or line shares its instruction), the same point flux on the same points
+// in the same order, the same grouping of each face sum, the same FP64 differences and finish_cell.  The two
 // decompositions therefore give the same bits.
 #pragma once
 #include <type_traits>
