@@ -211,7 +211,7 @@ int hydro_autotune_step(hydro_ctx_t* ctx, const hydro_batch_t* B, double* dUdt, 
  * the decomposition (HYDRO_DECOMP_*; mixed precision only, the FP64 kernels
  * have rows alone) and the number of persistent CTAs of hydro_step (0: the
  * decomposition's default, one or two per SM).  The fused RK3 step runs the
- * decomposition with as many CTAs as can be resident.  Not in the paper.
+ * decomposition with its default number of CTAs.  Not in the paper.
  * Errors: EINVAL (unknown decomposition, ctas < 0), EUNSUP (PLANES in FP64). */
 int hydro_set_launch(hydro_ctx_t* ctx, int decomposition, int ctas);
 
@@ -375,11 +375,11 @@ typedef struct {
    * buffers held by same-level or finer leaves are then not written. */
   const hydro_amr_t* amr;
   double* face_flux;  /* [n_sub][6][F+3][N][N], used with amr */
-  /* Nonzero: the whole time step as one persistent launch (uniform mesh and
+  /* Nonzero: the whole time step as four launches (uniform mesh and
    * HYDRO_PREC_MIXED only; otherwise the step returns EUNSUP).  Ghost cells
    * are read from the neighbouring sub-grids' interiors instead of being
    * filled (in the context's decomposition, hydro_set_launch), stages 1 and
-   * 2 apply their update inside the launch, and a
+   * 2 apply their update inside one launch, and a
    * sub-grid's third stage starts as soon as its 27 neighbours have finished
    * their second (bounded waits; HYDRO_ST_TIMEOUT if one expires).  The
    * interiors of the new state and *dt equal the separate launches' bit for
@@ -391,8 +391,8 @@ typedef struct {
 typedef struct hydro_graph hydro_graph_t;
 
 /* Enqueue one time step on a stream: parity 0 advances a -> b, 1 advances
- * b -> a.  Ten launches on a uniform mesh (two with fused: a clear of the
- * context's sync words and the step); on an adaptive mesh 16 (five per
+ * b -> a.  Ten launches on a uniform mesh (five with fused: a clear of the
+ * context's sync words and four kernels); on an adaptive mesh 16 (five per
  * stage and dt), or 15 in the direct-read form (four per stage, two more at
  * the first stage for its restriction images and finer-neighbour tables,
  * and dt).  Errors: EINVAL (inconsistent descriptor, or state

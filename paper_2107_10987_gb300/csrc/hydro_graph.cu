@@ -4,7 +4,7 @@
 // graphs that are replayed step after step.
 //
 // One time step (three hydro iterations, Sec. IV-A.2), state X -> Y (the
-// fused form, one persistent launch for a uniform mesh in mixed precision,
+// fused form, four launches for a uniform mesh in mixed precision,
 // is in hydro_rk3_fused.cu):
 //   ghost(X); step(X) -> dU, amax; dt = cfl min h/amax; Y = X + dt dU
 //   ghost(Y); step(Y);            Y = 3/4 X + 1/4 (Y + dt dU)

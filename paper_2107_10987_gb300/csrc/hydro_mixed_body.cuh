@@ -148,9 +148,9 @@ __device__ __forceinline__ void finish_cell(const StepArgs64& A, const Io& io, c
 // thread's plus-states (hydro_tmem.cuh).  Ends with a barrier, so the next
 // sub-grid may reuse all of them.
 // kContact: contact steepening of the density and species lines (line10fc).
-template <bool kGate, bool kContact = false, bool kSpin = false, class Plus, class Io>
+template <bool kGate, bool kContact = false, bool kSpin = false, class Io>
 __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io, int s, const RowMap& R, float2* Qf,
-                                              float* red, double* __restrict__ D, Plus& plus) {
+                                              float* red, double* __restrict__ D, RowPlusTmem plus) {
   uint8_t* smooth = reinterpret_cast<uint8_t*>(Qf + F / 2 * S3);
   float* coord = reinterpret_cast<float*>(smooth + 2 * S3);
   const int tid = threadIdx.x;
@@ -204,7 +204,7 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
 #pragma unroll 1
   for (int j = -1; j <= N; ++j) {
     const int cj = c0 + j * sa;
-    plus_next(plus);  // cell j - 1's plus-states
+    plus.next();  // cell j - 1's plus-states
     // face j-1/2: completed groups S (fluxes, left-cell torques) and the
     // group being summed, G
     float Sf[F], Stl[3], Gf[F], Gtl[3];
@@ -269,7 +269,7 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
           const int u1 = face_u1(n), u2 = face_u2(n);
           const float w = face_w(u1, u2, npt);
           const float e1 = u1 == 0 ? 0.f : u1 > 0 ? 1.f : -1.f, e2 = u2 == 0 ? 0.f : u2 > 0 ? 1.f : -1.f;
-          const auto qL = plus_record(plus, (u1 + 1) * 3 + (u2 + 1));
+          const auto qL = plus.record((u1 + 1) * 3 + (u2 + 1));
           point32(qL, qR, a, a == 0 ? PF.omega : a == 1 ? -PF.omega : 0.f,
                   __fmaf_rn(half_h, e1, a == 0 ? yc : xc), a == 0 ? 1.f : e1, a == 1 ? 1.f : a == 0 ? e1 : e2,
                   a == 2 ? 1.f : e2, PF, 0.5f * w, 0.5f * __fmul_rn(w, half_h), Gf, Gtl, amax);
@@ -292,8 +292,8 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
           first = false;
         }
       }
-      plus_store(plus, p, qpA);
-      if (kTwo) plus_store(plus, 8 - p, qpB);
+      plus.store(p, qpA);
+      if (kTwo) plus.store(8 - p, qpB);
     };
 #pragma unroll 1
     for (int p = npt == 1 ? 4 : 0; p < 4; ++p) pair_step(p, std::integral_constant<bool, true>{});

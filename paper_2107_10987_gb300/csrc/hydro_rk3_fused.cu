@@ -27,7 +27,7 @@ cudaError_t launch_wait_selftest(unsigned* words, unsigned* status, long long li
   return cudaGetLastError();
 }
 
-size_t rk3_fused_sync_words(int n_sub) { return (size_t)kSyncHead + 2 * (size_t)n_sub; }
+size_t rk3_fused_sync_words(int n_sub) { return (size_t)kSyncHead + (size_t)n_sub; }
 
 // Both the plain instances and those with the spin feedback (once per
 // device), so that a capture finds either ready; *max_grid for the plain ones.

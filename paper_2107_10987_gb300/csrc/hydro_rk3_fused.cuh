@@ -3,36 +3,41 @@
 // hydro_rk3_fused16.cu.
 //
 // One whole SSP-RK3 time step (three hydro iterations,
-// Sec. IV-A.2) of a uniform mesh in mixed precision, as one persistent
-// cooperative launch.
+// Sec. IV-A.2) of a uniform mesh in mixed precision, as four launches.
 //
 // The separate-launch step (hydro_graph.cu) runs per stage a ghost fill, the
 // step kernel and the update, with the whole mesh finishing each launch
 // before the next starts.  Here, state X -> Y:
-//   stage 0  every sub-grid: dU0 = L(X), amax (static schedule);
-//            one grid-wide barrier; dt = cfl min h/amax (every CTA); each
-//            CTA writes U1 = X + dt dU0 (with the tracer resync) of its
-//            stage-0 sub-grids into the interiors of Y and publishes them;
-//   stage 1  sub-grid s reads U1 and writes U2 = 3/4 X + 1/4 (U1 + dt L(U1))
-//            to an interior-only scratch and publishes it;
-//   stage 2  sub-grid s reads U2 and writes U3 = 1/3 X + 2/3 (U2 + dt L(U2))
+//   prims    the primitives of X;
+//   stage 0  every sub-grid: dU0 = L(X), amax;
+//   first    dt = cfl min h/amax (every CTA); U1 = X + dt dU0 (with the tracer
+//            resync) into the interiors of Y;
+//   fused    stage 1: sub-grid s reads U1 and writes U2 = 3/4 X + 1/4 (U1 + dt
+//            L(U1)) to an interior-only scratch and publishes it; stage 2:
+//            sub-grid s reads U2 and writes U3 = 1/3 X + 2/3 (U2 + dt L(U2))
 //            into the interiors of Y.
 // Ghost cells are read straight from the neighbouring sub-grids' interiors
 // through the boundary map of hydro_fill_ghosts_uniform, so no ghost layer
 // is written and no separate update runs.  Stage-1 and stage-2 sub-grids come
-// from one work counter, all stage-1 ones first; a sub-grid waits until its
-// 27 neighbours (itself included) have published its input (U1, U2).  U3
-// overwrites U1 in Y only after every reader of that U1 (the neighbours'
-// stage 1) has published.  The waits end: every CTA writes its U1 before it
-// takes a unit, so a stage-1 unit waits only for CTAs that are not waiting,
-// and a stage-2 unit waits only for stage-1 units, all taken before it by
-// resident CTAs.  Each wait is still bounded in time and polls and reports
-// HYDRO_ST_TIMEOUT.
+// from one work counter, all stage-1 ones first; a stage-2 sub-grid waits until
+// its 27 neighbours (itself included) have published their U2.  U3 overwrites
+// U1 in Y only after every reader of that U1 (the neighbours' stage 1) has
+// published.  The waits end: a stage-2 unit waits only for stage-1 units, all
+// taken before it by running CTAs that wait for none.  Each wait is still
+// bounded in time and polls and reports HYDRO_ST_TIMEOUT.
+//
+// Four launches and not one cooperative one with grid barriers in the places of
+// the first three boundaries: a cooperative launch takes one CTA per SM of a
+// kernel that allocates tensor memory, where the row sweep keeps its
+// plus-states (hydro_tmem.cuh), and no CTA here waits for one that might not be
+// resident.  512 sub-grids 0.836 -> 0.767 ms,
+// 32,768 47.7 -> 43.7 (the cooperative kernel with the plus-states in tensor
+// memory and one CTA per SM: 1.15 and 69.2; as two groups of a CTA 0.87, 48.8).
 //
 // The row sweep reads the FP32 primitives of its windows (prims_mixed of
 // the FP64 state) from a buffer that the producer of each state fills, once
-// per cell: a pass over X's interiors before stage 0 (with one more grid
-// barrier), the U1 writes and the stage-1 stores.  The separate launches
+// per cell: the pass over X's interiors, the U1 writes and the stage-1
+// stores.  The separate launches
 // recover them in every padded cell of every window, from the same FP64
 // values, so the bits are the same; the conversions and the dual-energy
 // recovery in FP64 drop from 2,744 to 512 per sub-grid and stage.
@@ -55,8 +60,8 @@ struct FusedArgs {
   double* Y;            // padded output state (interiors written)
   double* U2;           // [n][F][N3] second-stage state
   double* dt_out;       // the step's dt
-  unsigned* sync;       // zero at launch: [0] barrier arrivals, [1] work counter, [2] abort,
-                        // [kSyncHead + s] U2 of sub-grid s published, [kSyncHead + n + s] its U1
+  unsigned* sync;       // zero at launch: [0] work counter, [1] abort,
+                        // [kSyncHead + s] U2 tiles of sub-grid s published
   int nbx, nby, nbz, bc;
   double cfl, eta2, inv_gamma;
   double alpha[3], beta[3];  // the stage coefficients of the update kernel
@@ -65,7 +70,7 @@ struct FusedArgs {
                         // [n][F/2][NN^3] each: P[0] holds X's, then U2's; P[1]
                         // holds U1's
 };
-constexpr int kSyncHead = 4;
+constexpr int kSyncHead = 2;
 
 // Where the state of a tile (an 8^3 sub-grid, or an octant of a 16^3 one:
 // Tile) comes from, per stage (see above).
@@ -227,12 +232,16 @@ struct RowBody {
   float2* Qf;
   float* red;
   double* D;
+  RowPlusTmem plus;  // held until the kernel returns
   __device__ RowBody(const StepArgs64& S, unsigned char* sm)
       : R(row_map(threadIdx.x)), Qf(reinterpret_cast<float2*>(sm)), red(reinterpret_cast<float*>(sm + kRed)),
-        D(S.scratch + (size_t)blockIdx.x * kScratchPerSub) {}
+        D(S.scratch + (size_t)blockIdx.x * kScratchPerSub) {
+    __shared__ uint32_t sh_tm;
+    plus.t = tmem_alloc(&sh_tm);
+  }
+  __device__ ~RowBody() { tmem_free(plus.t); }
   template <class Io>
   __device__ __forceinline__ void run(const StepArgs64& S, const Io& io, int s) const {
-    RowPlusLocal plus;  // (not in tensor memory: hydro_tmem.cuh)
     mixed_subgrid<kGate, kContact, kSpin>(S, io, s, R, Qf, red, D, plus);
   }
 };
@@ -250,83 +259,57 @@ struct PlaneBody {
   }
 };
 
-template <class Body, int NN>
-__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fused_kernel(FusedArgs A) {
+// The primitives of X's interiors, once per cell.
+constexpr int kThreadsCell = 256;
+template <int NN>
+__global__ void __launch_bounds__(kThreadsCell) hydro_rk3_prims_kernel(FusedArgs A) {
   using T = Tile<NN>;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ double dred[Body::kThreads / 32];
-  __shared__ int sh_unit, sh_ok;
-  const int tid = threadIdx.x;
-  const int n = A.S.n_sub;
-  const int units = n * T::kTiles;  // work units: tiles
-  const Body body(A.S, smem_raw);
-  unsigned* arrive = A.sync;
-  unsigned* counter = A.sync + 1;
-  unsigned* abort = A.sync + 2;
-  unsigned* published = A.sync + kSyncHead;    // U2 tiles done, per sub-grid
-  unsigned* published1 = published + n;        // U1 tiles done, per sub-grid
-
-  using Io = FusedIo<NN>;
-  // grid-wide barrier number k (1, 2, ...): every CTA arrives once per barrier
-  auto grid_sync = [&](unsigned k) {
-    if (tid == 0) {
-      __threadfence();
-      atomicAdd(arrive, 1u);
-      const bool ok = wait_geq(arrive, k * gridDim.x, abort, A.wait_ns);
-      if (!ok) {
-        atomicOr(A.S.status, 2u);
-        atomicExch(abort, 1u);
-      }
-      sh_ok = ok;
-    }
-    __syncthreads();
-    return sh_ok != 0;
-  };
-  unsigned barriers = 0;
-
-  // ---- the primitives of X's interiors, once per cell ---------------------
-  {
-    for (int u = blockIdx.x; u < units; u += gridDim.x) {
-      const T t(u);
-      const double* __restrict__ x = A.S.U + (size_t)t.s * F * T::kS3;
-      for (int c = tid; c < N3; c += Body::kThreads) {
-        const int uc = t.pad((((c >> 6) + G) * S + (((c >> 3) & (N - 1)) + G)) * S + ((c & (N - 1)) + G));
-        double xv[F];
+  for (int u = blockIdx.x; u < A.S.n_sub * T::kTiles; u += gridDim.x) {
+    const T t(u);
+    const double* __restrict__ x = A.S.U + (size_t)t.s * F * T::kS3;
+    for (int c = threadIdx.x; c < N3; c += kThreadsCell) {
+      const int uc = t.pad((((c >> 6) + G) * S + (((c >> 3) & (N - 1)) + G)) * S + ((c & (N - 1)) + G));
+      double xv[F];
 #pragma unroll
-        for (int k = 0; k < F; ++k) xv[k] = __ldg(x + (size_t)k * T::kS3 + uc);
-        store_prims(A, A.P[0], t.s, t.cell(c), xv, T::kN3);
-      }
+      for (int k = 0; k < F; ++k) xv[k] = __ldg(x + (size_t)k * T::kS3 + uc);
+      store_prims(A, A.P[0], t.s, t.cell(c), xv, T::kN3);
     }
-    if (!grid_sync(++barriers)) return;
   }
+}
 
-  // ---- stage 0 --------------------------------------------------------
-  {
-    const Io io{A, 0, 0.0};
-    for (int u = blockIdx.x; u < units; u += gridDim.x) body.run(A.S, io, u);
-  }
+// Stage 0: dU0 = L(X), amax.
+template <class Body, int NN>
+__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_stage0_kernel(FusedArgs A) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const Body body(A.S, smem_raw);
+  const FusedIo<NN> io{A, 0, 0.0};
+  for (int u = blockIdx.x; u < A.S.n_sub * Tile<NN>::kTiles; u += gridDim.x) body.run(A.S, io, u);
+}
 
-  // ---- grid-wide barrier, then dt (the reduction of hydro_dt_kernel) ----
-  if (!grid_sync(++barriers)) return;
+// dt (the reduction of hydro_dt_kernel, by every CTA), then U1 = X + dt dU0
+// into the interiors of Y, with its primitives.
+template <int NN>
+__global__ void __launch_bounds__(kThreadsCell) hydro_rk3_first_kernel(FusedArgs A) {
+  using T = Tile<NN>;
+  __shared__ double dred[kThreadsCell / 32];
+  const int tid = threadIdx.x;
   double m = INFINITY;
-  for (int i = tid; i < n; i += Body::kThreads) m = fmin(m, A.S.h[i] / __ldcg(A.S.amax + i));
+  for (int i = tid; i < A.S.n_sub; i += kThreadsCell) m = fmin(m, A.S.h[i] / A.S.amax[i]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((tid & 31) == 0) dred[tid >> 5] = m;
   __syncthreads();
   m = dred[0];
 #pragma unroll
-  for (int w = 1; w < Body::kThreads / 32; ++w) m = fmin(m, dred[w]);
+  for (int w = 1; w < kThreadsCell / 32; ++w) m = fmin(m, dred[w]);
   const double dt = A.cfl * m;
   if (blockIdx.x == 0 && tid == 0) *A.dt_out = dt;
-
-  // ---- U1 of this CTA's stage-0 tiles, into the interiors of Y ---------
-  for (int u = blockIdx.x; u < units; u += gridDim.x) {
+  for (int u = blockIdx.x; u < A.S.n_sub * T::kTiles; u += gridDim.x) {
     const T t(u);
     const double* __restrict__ x = A.S.U + (size_t)t.s * F * T::kS3;
     const double* r = A.S.dUdt + (size_t)t.s * F * T::kN3;
     double* y = A.Y + (size_t)t.s * F * T::kS3;
-    for (int c = tid; c < N3; c += Body::kThreads) {
+    for (int c = tid; c < N3; c += kThreadsCell) {
       const int uc = t.pad((((c >> 6) + G) * S + (((c >> 3) & (N - 1)) + G)) * S + ((c & (N - 1)) + G));
       const int ci = t.cell(c);
       double xv[F], rv[F], u1[F];
@@ -340,14 +323,22 @@ __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fu
       for (int k = 0; k < F; ++k) y[(size_t)k * T::kS3 + uc] = u1[k];
       store_prims(A, A.P[1], t.s, ci, u1, T::kN3);
     }
-    __syncthreads();
-    if (tid == 0) {
-      __threadfence();
-      atomicAdd(published1 + t.s, 1u);
-    }
   }
+}
 
-  // ---- stages 1 and 2 from one work counter ---------------------------
+// Stages 1 and 2 from one work counter, all stage-1 units first.
+template <class Body, int NN>
+__global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fused_kernel(FusedArgs A) {
+  using T = Tile<NN>;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ int sh_unit, sh_ok;
+  const int tid = threadIdx.x;
+  const int units = A.S.n_sub * T::kTiles;  // work units: tiles
+  const Body body(A.S, smem_raw);
+  unsigned* counter = A.sync;
+  unsigned* abort = A.sync + 1;
+  unsigned* published = A.sync + kSyncHead;  // U2 tiles done, per sub-grid
+  const double dt = __ldg(A.dt_out);
   for (;;) {
     if (tid == 0) {
       int u = (int)atomicAdd(counter, 1u);
@@ -360,8 +351,8 @@ __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fu
     const int stage = u < units ? 1 : 2;
     const int tu = stage == 1 ? u : u - units;
     const int s = tu / T::kTiles;
-    if (!wait_neighbours(A, stage == 1 ? published1 : published, s, (unsigned)T::kTiles, abort, &sh_ok)) break;
-    body.run(A.S, Io{A, stage, dt}, tu);  // ends with a barrier
+    if (stage == 2 && !wait_neighbours(A, published, s, (unsigned)T::kTiles, abort, &sh_ok)) break;
+    body.run(A.S, FusedIo<NN>{A, stage, dt}, tu);  // ends with a barrier
     if (stage == 1 && tid == 0) {
       __threadfence();
       atomicAdd(published + s, 1u);
@@ -373,65 +364,38 @@ __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_fu
 // indicator, with contact steepening, with both; the plane sweep plain and
 // with contact steepening (the indicator runs in the row sweep only).
 template <class Body, int NN>
-static cudaError_t fused_attr(int* per_sm) {
-  cudaError_t e = cudaFuncSetAttribute(hydro_rk3_fused_kernel<Body, NN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Body::kSmem);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, hydro_rk3_fused_kernel<Body, NN>, Body::kThreads,
-                                                      Body::kSmem);
-  return e;
+static cudaError_t fused_attr() {
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  const cudaError_t e = cudaFuncSetAttribute(hydro_rk3_stage0_kernel<Body, NN>, at, (int)Body::kSmem);
+  return e == cudaSuccess ? cudaFuncSetAttribute(hydro_rk3_fused_kernel<Body, NN>, at, (int)Body::kSmem) : e;
 }
 
-// Opt in to the dynamic shared memory (once per device); the most CTAs of
-// the decomposition's kernels that can be resident at once (the cooperative
-// launch's limit).
+// Opt in to the dynamic shared memory (once per device); the persistent
+// launches' CTAs in the decomposition.
 template <int NN, bool kSpin = false>
 static cudaError_t prepare_fused_nn(int num_sms, int planes, int* max_grid) {
   static unsigned long long done = 0;
-  static int per_sm_dev[64][2];
-  cudaError_t e = once_per_device(&done, [] {
-    int dev = 0, p[6] = {0, 0, 0, 0, 0, 0};
-    cudaError_t r = cudaGetDevice(&dev);
-    if (r == cudaSuccess) r = fused_attr<RowBody<false, false, kSpin>, NN>(&p[0]);
-    if (r == cudaSuccess) r = fused_attr<RowBody<true, false, kSpin>, NN>(&p[1]);
-    if (r == cudaSuccess) r = fused_attr<RowBody<false, true, kSpin>, NN>(&p[2]);
-    if (r == cudaSuccess) r = fused_attr<PlaneBody<false, kSpin>, NN>(&p[3]);
-    if (r == cudaSuccess) r = fused_attr<PlaneBody<true, kSpin>, NN>(&p[4]);
-    if (r == cudaSuccess) r = fused_attr<RowBody<true, true, kSpin>, NN>(&p[5]);
-    if (r != cudaSuccess) return r;
-    int rows = p[0] < p[1] ? p[0] : p[1];
-    rows = rows < p[2] ? rows : p[2];
-    rows = rows < p[5] ? rows : p[5];
-    if (rows > 2) rows = 2;
-    int pl = p[3] < p[4] ? p[3] : p[4];
-    if (pl > 1) pl = 1;
-    if (rows < 1 || pl < 1) return cudaErrorInvalidConfiguration;
-    per_sm_dev[dev][0] = rows;
-    per_sm_dev[dev][1] = pl;
-    return cudaSuccess;
+  *max_grid = (planes ? PlaneBody<false, kSpin>::kMinBlocks : RowBody<false, false, kSpin>::kMinBlocks) * num_sms;
+  return once_per_device(&done, [] {
+    cudaError_t r = fused_attr<RowBody<false, false, kSpin>, NN>();
+    if (r == cudaSuccess) r = fused_attr<RowBody<true, false, kSpin>, NN>();
+    if (r == cudaSuccess) r = fused_attr<RowBody<false, true, kSpin>, NN>();
+    if (r == cudaSuccess) r = fused_attr<RowBody<true, true, kSpin>, NN>();
+    if (r == cudaSuccess) r = fused_attr<PlaneBody<false, kSpin>, NN>();
+    if (r == cudaSuccess) r = fused_attr<PlaneBody<true, kSpin>, NN>();
+    return r;
   });
-  if (e != cudaSuccess) return e;
-  int dev = 0;
-  e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  *max_grid = per_sm_dev[dev][planes ? 1 : 0] * num_sms;
-  return cudaSuccess;
 }
 
 template <class Body, int NN>
-static cudaError_t launch_fused(const FusedArgs& A, int max_grid, cudaStream_t st) {
+static cudaError_t launch_fused(const FusedArgs& A, int max_grid, int num_sms, cudaStream_t st) {
   const int units = A.S.n_sub * Tile<NN>::kTiles;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(units < max_grid ? units : max_grid));
-  cfg.blockDim = dim3(Body::kThreads);
-  cfg.dynamicSmemBytes = Body::kSmem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, hydro_rk3_fused_kernel<Body, NN>, A);
+  const int grid = units < max_grid ? units : max_grid, cells = units < 8 * num_sms ? units : 8 * num_sms;
+  hydro_rk3_prims_kernel<NN><<<cells, kThreadsCell, 0, st>>>(A);
+  hydro_rk3_stage0_kernel<Body, NN><<<grid, Body::kThreads, Body::kSmem, st>>>(A);
+  hydro_rk3_first_kernel<NN><<<cells, kThreadsCell, 0, st>>>(A);
+  hydro_rk3_fused_kernel<Body, NN><<<grid, Body::kThreads, Body::kSmem, st>>>(A);
+  return cudaGetLastError();
 }
 
 // One fused RK3 step of a mesh of NN^3 sub-grids; sync must hold
@@ -470,19 +434,19 @@ static cudaError_t launch_fused_nn(const StepArgs64& S, double* Y, double* U2, f
   }
   // a second plus 20 us per tile: far above any stage's duration
   A.wait_ns = 1000000000ll + 20000ll * (long long)S.n_sub * Tile<NN>::kTiles;
-  e = cudaMemsetAsync(sync, 0, ((size_t)kSyncHead + 2 * (size_t)S.n_sub) * sizeof(unsigned), st);
+  e = cudaMemsetAsync(sync, 0, ((size_t)kSyncHead + (size_t)S.n_sub) * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   if (Tile<NN>::kTiles > 1) {
     e = cudaMemsetAsync(S.amax, 0, (size_t)S.n_sub * sizeof(double), st);
     if (e != cudaSuccess) return e;
   }
   if (planes && !S.gate)
-    return S.P.contact ? launch_fused<PlaneBody<true, kSpin>, NN>(A, max_grid, st)
-                       : launch_fused<PlaneBody<false, kSpin>, NN>(A, max_grid, st);
-  if (S.gate && S.P.contact) return launch_fused<RowBody<true, true, kSpin>, NN>(A, max_grid, st);
-  if (S.gate) return launch_fused<RowBody<true, false, kSpin>, NN>(A, max_grid, st);
-  if (S.P.contact) return launch_fused<RowBody<false, true, kSpin>, NN>(A, max_grid, st);
-  return launch_fused<RowBody<false, false, kSpin>, NN>(A, max_grid, st);
+    return S.P.contact ? launch_fused<PlaneBody<true, kSpin>, NN>(A, max_grid, num_sms, st)
+                       : launch_fused<PlaneBody<false, kSpin>, NN>(A, max_grid, num_sms, st);
+  if (S.gate && S.P.contact) return launch_fused<RowBody<true, true, kSpin>, NN>(A, max_grid, num_sms, st);
+  if (S.gate) return launch_fused<RowBody<true, false, kSpin>, NN>(A, max_grid, num_sms, st);
+  if (S.P.contact) return launch_fused<RowBody<false, true, kSpin>, NN>(A, max_grid, num_sms, st);
+  return launch_fused<RowBody<false, false, kSpin>, NN>(A, max_grid, num_sms, st);
 }
 
 }  // namespace hyd

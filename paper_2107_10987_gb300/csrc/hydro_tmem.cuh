@@ -1,11 +1,12 @@
-// hydro_tmem.cuh -- where a row of the row sweep keeps its plus-states.
+// hydro_tmem.cuh -- tensor memory, where a row of the row sweep keeps its
+// plus-states.
 //
 // The sweep carries the nine plus-states of its row, 90 floats a thread, from
 // one cell to the next: too many for registers, and indexed by the loop over
-// the points.  As a local array (RowPlusLocal) they go to L2 and back (two CTAs'
+// the points.  As a local array they went to L2 and back (two CTAs'
 // 110 KB of primitives leave 26 KB of first-level cache, and 0.2 % of the reads
 // hit): 40 % of the kernel's L2 traffic and a latency in every point.  Tensor
-// memory (RowPlusTmem; 256 KB per SM, otherwise idle here) holds a 32-bit word
+// memory (256 KB per SM, otherwise idle here) holds a 32-bit word
 // per thread and column: a warp reads and writes the 32 lanes of its quarter
 // (warp index mod 4), the column is a register.  4,096 sub-grids: 2.06 ->
 // 1.84 ms.
@@ -16,11 +17,6 @@
 // The allocation waits where other work on the SM holds the columns, until
 // that work's CTA ends; a CTA of these kernels holds its own from start to end
 // and waits for none while it does.
-//
-// The fused step keeps the local array: a cooperative launch takes one CTA per
-// SM of a kernel that allocates tensor memory (512 sub-grids 1.15 ms against
-// 0.84 with two CTAs), and one CTA of two six-warp groups, each with its own
-// tiles, takes 0.87 (32,768 sub-grids 48.8 ms against 47.7).
 #pragma once
 #include "hydro_common.cuh"
 
@@ -53,8 +49,8 @@ __device__ __forceinline__ void tmem_free(uint32_t t) {
   if (threadIdx.x < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(t), "n"(kTmemCols));
 }
 
-// Record r of this thread; plus_next: the stores so far are visible to the reads
-// that follow.
+// Record r of this thread; next: the stores so far are visible to the reads that
+// follow.
 struct RowPlusTmem {
   uint32_t t;  // tmem_alloc's; the warp's threads call together, converged
   __device__ __forceinline__ void next() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -85,17 +81,4 @@ struct RowPlusTmem {
         : "memory");
   }
 };
-__device__ __forceinline__ void plus_next(RowPlusTmem& p) { p.next(); }
-__device__ __forceinline__ RowPlusTmem::Rec plus_record(const RowPlusTmem& p, int r) { return p.record(r); }
-__device__ __forceinline__ void plus_store(RowPlusTmem& p, int r, const float q[F]) { p.store(r, q); }
-
-// (an array and not a member of one: 40 registers of it spill otherwise)
-using RowPlusLocal = float[9][F];
-__device__ __forceinline__ void plus_next(RowPlusLocal&) {}
-__device__ __forceinline__ const float* plus_record(const RowPlusLocal& p, int r) { return p[r]; }
-__device__ __forceinline__ void plus_store(RowPlusLocal& p, int r, const float q[F]) {
-#pragma unroll
-  for (int k = 0; k < F; ++k) p[r][k] = q[k];
-}
-
 }  // namespace hyd

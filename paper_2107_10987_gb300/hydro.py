@@ -269,7 +269,7 @@ def make_rk3_desc(Ua, Ub, origin, h, nb, bc, dUdt, amax, dt, cfl=0.4, g=None, me
                   fused=False) -> RK3Desc:
     """Descriptor of one RK3 time step: of a uniform mesh of nb = (nbx, nby, nbz)
     sub-grids, or (mesh: an amr.AMRMesh, face_flux its work buffer) of an
-    adaptive mesh.  fused: the whole step as one persistent launch (uniform
+    adaptive mesh.  fused: the whole step as four launches (uniform
     mesh, mixed precision)."""
     nb = nb or (0, 0, 0)
     d = RK3Desc(make_batch(Ua, origin, h, g), _ptr(Ub), nb[0], nb[1], nb[2], bc, _ptr(dUdt), _ptr(amax), _ptr(dt),

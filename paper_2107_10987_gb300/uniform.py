@@ -22,7 +22,7 @@ class UniformRun:
         or tensor; N the context's sub-grid edge, 8 or 16, S = N + 6); origin
         [n][3]; h scalar or [n]; nb = (nbx, nby, nbz) or an int; g: optional
         [n][3][N][N][N] gravitational acceleration; fused:
-        each time step as one persistent launch (mixed precision; the ghost
+        each time step as four launches (mixed precision; the ghost
         layers of the state buffers are then not maintained)."""
         self.ctx = ctx
         self.nb = (nb, nb, nb) if isinstance(nb, int) else tuple(nb)
