@@ -172,17 +172,17 @@ class ClockSampler:
 ALGO = {"fp64_flops_per_subgrid_stage": 6565962.0, "bytes_per_subgrid_stage": 260520}
 # DRAM bytes per launch from ncu (dram__bytes_read.sum + dram__bytes_write.sum)
 # by form and workload: the hydro_step launch of each precision form, and the
-# fused RK3 step (three stages per launch).  Captures on the 256^3 polytrope
+# fused RK3 step (three stages in four launches).  Captures on the 256^3 polytrope
 # are taken on its 128^3 cut (4,096 sub-grids) and scaled by 8 (traffic
 # grows with the sub-grids processed).  None until captured for the current
 # kernel.
-# Sedov: the mean over the 42 (fused: 14) launches of one ncu launch list of
-# `--workload sedov --precision both --steps 3 --warmup 3`; polytrope: one
-# full capture at 128^3.
-TRAFFIC_PER_LAUNCH = {"fp64_sedov": 1503850831.0 + 1085510120.0, "mixed_sedov": 142870894.0 + 93039927.0,
-                      "fused_sedov": 342275310.0 + 444961573.0,
+# Sedov: the mean over the 42 (fused: 19) launches of one ncu launch list of
+# `--workload sedov --precision both --steps 3 --warmup 3`; polytrope: two
+# steps at 128^3.
+TRAFFIC_PER_LAUNCH = {"fp64_sedov": 1024.0e6 + 1050.5e6, "mixed_sedov": 131.0e6 + 48.5e6,
+                      "fused_sedov": 330.2e6 + 171.8e6,
                       "fp64_polytrope": None, "mixed_polytrope": None,
-                      "fused_polytrope": 8 * (3430653e3 + 3719836e3)}
+                      "fused_polytrope": 8 * (3003e6 + 2005e6)}
 
 
 def algorithmic_work():
@@ -697,7 +697,7 @@ def gpu_arm(args):
         head_fused = forms[head][1]
         flops = work["fp64_flops_per_subgrid_stage"] * n  # one stage of the mesh
         bytes_launch = work["bytes_per_subgrid_stage"] * n
-        # the timed kernel: the fused step does three stages per launch and
+        # the timed kernel: the fused step does three stages in one call and
         # reads the state once and writes the new state once (interiors)
         k_flops = 3 * flops if head_fused else flops
         k_bytes = 2 * n * 10 * N ** 3 * 8 if head_fused else bytes_launch
@@ -729,7 +729,9 @@ def gpu_arm(args):
                          "peak_source": ("FP32: 152 SMs x 128 lanes x 2 flops x 2070 MHz (profiling recipe units)"
                                          if not head.startswith("fp64") else "nominal GB300 FP64 from the profiling "
                                                                              "recipe"),
-                         "flops_counted": "algorithmic ops of the method (oracle count), each op one flop",
+                         "flops_counted": "algorithmic ops of the method (oracle count), each op one flop; the FP64 form "
+                                          "does the comparisons, minima, negations and halvings among them on the "
+                                          "integer pipes, so its fraction of the FP64 peak can pass 1",
                          "hbm_frac": (k_bytes / r["kern_s"] / 1e9) / pk["hbm_gbs"] if "hbm_gbs" in pk else None},
             "e2e": {"value": rate(r, "t_e2e"), "unit": UNIT,
                     "h2d_bytes_per_step": r["bytes_step"], "d2h_bytes_per_step": r["bytes_step"]},
