@@ -9,8 +9,8 @@
 // step kernel and the update, with the whole mesh finishing each launch
 // before the next starts.  Here, state X -> Y:
 //   prims    the primitives of X;
-//   stage 0  every sub-grid: dU0 = L(X), amax;
-//   first    dt = cfl min h/amax (every CTA); U1 = X + dt dU0 (with the tracer
+//   stage 0  every sub-grid: dU0 = L(X), amax and the least h/amax;
+//   first    dt = cfl min h/amax; U1 = X + dt dU0 (with the tracer
 //            resync) into the interiors of Y;
 //   fused    stage 1: sub-grid s reads U1 and writes U2 = 3/4 X + 1/4 (U1 + dt
 //            L(U1)) to an interior-only scratch and publishes it; stage 2:
@@ -30,20 +30,20 @@
 // the first three boundaries: a cooperative launch takes one CTA per SM of a
 // kernel that allocates tensor memory, where the row sweep keeps its
 // plus-states (hydro_tmem.cuh), and no CTA here waits for one that might not be
-// resident.  512 sub-grids 0.836 -> 0.767 ms,
-// 32,768 47.7 -> 43.7 (the cooperative kernel with the plus-states in tensor
-// memory and one CTA per SM: 1.15 and 69.2; as two groups of a CTA 0.87, 48.8).
+// resident.  512 sub-grids 0.836 -> 0.767 ms, 32,768 47.7 -> 43.7 (the
+// cooperative kernel with the plus-states in tensor memory and one CTA per SM:
+// 1.15 and 69.2; as two groups of a CTA 0.87, 48.8).
 //
 // The row sweep reads the FP32 primitives of its windows (prims_mixed of
 // the FP64 state) from a buffer that the producer of each state fills, once
 // per cell: the pass over X's interiors, the U1 writes and the stage-1
-// stores.  The separate launches
-// recover them in every padded cell of every window, from the same FP64
+// stores.  The separate launches recover them in every padded cell of every
+// window, from the same FP64
 // values, so the bits are the same; the conversions and the dual-energy
 // recovery in FP64 drop from 2,744 to 512 per sub-grid and stage.
 //
 // With 16^3 sub-grids a work unit is one of a sub-grid's eight 8^3 octant
-// tiles (Tile), and a sub-grid's U1 or U2 counts as published once all
+// tiles (Tile), and a sub-grid's U2 counts as published once all
 // eight tiles have added theirs to its flag.
 //
 // The per-cell arithmetic is the separate-launch step's own (the same
@@ -60,8 +60,9 @@ struct FusedArgs {
   double* Y;            // padded output state (interiors written)
   double* U2;           // [n][F][N3] second-stage state
   double* dt_out;       // the step's dt
-  unsigned* sync;       // zero at launch: [0] work counter, [1] abort,
-                        // [kSyncHead + s] U2 tiles of sub-grid s published
+  unsigned* sync;       // zero at launch: [0] work counter, [1] abort, [2-3] the
+                        // least h / amax (put_least), [kSyncHead + s] U2
+                        // tiles of sub-grid s published
   int nbx, nby, nbz, bc;
   double cfl, eta2, inv_gamma;
   double alpha[3], beta[3];  // the stage coefficients of the update kernel
@@ -70,7 +71,18 @@ struct FusedArgs {
                         // [n][F/2][NN^3] each: P[0] holds X's, then U2's; P[1]
                         // holds U1's
 };
-constexpr int kSyncHead = 2;
+constexpr int kSyncHead = 4;
+
+// The minimum of non-negative doubles, starting from infinity where the word
+// starts from zero: the greatest distance of their bits below infinity's.
+__device__ __forceinline__ void put_least(unsigned* word, double v) {
+  atomicMax(reinterpret_cast<unsigned long long*>(word),
+            0x7ff0000000000000ull - (unsigned long long)__double_as_longlong(v));
+}
+__device__ __forceinline__ double get_least(const unsigned* word) {
+  return __longlong_as_double(
+      (long long)(0x7ff0000000000000ull - *reinterpret_cast<const unsigned long long*>(word)));
+}
 
 // Where the state of a tile (an 8^3 sub-grid, or an octant of a 16^3 one:
 // Tile) comes from, per stage (see above).
@@ -179,8 +191,11 @@ struct FusedIo {
       for (int k = 0; k < F; ++k) o[(size_t)k * T::kS3] = un[k];
     }
   }
+  // (m is the maximum of a chain from zero that drops NaN: h / m is in [0, inf],
+  // and a sub-grid's least over its tiles is h over their maximum)
   __device__ __forceinline__ void amax(const Sub& q, double m) const {
     if (stage != 0) return;
+    put_least(A.sync + 2, A.S.h[q.t.s] / m);
     if (T::kTiles == 1)
       A.S.amax[q.t.s] = m;
     else
@@ -286,23 +301,16 @@ __global__ void __launch_bounds__(Body::kThreads, Body::kMinBlocks) hydro_rk3_st
   for (int u = blockIdx.x; u < A.S.n_sub * Tile<NN>::kTiles; u += gridDim.x) body.run(A.S, io, u);
 }
 
-// dt (the reduction of hydro_dt_kernel, by every CTA), then U1 = X + dt dU0
-// into the interiors of Y, with its primitives.
+// dt (hydro_dt_kernel's value), then U1 = X + dt dU0 into the interiors of Y,
+// with its primitives.  Stage 0 leaves the least h / amax: with every CTA
+// reducing the mesh's instead, its n divisions in FP64 per CTA took a third of
+// this kernel's 245 us at 4,096 sub-grids (a step of 512 sub-grids 0.767 -> 0.760
+// ms, of 32,768 43.7 -> 43.3).
 template <int NN>
 __global__ void __launch_bounds__(kThreadsCell) hydro_rk3_first_kernel(FusedArgs A) {
   using T = Tile<NN>;
-  __shared__ double dred[kThreadsCell / 32];
   const int tid = threadIdx.x;
-  double m = INFINITY;
-  for (int i = tid; i < A.S.n_sub; i += kThreadsCell) m = fmin(m, A.S.h[i] / A.S.amax[i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((tid & 31) == 0) dred[tid >> 5] = m;
-  __syncthreads();
-  m = dred[0];
-#pragma unroll
-  for (int w = 1; w < kThreadsCell / 32; ++w) m = fmin(m, dred[w]);
-  const double dt = A.cfl * m;
+  const double dt = A.cfl * get_least(A.sync + 2);
   if (blockIdx.x == 0 && tid == 0) *A.dt_out = dt;
   for (int u = blockIdx.x; u < A.S.n_sub * T::kTiles; u += gridDim.x) {
     const T t(u);

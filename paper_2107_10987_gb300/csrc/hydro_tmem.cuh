@@ -16,7 +16,7 @@
 // that share an SM both have theirs; no third fits beside their shared memory.
 // The allocation waits where other work on the SM holds the columns, until
 // that work's CTA ends; a CTA of these kernels holds its own from start to end
-// and waits for none while it does.
+// and waits at most for CTAs that hold theirs.
 #pragma once
 #include "hydro_common.cuh"
 
