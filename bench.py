@@ -176,13 +176,13 @@ ALGO = {"fp64_flops_per_subgrid_stage": 6565962.0, "bytes_per_subgrid_stage": 26
 # are taken on its 128^3 cut (4,096 sub-grids) and scaled by 8 (traffic
 # grows with the sub-grids processed).  None until captured for the current
 # kernel.
-# Sedov: the mean over the 42 (fused: 19) launches of one ncu launch list of
+# Sedov: the mean over the 42 (fused: 10) launches of one ncu launch list of
 # `--workload sedov --precision both --steps 3 --warmup 3`; polytrope: two
 # steps at 128^3.
 TRAFFIC_PER_LAUNCH = {"fp64_sedov": 1024.0e6 + 1050.5e6, "mixed_sedov": 131.0e6 + 48.5e6,
-                      "fused_sedov": 330.2e6 + 171.8e6,
+                      "fused_sedov": 328.6e6 + 171.6e6,
                       "fp64_polytrope": None, "mixed_polytrope": None,
-                      "fused_polytrope": 8 * (3003e6 + 2005e6)}
+                      "fused_polytrope": 8 * (3002e6 + 2010e6)}
 
 
 def algorithmic_work():
