@@ -238,7 +238,6 @@ __device__ __forceinline__ void mixed_subgrid(const StepArgs64& A, const Io& io,
         line10f(Qf, cj, sa + t1 * sb + t2 * sc, qpA, qmA);
         if (kTwo) line10f(Qf, cj, sa - t1 * sb - t2 * sc, qpB, qmB);
       }
-      if (kGate) __syncwarp();
       if constexpr (kSpin) {
         // the cell's spin fed back into the velocity at both ends of both
         // lines (spin_dv32; the plane sweep's values, bit for bit)

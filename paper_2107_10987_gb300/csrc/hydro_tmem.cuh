@@ -42,18 +42,28 @@ __device__ __forceinline__ uint32_t tmem_alloc(uint32_t* sh) {
   return *(volatile uint32_t*)sh + ((threadIdx.x & 96u) << 16) + (threadIdx.x >> 7) * kTmemThread;
 }
 
-// End of the CTA (all threads), t: what tmem_alloc returned.
+// End of the CTA (all threads), t: what tmem_alloc returned.  The fences order
+// every thread's accesses before the barrier and the deallocation after it.
 __device__ __forceinline__ void tmem_free(uint32_t t) {
+  __syncwarp();
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (threadIdx.x < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(t), "n"(kTmemCols));
 }
 
 // Record r of this thread; next: the stores so far are visible to the reads that
-// follow.
+// follow.  The warp's threads call together: each access is one instruction of
+// the whole warp, so each reconverges it first (the row sweep branches per
+// thread before them: the smooth cells' lines, the contact test, the spin's cap,
+// conversions outside FP32's normal range).
 struct RowPlusTmem {
-  uint32_t t;  // tmem_alloc's; the warp's threads call together, converged
-  __device__ __forceinline__ void next() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+  uint32_t t;  // tmem_alloc's
+  __device__ __forceinline__ void next() {
+    __syncwarp();
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  }
   struct Rec {
     float q[F];
     __device__ __forceinline__ operator const float*() const { return q; }
@@ -62,6 +72,7 @@ struct RowPlusTmem {
     static_assert(F == 10, "a record is 8 + 2 columns");
     Rec v;
     float* q = v.q;
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%10];\n\t"
         "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%8, %9}, [%11];\n\t"
@@ -73,6 +84,7 @@ struct RowPlusTmem {
     return v;
   }
   __device__ __forceinline__ void store(int r, const float q[F]) {
+    __syncwarp();
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%2, %3, %4, %5, %6, %7, %8, %9};\n\t"
         "tcgen05.st.sync.aligned.32x32b.x2.b32 [%1], {%10, %11};" ::"r"(t + F * r),
