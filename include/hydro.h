@@ -162,8 +162,10 @@ int hydro_set_mode(hydro_ctx_t* ctx, const hydro_mode_t* mode);
  * about the adjacent interior cell.
  * Scratch (context-owned, allocated on first need and kept): in mixed
  * precision 159,744 bytes of flux differences per persistent CTA; in FP64 mode
- * 2,936,704 bytes of line ends, face sums and primitives per team of CTAs
- * (446 MB for one CTA per SM on a 152-SM GPU).
+ * 2,936,704 bytes of line ends, face sums and primitives per 8^3 tile of the
+ * largest batch so far, for at most one tile per SM (446 MB on a 152-SM GPU).
+ * A batch no larger than an earlier one allocates nothing, so it may be
+ * captured.
  * Errors: EINVAL (NULL ctx/batch/pointers, n_sub < 0, misaligned U, dt < 0),
  * ENOMEM, ECUDA.
  * n_sub == 0 is a no-op. */

@@ -125,14 +125,16 @@ static int fp64_teams(const hydro_ctx* c, int units, int* T) {
   return units < most ? units : most;
 }
 
-// Its per-team buffers (2.94 MB each) and the teams' barrier words.
+// Its per-team buffers (2.94 MB each) and the teams' barrier words, enough for
+// every batch of up to `units` tiles: a smaller batch may make more teams, or
+// the first of more than one CTA, and may come in a stream capture.
 static int ensure_lines(hydro_ctx* c, int units) {
-  int T = 1;
-  const int teams = fp64_teams(c, units, &T);
-  int rc = ensure_buf(c, &c->lines, &c->lines_bytes, (size_t)teams * hyd::step_fp64_lines_per_team() * sizeof(double),
+  const int most = c->slots_tuned[0] > 0 ? c->slots_tuned[0] : c->num_sms;
+  const size_t teams = units < most ? units : most;
+  int rc = ensure_buf(c, &c->lines, &c->lines_bytes, teams * hyd::step_fp64_lines_per_team() * sizeof(double),
                       "cudaMalloc(FP64 line ends)");
-  if (rc || T == 1) return rc;
-  return ensure_buf(c, &c->sync, &c->sync_bytes, hyd::step_fp64_lines_sync_words(teams) * sizeof(unsigned),
+  if (rc || c->slots_tuned[0] > 0) return rc;
+  return ensure_buf(c, &c->sync, &c->sync_bytes, hyd::step_fp64_lines_sync_words(c->num_sms) * sizeof(unsigned),
                     "cudaMalloc(FP64 team barriers)");
 }
 
