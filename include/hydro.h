@@ -184,7 +184,8 @@ int hydro_step(hydro_ctx_t* ctx, const hydro_batch_t* B, double dt, double* dUdt
  *                        each of the 13 lines once per cell along its own
  *                        direction into a buffer, then sums the faces; where
  *                        the batch does not fill whole rounds of the SMs,
- *                        teams of CTAs share a sub-grid.
+ *                        teams of CTAs share a sub-grid (of the SMs that the
+ *                        stream has, where it owns part of the device).
  *   HYDRO_DECOMP_PLANES  mixed precision: the sub-grid swept plane by plane
  *                        along z by 640 threads (one CTA per SM), each of the
  *                        13 lines through a cell reconstructed once, the

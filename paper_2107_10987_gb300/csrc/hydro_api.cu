@@ -5,6 +5,8 @@
 #include <cstring>
 #include <new>
 
+#include <cuda.h>
+
 #include "hydro.h"
 #include "hydro_amr.cuh"
 #include "hydro_common.cuh"
@@ -117,11 +119,45 @@ static int step_slots(const hydro_ctx* c, int units) {
   return 2 * c->num_sms;
 }
 
-// The FP64 step's launch over `units` tiles: teams of *T CTAs each.  A grid
-// fixed by the caller or the autotuner is that many single CTAs.
-static int fp64_teams(const hydro_ctx* c, int units, int* T) {
-  *T = c->slots_tuned[0] > 0 ? 1 : hyd::step_fp64_choose_team(units, c->num_sms, c->mode.flux_points);
-  const int most = c->slots_tuned[0] > 0 ? c->slots_tuned[0] : c->num_sms / *T;
+// The SMs that a launch on st may have: the device's, or those of the stream's
+// green context.  0 if the driver does not say.
+static int stream_sms(const hydro_ctx* c, cudaStream_t st) {
+  typedef CUresult (*StreamGetCtx)(CUstream, CUcontext*, CUgreenCtx*);
+  typedef CUresult (*GreenResource)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+  auto entry = [](const char* name, unsigned version) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    return cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &found) == cudaSuccess &&
+                   found == cudaDriverEntryPointSuccess
+               ? f
+               : nullptr;
+  };
+  static const StreamGetCtx get_ctx = reinterpret_cast<StreamGetCtx>(entry("cuStreamGetCtx", 12050));
+  static const GreenResource get_res = reinterpret_cast<GreenResource>(entry("cuGreenCtxGetDevResource", 12040));
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  if (!get_ctx || !get_res || get_ctx(st, &ctx, &green) != CUDA_SUCCESS) return 0;
+  if (!green) return c->num_sms;
+  CUdevResource r;
+  return get_res(green, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS ? (int)r.sm.smCount : 0;
+}
+
+// The FP64 step's launch over `units` tiles on st: teams of *T CTAs each.  A
+// grid fixed by the caller or the autotuner is that many single CTAs.  The CTAs
+// of a team wait for one another, so teams are made of the SMs that the stream
+// has; where that is not known, of one CTA.
+static int fp64_teams(const hydro_ctx* c, int units, cudaStream_t st, int* T) {
+  int most = c->slots_tuned[0];
+  *T = 1;
+  if (most == 0) {
+    most = c->num_sms;
+    *T = hyd::step_fp64_choose_team(units, most, c->mode.flux_points);
+    if (*T > 1) {
+      const int sms = stream_sms(c, st);
+      if (sms < most) *T = sms > 0 ? hyd::step_fp64_choose_team(units, sms, c->mode.flux_points) : 1;
+      if (*T > 1) most = sms / *T;
+    }
+  }
   return units < most ? units : most;
 }
 
@@ -349,7 +385,7 @@ int hydro_step(hydro_ctx_t* c, const hydro_batch_t* B, double dt, double* dUdt, 
     rc = ensure_lines(c, units);
     if (rc) return rc;
     int T = 1;
-    const int teams = fp64_teams(c, units, &T);
+    const int teams = fp64_teams(c, units, st, &T);
     e = hyd::launch_step_fp64_lines(step_args(c, B, dUdt, amax, face_flux), teams, T,
                                     reinterpret_cast<unsigned*>(c->sync), c->N, st);
   }
