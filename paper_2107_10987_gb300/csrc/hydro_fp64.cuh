@@ -32,6 +32,11 @@ __device__ __forceinline__ double flip64(double x, bool neg) {
   return __longlong_as_double(r);
 }
 __device__ __forceinline__ long long min64(long long a, long long b) { return a < b ? a : b; }
+// The same on patterns that may reach beyond those of magnitudes (twice_mag of
+// an infinity or a NaN).
+__device__ __forceinline__ long long umin64(long long a, long long b) {
+  return (unsigned long long)a < (unsigned long long)b ? a : b;
+}
 
 __device__ __forceinline__ double max_nonneg(double x, double y) {
   const long long a = __double_as_longlong(x), b = __double_as_longlong(y);
@@ -40,7 +45,8 @@ __device__ __forceinline__ double max_nonneg(double x, double y) {
 
 // 2x for a finite double of magnitude pattern b, exactly: a normal one gains
 // one in the exponent field, a subnormal one (exponent field 0) doubles its
-// pattern, which carries into the exponent field where 2x is normal.
+// pattern, which carries into the exponent field where 2x is normal.  Of an
+// infinity or a NaN: a pattern above every magnitude's, as unsigned.
 __device__ __forceinline__ long long twice_mag(long long b) { return b < (1LL << 52) ? b + b : b + (1LL << 52); }
 
 // Half a magnitude as the FP64 product 0.5 x rounds it (to nearest, ties to
@@ -79,7 +85,7 @@ __device__ __forceinline__ double slope64(double a, double b) {
   if (signs_differ(a, b) || lo == 0LL) return 0.0;
   const unsigned ea = (unsigned)(ma >> 52), eb = (unsigned)(mb >> 52);
   if ((ea + eb < 972u || lo < (1LL << 52)) && nonpositive(rmul(a, b))) return 0.0;
-  return sign64(min64(twice_mag(lo), half_mag(mag64(radd(a, b)))), b);
+  return sign64(umin64(twice_mag(lo), half_mag(mag64(radd(a, b)))), b);
 }
 
 // PPM's interface value between two neighbouring samples of a line, taken from
@@ -121,13 +127,41 @@ __device__ __forceinline__ void ppm_steep_sides64(double s1, double s2, double s
 // reads |w| > 2|u| (m moves to s2 - 2u) and |u| > 2|w| (p moves to s2 + 2w):
 // magnitudes cut to twice the other's, on the bit patterns, and two FP64
 // additions where the tests and moves took twelve.  The limited values are
-// continuous where the tests switch.
+// continuous where the tests switch.  For the sides of ordinary tiles (WildTile).
 __device__ __forceinline__ void ppm_limit64(double s2, double u, double w, double& p, double& m) {
   const long long au = mag64(u), aw = mag64(w);
   const bool flat = signs_differ(u, w);
   const long long lu = flat ? 0LL : min64(au, twice_mag(aw)), lw = flat ? 0LL : min64(aw, twice_mag(au));
   p = radd(s2, sign64(lu, u));
   m = rsub(s2, sign64(lw, w));
+}
+
+// A tile with a primitive of 2^508 or above, an infinity or a NaN has its lines
+// by PPM's formula itself (ppm_call64): the formula's squares may overflow and its
+// comparisons fail, and a non-finite cell then shows in its neighbours' values
+// as the formula has it, which ppm_limit64's cuts would hide.  The test is on the
+// tile, where the primitives are formed, because a test in every limit costs
+// 2 % of the step (512 sub-grids 7.05 -> 7.23 ms a step of three).
+struct WildTile {
+  unsigned hi = 0;  // the greatest high word of the magnitudes seen
+  __device__ __forceinline__ void see(double x) { hi = max(hi, (unsigned)__double2hiint(x) & 0x7fffffffu); }
+  __device__ __forceinline__ bool wild() const { return hi >= (1023u + 508u) << 20; }
+};
+static __device__ __noinline__ double2 ppm_call64(double s0, double s1, double s2, double s3, double s4, double eta) {
+  const double sixth = 1.0 / 6.0;
+  const double d0 = rsub(s1, s0), d1 = rsub(s2, s1), d2 = rsub(s3, s2), d3 = rsub(s4, s3);
+  const double D0 = slope64(d0, d1), D1 = slope64(d1, d2), D2 = slope64(d2, d3);
+  double p = rsub(rmul(0.5, radd(s2, s3)), rmul(rsub(D2, D1), sixth));
+  double m = rsub(rmul(0.5, radd(s1, s2)), rmul(rsub(D1, D0), sixth));
+  if (eta > 0.0) ppm_steep64(s1, s3, D0, D2, eta, p, m);
+  if (rmul(rsub(p, s2), rsub(s2, m)) <= 0.0) return make_double2(s2, s2);
+  const double dq = rsub(p, m);
+  const double lhs = rmul(dq, rsub(s2, rmul(0.5, radd(p, m)))), rhs = rmul(rmul(dq, dq), sixth);
+  if (lhs > rhs)
+    m = rsub(rmul(3.0, s2), rmul(2.0, p));
+  else if (lhs < -rhs)
+    p = rsub(rmul(3.0, s2), rmul(2.0, m));
+  return make_double2(p, m);
 }
 
 // PPM on the five samples s0..s4 of one line: qp = value at the +d end of the
@@ -220,6 +254,27 @@ __device__ __forceinline__ void line10u(const double* __restrict__ Q, int c, int
       qp[k] = rsub(rmul(c7, radd(q[0], q[st])), rmul(c1, radd(q[-st], q[2 * st])));
       qm[k] = rsub(rmul(c7, radd(q[0], q[-st])), rmul(c1, radd(q[st], q[-2 * st])));
     }
+  }
+}
+
+// line10, line10c (contact) or line10u (smooth) of a wild tile.
+static __device__ __noinline__ void line10_wild(const double* __restrict__ Q, int c, int st, bool smooth, bool contact,
+                                                const StepParams& P, double qp[F], double qm[F]) {
+  const bool steep = contact && !smooth && contact_line64(Q, c, st, P);
+#pragma unroll 1
+  for (int k = 0; k < F; ++k) {
+    const double* q = Q + k * S3 + c;
+    const double s0 = q[-2 * st], s1 = q[-st], s2 = q[0], s3 = q[st], s4 = q[2 * st];
+    double2 v;
+    if (smooth && !(k == ZX || k == ZY || k == ZZ)) {
+      const double c7 = 7.0 / 12.0, c1 = 1.0 / 12.0;
+      v.x = rsub(rmul(c7, radd(s2, s3)), rmul(c1, radd(s1, s4)));
+      v.y = rsub(rmul(c7, radd(s2, s1)), rmul(c1, radd(s3, s0)));
+    } else {
+      v = ppm_call64(s0, s1, s2, s3, s4, steep && (k == RHO || k >= SP0) ? contact_eta64(s0, s1, s2, s3, s4) : 0.0);
+    }
+    qp[k] = v.x;
+    qm[k] = v.y;
   }
 }
 

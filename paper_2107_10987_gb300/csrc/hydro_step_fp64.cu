@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(kThreads64, 1) hydro_step_fp64_kernel(StepArgs
 
     // ---- 2. primitives in place ----------------------------------------
     bool bad = false;
+    WildTile seen;
     for (int c = tid; c < S3; c += kThreads64) {
       double w[EGAS + 1];
 #pragma unroll
@@ -115,9 +116,11 @@ __global__ void __launch_bounds__(kThreads64, 1) hydro_step_fp64_kernel(StepArgs
       bad |= !prims64(w, Q[TAU * S3 + c], A.P);
 #pragma unroll
       for (int k = SX; k <= EGAS; ++k) Q[k * S3 + c] = w[k];
+#pragma unroll
+      for (int k = 0; k < F; ++k) seen.see(k <= EGAS ? w[k] : Q[k * S3 + c]);
     }
     if (bad) atomicOr(A.status, 1u);
-    __syncthreads();
+    const bool wild = __syncthreads_or(seen.wild());
 
     // ---- 2b. learned smoothness indicator (gate_phase; features in FP32) ----
     if (kGate)
@@ -150,7 +153,21 @@ __global__ void __launch_bounds__(kThreads64, 1) hydro_step_fp64_kernel(StepArgs
       for (int p = A.P.face_points == 1 ? 4 : 0; p <= 4; ++p) {
         const int t1 = p / 3 - 1, t2 = p % 3 - 1;  // point p; its mirror 8-p has (-t1,-t2)
         double qpA[F], qmA[F], qpB[F], qmB[F];
-        if (kGate && smooth[cj]) {
+        if (wild) {
+          double e[2][F];
+          line10_wild(Q, cj, sa + t1 * sb + t2 * sc, kGate && smooth[cj], kContact, A.P, e[0], e[1]);
+#pragma unroll
+          for (int k = 0; k < F; ++k) {
+            qpA[k] = e[0][k];
+            qmA[k] = e[1][k];
+          }
+          if (p != 4) line10_wild(Q, cj, sa - t1 * sb - t2 * sc, kGate && smooth[cj], kContact, A.P, e[0], e[1]);
+#pragma unroll
+          for (int k = 0; k < F; ++k) {
+            qpB[k] = e[0][k];
+            qmB[k] = e[1][k];
+          }
+        } else if (kGate && smooth[cj]) {
           line10u(Q, cj, sa + t1 * sb + t2 * sc, qpA, qmA);
           if (p != 4) line10u(Q, cj, sa - t1 * sb - t2 * sc, qpB, qmB);
         } else if (kContact) {

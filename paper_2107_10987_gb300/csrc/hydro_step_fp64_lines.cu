@@ -267,6 +267,41 @@ __device__ __forceinline__ void line_run(const double* __restrict__ Q, const uin
   }
 }
 
+// line_run of a wild tile (WildTile), both field groups in one item, a cell at a
+// time from shared memory; out of line: the ordinary runs keep their registers.
+// Both ends of every cell are stored, also those of a ghost cell that are not
+// read, and a number at a time: st_sector in an out-of-line function stored its
+// first number and zeros.
+static __device__ __noinline__ void line_run_wild(const double* __restrict__ Q, const uint8_t* __restrict__ smooth,
+                                                  bool contact, const StepParams& P, double* __restrict__ R, uint32_t e,
+                                                  double k3h) {
+  const int c0 = (int)(e & 0xfffu), b0 = (int)((e >> 12) & 0x3ffu), n = (int)((e >> 22) & 0xfu);
+  const int dx = (int)((e >> 26) & 3u) - 1, dy = (int)((e >> 28) & 3u) - 1, dz = (int)(e >> 30) - 1;
+  const int sv = dx + S * dy + S * S * dz, bv = dx + (N + 2) * dy + (N + 2) * (N + 2) * dz;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    const int ci = c0 + i * sv;
+    double q[2][F], dv[3] = {0.0, 0.0, 0.0};
+    line10_wild(Q, ci, sv, smooth && smooth[ci], contact, P, q[0], q[1]);
+    if (P.spin)
+      spin_dv64(Q[RHO * S3 + ci], Q[EGAS * S3 + ci], Q[ZX * S3 + ci], Q[ZY * S3 + ci], Q[ZZ * S3 + ci], k3h,
+                rmul(P.gamma, P.gm1), dx, dy, dz, dv);
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+      const double* v = q[side];
+      double vel[3];
+#pragma unroll
+      for (int m = 0; m < 3; ++m)
+        vel[m] = P.spin ? (side ? rsub(v[SX + m], dv[m]) : radd(v[SX + m], dv[m])) : v[SX + m];
+      double* d = R + ((size_t)(2 * dir_index(dx, dy, dz) + side) * kBox + b0 + i * bv) * kRec;
+      const End64 w = end64(v[RHO], vel[0], vel[1], vel[2], v[EGAS], P);
+      const double rec[kRec] = {v[RHO], vel[0], vel[1], vel[2], w.p, w.E, w.c, v[TAU], v[ZX], v[ZY], v[ZZ], v[SP0]};
+#pragma unroll
+      for (int k = 0; k < kRec; ++k) d[k] = rec[k];
+    }
+  }
+}
+
 // Barrier of a team (T = 1: of the CTA): every thread's earlier writes are
 // visible to the team's threads after it.  k counts the team's barriers since
 // the launch; sync[0] is the launch's abort word, sync[32 (1 + team)] the
@@ -359,6 +394,7 @@ __global__ void __launch_bounds__(kLThreads, 1)
 
     // ---- 1. primitives ------------------------------------------------------
     bool bad = false;
+    WildTile seen;
     if (T == 1) {
       if (!mbar_wait_bounded(&bar, phase, kLWaitPolls)) {
         atomicOr(A.status, 2u);
@@ -374,6 +410,8 @@ __global__ void __launch_bounds__(kLThreads, 1)
         bad |= !prims64(w, Q[TAU * S3 + c], A.P);
 #pragma unroll
         for (int k = SX; k <= EGAS; ++k) Q[k * S3 + c] = w[k];
+#pragma unroll
+        for (int k = 0; k < F; ++k) seen.see(k <= EGAS ? w[k] : Q[k * S3 + c]);
       }
     } else {
       // the team converts each cell once; Pb was last read before the
@@ -392,10 +430,15 @@ __global__ void __launch_bounds__(kLThreads, 1)
       const double2* pb2 = reinterpret_cast<const double2*>(Pb);
       double2* q2 = reinterpret_cast<double2*>(Q);
 #pragma unroll 6
-      for (int c = tid; c < F * S3 / 2; c += kLThreads) q2[c] = __ldcg(pb2 + c);
+      for (int c = tid; c < F * S3 / 2; c += kLThreads) {
+        const double2 v = __ldcg(pb2 + c);
+        seen.see(v.x);
+        seen.see(v.y);
+        q2[c] = v;
+      }
     }
     if (bad) atomicOr(A.status, 1u);
-    __syncthreads();
+    const bool wild = __syncthreads_or(seen.wild());
 
     // ---- 2. learned smoothness indicator -----------------------------------
     if (kGate)
@@ -408,7 +451,9 @@ __global__ void __launch_bounds__(kLThreads, 1)
       const int n_items = 2 * n_runs;
 #pragma unroll 1
       for (int it = (rank + T * warp) * 32 + lane; it < n_items; it += T * kLThreads) {
-        if (it < n_runs)
+        if (wild) {
+          if (it < n_runs) line_run_wild(Q, kGate ? smooth : nullptr, kContact, A.P, R, g_line_runs[it], k3h);
+        } else if (it < n_runs)
           line_run<kGate, kContact, 6>(Q, smooth, A.P, R, g_line_runs[it], 0, k3h);
         else
           line_run<kGate, kContact, 4>(Q, smooth, A.P, R, g_line_runs[it - n_runs], 6, k3h);
