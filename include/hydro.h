@@ -434,6 +434,17 @@ int hydro_selftest_wait(hydro_ctx_t* ctx, double seconds, void* stream);
  * for.  Asynchronous.  Errors: EINVAL (n < 0, null pointers with n > 0). */
 int hydro_selftest_arith(const double* x, const double* y, int n, double* out, void* stream);
 
+/* Self-test of the step kernels' scalar helpers that stand for a division, a
+ * square root, a conversion or a comparison.  For i < n (device arrays x, y of n
+ * doubles, out of 5n doubles):
+ *   out[5i]     = x_i / y_i as the FP64 step forms velocities from momenta,
+ *   out[5i + 1] = 1 / sqrt(y_i) as its sound speeds take it,
+ *   out[5i + 2] = x_i rounded to FP32 by the mixed form's conversion,
+ *   out[5i + 3] = (float)x_i widened by the mixed form's conversion,
+ *   out[5i + 4] = whether x_i > eta y_i, as the dual-energy selections decide.
+ * Asynchronous.  Errors: EINVAL (n < 0, null pointers with n > 0). */
+int hydro_selftest_scalar(const double* x, const double* y, double eta, int n, double* out, void* stream);
+
 /* Which buffer holds the current state: 0 = a, 1 = b. */
 int hydro_rk3_graph_state(const hydro_graph_t* g);
 

@@ -293,15 +293,40 @@ __device__ __forceinline__ double rsqrt64(double x) {
 // The primitives of one cell from its conserved rho, s, E in u (v and eps in
 // place) and the tracer; false for a non-physical cell.  The three quotients
 // by rho from one reciprocal, each with Markstein's correction (the remainder
-// s - q rho, exact in a fused step, times 1/rho), which rounds them correctly.
+// s - q rho, exact in a fused step, times 1/rho): the division's bits wherever
+// the reciprocal, the quotient and the remainder neither overflow nor
+// underflow, as with rho in [2^-500, 2^500) and |s| in [2^-520, 2^520) or zero
+// (compared over 1.4e7 quotients as near to a rounding boundary as they get).
+// Elsewhere, and for rho <= 0, infinities and NaN, the division.
+static __device__ __noinline__ double div_call(double a, double b) { return a / b; }
 __device__ __forceinline__ bool prims64(double u[EGAS + 1], double tau, const StepParams& P) {
   const double rho = u[RHO];
-  const double ri = __drcp_rn(rho);
-  double v[3];
+  bool fast = (unsigned)__double2hiint(rho) - ((1023u - 500u) << 20) < 1000u << 20;
+  bool zero[3];
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
-    const double q = rmul(u[SX + m], ri);
-    v[m] = fma(fma(-q, rho, u[SX + m]), ri, q);
+    const unsigned hs = (unsigned)__double2hiint(u[SX + m]) & 0x7fffffffu;
+    zero[m] = (hs | (unsigned)__double2loint(u[SX + m])) == 0u;
+    fast &= zero[m] | (hs - ((1023u - 520u) << 20) < 1040u << 20);
+  }
+  double v[3];
+  if (fast) {
+    const double ri = __drcp_rn(rho);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      const double q = rmul(u[SX + m], ri);
+      v[m] = zero[m] ? u[SX + m] : fma(fma(-q, rho, u[SX + m]), ri, q);  // a zero keeps its sign
+    }
+  } else {
+#pragma unroll 1
+    for (int m = 0; m < 3; ++m) {
+      const double q = div_call(u[SX], rho);  // (the three in turn, without an index)
+      u[SX] = u[SY];
+      u[SY] = u[SZ];
+      u[SZ] = q;
+    }
+#pragma unroll
+    for (int m = 0; m < 3; ++m) v[m] = u[SX + m];
   }
   const double E = u[EGAS];
   const double ek = rmul(half64(rho), radd(radd(rmul(v[0], v[0]), rmul(v[1], v[1])), rmul(v[2], v[2])));

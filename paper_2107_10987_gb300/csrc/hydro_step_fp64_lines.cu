@@ -742,6 +742,21 @@ __global__ void selftest_arith_kernel(const double* __restrict__ x, const double
   }
 }
 
+__global__ void selftest_scalar_kernel(const double* __restrict__ x, const double* __restrict__ y, double eta, int n,
+                                       double* __restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double a = x[i], b = y[i];
+    double u[EGAS + 1] = {b, a, 0.0, 0.0, 1.0};
+    const StepParams P = {};
+    prims64(u, 1.0, P);
+    out[5 * i + 0] = u[SX];
+    out[5 * i + 1] = rsqrt64(b);
+    out[5 * i + 2] = (double)narrow(a);
+    out[5 * i + 3] = widen((float)a);
+    out[5 * i + 4] = above(a, narrow(a), eta, b, narrow(b)) ? 1.0 : 0.0;
+  }
+}
+
 }  // namespace hyd
 
 extern "C" int hydro_selftest_arith(const double* x, const double* y, int n, double* out, void* stream) {
@@ -749,5 +764,13 @@ extern "C" int hydro_selftest_arith(const double* x, const double* y, int n, dou
   if (n == 0) return HYDRO_OK;
   const int grid = (n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024;
   hyd::selftest_arith_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(x, y, n, out);
+  return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
+}
+
+extern "C" int hydro_selftest_scalar(const double* x, const double* y, double eta, int n, double* out, void* stream) {
+  if (n < 0 || (n > 0 && (!x || !y || !out))) return HYDRO_EINVAL;
+  if (n == 0) return HYDRO_OK;
+  const int grid = (n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024;
+  hyd::selftest_scalar_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(x, y, eta, n, out);
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
 }

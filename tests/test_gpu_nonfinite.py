@@ -81,3 +81,40 @@ def test_nan(field, value):
     for how, dU, am in _steps(_state(field, value), 0.0):
         assert np.array_equal(np.isnan(dU[0]), block), how
         assert np.isfinite(dU[0][~block]).all() and np.isfinite(am).all(), how
+
+
+@pytest.mark.parametrize("rho", [1e-308, 1e-300, 1e300, 1.7e308])
+@pytest.mark.parametrize("speed", [0.0, 0.5])
+def test_extreme_densities(rho, speed):
+    U = _state(0, rho)
+    U[(0, slice(1, 4)) + CELL] = 0.0
+    U[(0, 1) + CELL] = speed * rho
+    _check(U)
+
+
+@pytest.mark.parametrize("rho", [1e-309, 5e-324])
+def test_densities_below_the_reciprocals_range(rho):
+    """The reciprocal overflows, the quotients do not: dU/dt and amax stay finite,
+    and the oracle's values wherever its sound speed, a root of an
+    overflowing quotient, is finite."""
+    U = _state(0, rho)
+    U[(0, slice(1, 4)) + CELL] = 0.0
+    with np.errstate(all="ignore"):
+        want, _, _ = orc.step(orc.OracleParams(gamma=GAMMA, omega=0.2), U, np.zeros((1, 3)), np.array([H_CELL]))
+    fin = np.isfinite(want)
+    for how, dU, am in _steps(U, 0.2):
+        assert np.isfinite(dU).all() and 1e150 < am[0] < np.inf, how
+        assert (np.abs(dU - want)[fin] <= 1e-12 * np.abs(want[fin]).max()).all(), how
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf])
+def test_infinite_momentum_shows_in_amax(value):
+    U = _state(1, value)
+    with np.errstate(all="ignore"):
+        want, wam, _ = orc.step(orc.OracleParams(gamma=GAMMA, omega=0.2), U, np.zeros((1, 3)), np.array([H_CELL]))
+    fin = np.isfinite(want)
+    assert wam[0] == np.inf
+    for how, dU, am in _steps(U, 0.2):
+        assert am[0] == np.inf, how
+        assert np.isfinite(dU[fin]).all(), how  # nothing but what the oracle has
+        assert (np.abs(dU[fin] - want[fin]) <= 1e-12 * np.abs(want[fin]).max()).all(), how
