@@ -192,8 +192,9 @@ int hydro_step(hydro_ctx_t* ctx, const hydro_batch_t* B, double dt, double* dUdt
  *                        primitives in a ring of six planes that arrive
  *                        one step ahead.
  *   HYDRO_DECOMP_AUTO    the autotuner's choice, else by the number of 8^3
- *                        tiles: the plane sweep for at most one tile per SM,
- *                        the row sweep for more. */
+ *                        tiles: the plane sweep for at most one tile per SM
+ *                        with nine flux points per face, the row sweep for
+ *                        more and with one point. */
 #define HYDRO_DECOMP_AUTO 0
 #define HYDRO_DECOMP_ROWS 1
 #define HYDRO_DECOMP_PLANES 2

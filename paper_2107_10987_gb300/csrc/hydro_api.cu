@@ -99,14 +99,19 @@ static int ensure_buf(hydro_ctx* c, double** buf, size_t* have, size_t need, con
 // The sub-grid decomposition a step of this context over `units` tiles runs
 // (mixed precision; FP64 and the learned indicator have the row sweep): what
 // hydro_set_launch or the autotuner chose, else the plane sweep for a batch
-// of at most one tile per SM, the row sweep for more.  A tile alone on an SM
-// takes the plane sweep 94 us and the row sweep 109; two row-sweep tiles share
-// an SM in 150 (planes: 182 for the two; 200 tiles 147 against 181, 400 tiles
-// 240 against 273, 700 tiles 363 against 449).
+// of at most one tile per SM with nine points per face, the row sweep for the
+// others.  A tile alone on an SM takes the plane sweep 89 us and the row sweep
+// 105 (with contact steepening and spin feedback 97 and 134; a fused step of 64
+// tiles 255 and 320); two row-sweep tiles share an SM in 150 (planes: 182 for
+// the two; 200 tiles 147 against 181, 400 tiles 240 against 273, 700 tiles 363
+// against 449).  With one point per face the row sweep has 3 lines per cell
+// in place of 27 and takes 50 to 52 us at 1 to 152 tiles where the plane sweep
+// takes 62 to 64 (contact and spin 54 and 64; 16^3 sub-grids 53 and 65; fused
+// 157 and 169).
 static int eff_decomp(const hydro_ctx* c, int units) {
   if (c->mode.precision != HYDRO_PREC_MIXED || c->gate_on) return HYDRO_DECOMP_ROWS;
   if (c->decomp != HYDRO_DECOMP_AUTO) return c->decomp;
-  return units <= c->num_sms ? HYDRO_DECOMP_PLANES : HYDRO_DECOMP_ROWS;
+  return units <= c->num_sms && c->mode.flux_points != 1 ? HYDRO_DECOMP_PLANES : HYDRO_DECOMP_ROWS;
 }
 
 static int step_slots(const hydro_ctx* c, int units) {
