@@ -118,3 +118,30 @@ def test_infinite_momentum_shows_in_amax(value):
         assert am[0] == np.inf, how
         assert np.isfinite(dU[fin]).all(), how  # nothing but what the oracle has
         assert (np.abs(dU[fin] - want[fin]) <= 1e-12 * np.abs(want[fin]).max()).all(), how
+
+
+@pytest.mark.parametrize("sweep", ["rows", "planes"])
+@pytest.mark.parametrize("field", [1, 5, 6, 9])
+@pytest.mark.parametrize("value", [np.inf, -np.inf])
+def test_infinities_in_the_mixed_form(field, value, sweep):
+    """The same in FP32: the oracle's finite cells, their values to the mixed form's
+    rounding (about 1e-6 of a field's largest), and an infinite momentum in amax."""
+    from paper_2107_10987_gb300 import hydro as H
+    U = _state(field, value)
+    with np.errstate(all="ignore"):
+        want, wam, _ = orc.step(orc.OracleParams(gamma=GAMMA, omega=0.2), U, np.zeros((1, 3)), np.array([H_CELL]))
+    fin = np.isfinite(want)
+    ctx = H.Context(GAMMA, 0.2)
+    H.hydro_set_mode(ctx, H.HYDRO_PREC_MIXED)
+    H.hydro_set_launch(ctx, H.HYDRO_DECOMP_ROWS if sweep == "rows" else H.HYDRO_DECOMP_PLANES, 0)
+    dU = torch.zeros((1, 10, 8, 8, 8), dtype=torch.float64, device="cuda")
+    am = torch.zeros(1, dtype=torch.float64, device="cuda")
+    H.hydro_step(ctx, H.make_batch(torch.tensor(U, device="cuda"), torch.zeros((1, 3), dtype=torch.float64, device="cuda"),
+                                   torch.full((1,), H_CELL, dtype=torch.float64, device="cuda")), 0.0, dU, am)
+    torch.cuda.synchronize()
+    dU, am = dU.cpu().numpy(), am.cpu().numpy()
+    assert np.array_equal(np.isfinite(dU), fin)
+    for k in range(10):
+        f = fin[0, k]
+        assert np.abs(dU[0, k][f] - want[0, k][f]).max() <= 2e-5 * max(np.abs(want[0, k][f]).max(), 1.0), k
+    assert am[0] == wam[0] or abs(am[0] / wam[0] - 1.0) <= 1e-5
