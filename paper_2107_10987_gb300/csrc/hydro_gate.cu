@@ -303,6 +303,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) hydro_mlp_forward_kernel(const
         a[ks][2 * h + 1] = pack_bf16x2(v1.x, v1.y);
       }
     }
+    __syncwarp();  // the matrix instructions are the whole warp's, the loads above each lane's
     float acc[4][4];
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {

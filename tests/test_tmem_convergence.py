@@ -48,3 +48,12 @@ def test_no_other_file_touches_tensor_memory():
         if f.endswith((".cu", ".cuh")) and f != "hydro_tmem.cuh":
             with open(os.path.join(CSRC, f)) as s:
                 assert not re.search(r"asm[^;]*tcgen05", s.read()), f
+
+
+def test_predictions_reconverge_between_the_guarded_loads_and_the_matrix_instructions():
+    """mma.sync.aligned is an instruction of a whole warp too; the predictions'
+    loads are guarded per lane (the padding columns)."""
+    with open(os.path.join(CSRC, "hydro_gate.cu")) as f:
+        body = _body(re.sub(r"//[^\n]*", "", f.read()), "hydro_mlp_forward_kernel")
+    guard, sync, mma = body.find("if (c < kGateIn)"), body.find("__syncwarp();"), body.find("mma_bf16_16816(")
+    assert 0 <= guard < sync < mma
