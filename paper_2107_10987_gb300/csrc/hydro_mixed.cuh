@@ -24,21 +24,13 @@ __device__ __forceinline__ float slope32(float a, float b) {
   return (__fmul_rn(a, b) <= 0.f) ? 0.f : copysignf(m, b);
 }
 
-// PPM on one line in FP32 (branch-free form of the limiter).  kSteep: the
-// contact-steepening blend with weight eta before the fix-ups (as ppm64).
-template <bool kSteep = false>
-__device__ __forceinline__ void ppm32(float s0, float s1, float s2, float s3, float s4, float& qp, float& qm,
-                                      float eta = 0.f) {
+// PPM on one line in FP32 (branch-free form of the limiter).
+__device__ __forceinline__ void ppm32(float s0, float s1, float s2, float s3, float s4, float& qp, float& qm) {
   const float sixth = 1.f / 6.f;
   const float d0 = __fsub_rn(s1, s0), d1 = __fsub_rn(s2, s1), d2 = __fsub_rn(s3, s2), d3 = __fsub_rn(s4, s3);
   const float D0 = slope32(d0, d1), D1 = slope32(d1, d2), D2 = slope32(d2, d3);
   float p = __fmaf_rn(-sixth, __fsub_rn(D2, D1), __fmul_rn(0.5f, __fadd_rn(s2, s3)));
   float m = __fmaf_rn(-sixth, __fsub_rn(D1, D0), __fmul_rn(0.5f, __fadd_rn(s1, s2)));
-  if (kSteep) {
-    const float keep = __fsub_rn(1.f, eta);
-    p = __fmaf_rn(eta, __fmaf_rn(-0.5f, D2, s3), __fmul_rn(keep, p));
-    m = __fmaf_rn(eta, __fmaf_rn(0.5f, D0, s1), __fmul_rn(keep, m));
-  }
   const bool ext = __fmul_rn(__fsub_rn(p, s2), __fsub_rn(s2, m)) <= 0.f;
   const float dq = __fsub_rn(p, m);
   const float lhs = __fmul_rn(dq, __fmaf_rn(-0.5f, __fadd_rn(p, m), s2));
@@ -107,8 +99,8 @@ __device__ __forceinline__ void ppm_fix(float e, float lhs, float rhs, float s, 
 }
 
 // ppm32 on two lanes (two fields of a line, or two lines).  kSteep: the
-// contact-steepening blend with eta in no lane (0), in both (1), or in the
-// x (2) or y (3) lane alone.
+// contact-steepening blend with eta in no lane (0), or in the x (2) or y (3)
+// lane alone.
 template <int kSteep = 0>
 __device__ __forceinline__ void ppm32x2(float2 s0, float2 s1, float2 s2, float2 s3, float2 s4, float2& qp, float2& qm,
                                         float2 eta = make_float2(0.f, 0.f)) {
@@ -117,11 +109,6 @@ __device__ __forceinline__ void ppm32x2(float2 s0, float2 s1, float2 s2, float2 
   const float2 D0 = half_slope32x2(d0, d1), D1 = half_slope32x2(d1, d2), D2 = half_slope32x2(d2, d3);
   float2 p = fma2(mthird, sub2(D2, D1), mul2(half, add2(s2, s3)));
   float2 m = fma2(mthird, sub2(D1, D0), mul2(half, add2(s1, s2)));
-  if (kSteep == 1) {
-    const float2 keep = sub2(f2(1.f), eta);
-    p = fma2(eta, fma2(f2(-1.f), D2, s3), mul2(keep, p));
-    m = fma2(eta, fma2(f2(1.f), D0, s1), mul2(keep, m));
-  }
   if (kSteep == 2) {
     const float keep = __fsub_rn(1.f, eta.x);
     p.x = __fmaf_rn(eta.x, __fsub_rn(s3.x, D2.x), __fmul_rn(keep, p.x));
@@ -408,28 +395,6 @@ constexpr int kGateB1 = kGateH * kGateIn, kGateW2 = kGateB1 + kGateH, kGateB2 = 
               kGateW3 = kGateB2 + kGateH, kGateB3 = kGateW3 + kGateH;
 
 __device__ __forceinline__ float bf16r(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
-
-template <class W>
-__device__ __forceinline__ float gate_logit(const W& w, const float x[54]) {
-  float h1[kGateH];
-#pragma unroll
-  for (int j = 0; j < kGateH; ++j) {
-    float z = w(kGateH * kGateIn + j);
-#pragma unroll
-    for (int i = 0; i < kGateIn; ++i) z = fmaf(w(j * kGateIn + i), x[i], z);
-    h1[j] = fmaxf(z, 0.f);
-  }
-  const int o2 = kGateH * kGateIn + kGateH;
-  float out = w(o2 + kGateH * kGateH + kGateH + kGateH);
-#pragma unroll 4
-  for (int j = 0; j < kGateH; ++j) {
-    float z = w(o2 + kGateH * kGateH + j);
-#pragma unroll
-    for (int i = 0; i < kGateH; ++i) z = fmaf(w(o2 + j * kGateH + i), h1[i], z);
-    out = fmaf(w(o2 + kGateH * kGateH + kGateH + j), fmaxf(z, 0.f), out);
-  }
-  return out;
-}
 
 // The deployed (inference) form of the network: the inputs and the first
 // hidden layer rounded to BF16, products and sums in FP32 -- the arithmetic
