@@ -144,7 +144,8 @@ constexpr int kTile = 128;        // samples per partial of hydro_mlp_work_bytes
 constexpr int kMt = 64;           // samples per tile
 constexpr int kMThreads = 128;
 constexpr int kMStrX = 60, kMStrH = 36;
-constexpr int kGradCtas = 456;    // 3 resident CTAs (70 KB) on each of 152 SMs
+constexpr int kGradPerSm = 3;     // resident CTAs of the gradient (70 KB each)
+constexpr int kFwdPerSm = 4;      // and of the predictions
 
 // Network weights in shared memory, rows padded with zeros: W1 [32][kMStrX],
 // W2 [32][kMStrH], then b1, b2, w3 [32] each and b3.
@@ -263,9 +264,8 @@ __device__ __forceinline__ float mlp_head(const float* sm, const float* h2, int 
 // by reading X: features, labels and predictions of 512 sub-grids take 89 us,
 // with tiled FP32 multiply-adds 161, with a sample per thread 936.
 constexpr int kFwdThreads = 128;
-__global__ void __launch_bounds__(kFwdThreads, 4) hydro_mlp_forward_kernel(const float* __restrict__ params,
-                                                                           const float* __restrict__ X, int n,
-                                                                           bool vec, float* __restrict__ out) {
+__global__ void __launch_bounds__(kFwdThreads, kFwdPerSm) hydro_mlp_forward_kernel(
+    const float* __restrict__ params, const float* __restrict__ X, int n, bool vec, float* __restrict__ out) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   GateFrags f;
   gate_load_frags(params, lane, f);
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) hydro_mlp_forward_kernel(const
 // db2 and dw3 per lane of warp 3), so a CTA writes one partial
 // (kGateParams gradient entries, then the loss) at its end.
 constexpr int kGradSmem = MlpSmem::end + kGateH * kMStrH + kMt * kMStrX + 4 * kMt * kMStrH + 2 * kMt;  // floats
-__global__ void __launch_bounds__(kMThreads, 3) hydro_mlp_grad_kernel(const float* __restrict__ params,
+__global__ void __launch_bounds__(kMThreads, kGradPerSm) hydro_mlp_grad_kernel(const float* __restrict__ params,
                                                                       const float* __restrict__ X,
                                                                       const float* __restrict__ y, int n, bool vec,
                                                                       float w1, float w0, float inv_n,
@@ -561,6 +561,15 @@ __global__ void hydro_bf16_round_kernel(const float* in, float* out, int n) {
 
 size_t mlp_grad_smem() { return sizeof(float) * kGradSmem; }
 
+// SMs of the current device, at least 1 (the network's entry points have no context).
+static int device_sms() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 1;
+  return n;
+}
+
 }  // namespace hyd
 
 extern "C" {
@@ -587,7 +596,8 @@ int hydro_mlp_forward(const float* params, const float* X, int n, float* out, vo
   if (!params || n < 0 || (n > 0 && (!X || !out))) return HYDRO_EINVAL;
   if (n == 0) return HYDRO_OK;
   int blocks = (n - 1) / (16 * hyd::kFwdThreads / 32) + 1;
-  if (blocks > 608) blocks = 608;  // 4 resident CTAs on each of 152 SMs
+  const int most = hyd::kFwdPerSm * hyd::device_sms();
+  if (blocks > most) blocks = most;
   hyd::hydro_mlp_forward_kernel<<<blocks, hyd::kFwdThreads, 0, (cudaStream_t)stream>>>(
       params, X, n, ((uintptr_t)X & 7u) == 0, out);
   return cudaGetLastError() == cudaSuccess ? HYDRO_OK : HYDRO_ECUDA;
@@ -611,7 +621,8 @@ int hydro_mlp_loss_grad(const float* params, const float* X, const float* y, int
     return HYDRO_ECUDA;
   // one partial per CTA; the work buffer holds one per kTile samples
   int parts = (n - 1) / hyd::kTile + 1;
-  if (parts > hyd::kGradCtas) parts = hyd::kGradCtas;
+  const int most = hyd::kGradPerSm * hyd::device_sms();
+  if (parts > most) parts = most;
   cudaStream_t st = (cudaStream_t)stream;
   hyd::hydro_mlp_grad_kernel<<<parts, hyd::kMThreads, hyd::mlp_grad_smem(), st>>>(
       params, X, y, n, ((uintptr_t)X & 7u) == 0, w1, w0, 1.f / n, work);
