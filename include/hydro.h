@@ -221,7 +221,9 @@ int hydro_set_launch(hydro_ctx_t* ctx, int decomposition, int ctas);
 
 /* The launch shape the context's next step will use in its current
  * precision over a large batch: *decomposition (ROWS or PLANES) and *ctas
- * (either nullable). */
+ * (either nullable).  Setting it fixes it for small batches too, which the
+ * default gives another shape (the plane sweep, teams of CTAs in FP64):
+ * hydro_set_launch(ctx, HYDRO_DECOMP_AUTO, 0) brings the default back. */
 int hydro_get_launch(const hydro_ctx_t* ctx, int* decomposition, int* ctas);
 
 /* SSP-RK3 stage update of the interior cells (ghosts are not touched):

@@ -102,8 +102,8 @@ static int ensure_buf(hydro_ctx* c, double** buf, size_t* have, size_t need, con
 // of at most one tile per SM with nine points per face, the row sweep for the
 // others.  A tile alone on an SM takes the plane sweep 89 us and the row sweep
 // 105 (with contact steepening and spin feedback 97 and 134; a fused step of 64
-// tiles 255 and 320); two row-sweep tiles share an SM in 150 (planes: 182 for
-// the two; 200 tiles 147 against 181, 400 tiles 240 against 273, 700 tiles 363
+// tiles 255 and 320); two row-sweep tiles share an SM in 146 (planes: 182 for
+// the two; 200 tiles 142 against 181, 400 tiles 236 against 273, 700 tiles 363
 // against 449).  With one point per face the row sweep has 3 lines per cell
 // in place of 27 and takes 50 to 52 us at 1 to 152 tiles where the plane sweep
 // takes 62 to 64 (contact and spin 54 and 64; 16^3 sub-grids 53 and 65; fused

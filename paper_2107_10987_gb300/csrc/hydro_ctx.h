@@ -14,7 +14,7 @@ struct hydro_ctx {
   int device;
   int num_sms;
   int slots_tuned[2];    // persistent CTAs chosen by hydro_autotune_step or hydro_set_launch (0: default), [fp64, mixed]
-  int decomp;            // mixed-precision sub-grid decomposition, HYDRO_DECOMP_* (AUTO: planes)
+  int decomp;            // mixed-precision sub-grid decomposition, HYDRO_DECOMP_* (AUTO: by the batch, eff_decomp)
   unsigned* status;      // device word
   double* scratch;       // step scratch
   size_t scratch_bytes;
@@ -30,8 +30,8 @@ struct hydro_ctx {
   size_t u2_bytes;
   double* prims;         // fused RK3 step: 2 x [n_sub][F][N^3] FP32 primitives (float words)
   size_t prims_bytes;
-  double* sync;          // fused RK3 step: barrier, work counter and per-sub-grid flags; FP64 step: team
-                         // barriers (unsigned words, cleared by each launch that uses them)
+  double* sync;          // fused RK3 step: work counter, abort word, least h / amax and per-sub-grid flags; FP64
+                         // step: team barriers (unsigned words, cleared by each launch that uses them)
   size_t sync_bytes;
   double* amr_img;       // adaptive RK3 step: each leaf's restriction image [n_sub][F][(N/2)^3]
   size_t amr_img_bytes;
@@ -54,7 +54,7 @@ int hydro_ctx_prepare(hydro_ctx* c, int n_sub);
 // capture).
 int hydro_ctx_prepare_fused(hydro_ctx* c, int n_sub);
 // The adaptive RK3 sequence with direct neighbour reads: whether this
-// context's step takes it (mixed precision, 8^3 leaves, row sweep, no
+// context's step takes it (mixed precision, 8^3 leaves, either sweep, no
 // contact steepening or spin feedback), its image buffer for n_sub leaves
 // (allocated before a stream capture), its lean ghost fill, its step, and
 // its flux correction with the stage update.

@@ -12,7 +12,7 @@
 // The first update writes the second buffer, so the step's initial state X
 // is kept without a copy; the next step runs Y -> X.  Two graphs (X->Y and
 // Y->X) are instantiated and replayed alternately.
-// On an adaptive mesh in mixed precision (8^3 leaves, row sweep, no contact
+// On an adaptive mesh in mixed precision (8^3 leaves, no contact
 // steepening or spin feedback) the ghost fill is the lean one and the step
 // reads same-level and finer neighbours itself (hydro_step_mixed_amr.cu):
 // the same values, bit for bit, without copying them into ghost cells.

@@ -31,12 +31,12 @@
 // the integer pipes.
 //
 // What bounds it: the latency of its intervals with 20 warps and one tile per
-// SM (phase A alone 25 us of a tile's 95, the face fluxes 14, phase C 15, the
+// SM (phase A alone 25 us of a tile's 90, the face fluxes 14, phase C 15, the
 // conversion of a padded FP64 state 14, the first planes and the last finish
 // 25; measured with the others left out).  A row sweep with two tiles on the
-// SM overlaps them and takes 68 us a tile, but 109 for one alone, so the
+// SM overlaps them and takes 146 us for the two, but 105 for one alone, so the
 // dispatch gives this sweep the batches of at most one tile per SM (77 leaves
-// with contact steepening and spin: 173 -> 101 us).  Two fields of a line share
+// with contact steepening and spin: 173 -> 102 us).  Two fields of a line share
 // each packed instruction in phase A, and two fields of a point in phase B:
 // the records' float4 quarters are register pairs as they are loaded.  The
 // primitives live in a ring of six FP32 planes (the five planes a line of

@@ -84,8 +84,6 @@ __device__ __forceinline__ double get_least(const unsigned* word) {
       (long long)(0x7ff0000000000000ull - *reinterpret_cast<const unsigned long long*>(word)));
 }
 
-// Where the state of a tile (an 8^3 sub-grid, or an octant of a 16^3 one:
-// Tile) comes from, per stage (see above).
 // The FP32 primitives of one cell's state u (prims_mixed) into P at
 // compact cell ci of sub-grid s (NN^3 = n3 cells); a non-physical cell sets
 // the status bit.
@@ -97,9 +95,11 @@ __device__ __forceinline__ void store_prims(const FusedArgs& A, float2* P, int s
   for (int k = 0; k < F / 2; ++k) p[(size_t)k * n3] = make_float2(q[2 * k], q[2 * k + 1]);
 }
 
-// Both sweeps read the FP32 primitives of their windows from P (recovered
-// once per cell by the tile that produced the state) instead of recovering
-// them from the FP64 state of every padded cell.
+// Where the state of a tile (an 8^3 sub-grid, or an octant of a 16^3 one:
+// Tile) comes from and goes, per stage (see above).  Both sweeps read the
+// FP32 primitives of their windows from P (recovered once per cell by the tile
+// that produced the state) instead of recovering them from the FP64 state of
+// every padded cell.
 template <int NN>
 struct FusedIo {
   using T = Tile<NN>;

@@ -47,10 +47,10 @@
 // masks instead of |x| and -x, an interface value from both its sides at once,
 // line ends' sound speeds shared, unread ends of ghost cells left out, and the
 // flux in two fused steps per field.  A tile of random data takes a CTA 0.664
-// ms (about 1.09 before); the RK3 step of a 512-sub-grid blast 13.0 -> 7.0 ms.
+// ms (about 1.09 before); the RK3 step of a 512-sub-grid blast 13.0 -> 7.05 ms.
 // Teams serve the batches that do not fill whole rounds of the SMs
 // (step_fp64_choose_team): 512 tiles take pairs of CTAs 2.45 ms and single
-// ones 2.65, one tile takes the whole chip 0.08 ms and one CTA 0.66.
+// ones 2.62, one tile takes a team of 46 CTAs 0.081 ms and one CTA 0.647.
 #include <algorithm>
 #include <vector>
 
@@ -664,7 +664,14 @@ size_t step_fp64_lines_sync_words(int teams) { return 32 * (1 + (size_t)teams); 
 // chain of the longest line run and a face (kChainUs), plus the team's
 // barriers and copies (kTeamUs).  A batch that fills whole rounds of single
 // CTAs keeps T = 1; 512 tiles on 152 SMs take 3.4 rounds' work in 4 rounds
-// alone, and one tile alone leaves 151 SMs idle.
+// alone, and one tile alone leaves 151 SMs idle.  The three are the model's
+// weights and not times: a tile takes 647 us on one SM (with contact steepening
+// 960, and spin feedback 1,110), and the least that a team takes for one is 81
+// (118), so the estimates lie 15 to 70 % below the times, and no team has
+// more than 46 CTAs, where the shared work meets the chain.
+// Measured on 152 SMs, teams against single CTAs: 1 tile 81 against 647 us,
+// 8 tiles 84 and 647, 16 tiles 110 and 648, 38 tiles 204 and 650, 77 tiles 471
+// and 659, 512 tiles 2,454 and 2,618.
 int step_fp64_choose_team(int units, int num_sms, int face_points) {
   const double kTileUs = face_points == 1 ? 120.0 : 560.0, kChainUs = 12.0, kTeamUs = 12.0;
   int best = 1;
