@@ -300,19 +300,22 @@ __device__ __forceinline__ double rsqrt64(double x) {
 // by rho from one reciprocal, each with Markstein's correction (the remainder
 // s - q rho, exact in a fused step, times 1/rho): the division's bits wherever
 // the reciprocal, the quotient and the remainder neither overflow nor
-// underflow, as with rho in [2^-500, 2^500) and |s| in [2^-520, 2^520) or zero
+// underflow, as with rho in [2^-120, 2^120) and |s| in [2^-900, 2^900) or zero
 // (compared over 1.4e7 quotients as near to a rounding boundary as they get).
-// Elsewhere, and for rho <= 0, infinities and NaN, the division.
+// Elsewhere, and for rho <= 0, infinities and NaN, the division.  The range is
+// wide in s: ahead of a blast the momenta fall by many orders per cell, and with
+// those below 2^-520 divided a step of an early 512-sub-grid Sedov blast took
+// 7.35 ms in place of 7.19.
 static __device__ __noinline__ double div_call(double a, double b) { return a / b; }
 __device__ __forceinline__ bool prims64(double u[EGAS + 1], double tau, const StepParams& P) {
   const double rho = u[RHO];
-  bool fast = (unsigned)__double2hiint(rho) - ((1023u - 500u) << 20) < 1000u << 20;
+  bool fast = (unsigned)__double2hiint(rho) - ((1023u - 120u) << 20) < 240u << 20;
   bool zero[3];
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
     const unsigned hs = (unsigned)__double2hiint(u[SX + m]) & 0x7fffffffu;
     zero[m] = (hs | (unsigned)__double2loint(u[SX + m])) == 0u;
-    fast &= zero[m] | (hs - ((1023u - 520u) << 20) < 1040u << 20);
+    fast &= zero[m] | (hs - ((1023u - 900u) << 20) < 1800u << 20);
   }
   double v[3];
   if (fast) {

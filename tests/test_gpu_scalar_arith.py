@@ -46,7 +46,8 @@ def _near(values):
 
 def test_quotients():
     rng = np.random.default_rng(1)
-    edges = _near([2.0 ** e for e in (-1074, -1024, -1021, -969, -520, -500, -1, 0, 499, 500, 519, 520, 1021, 1023)])
+    edges = _near([2.0 ** e for e in (-1074, -1024, -1021, -969, -900, -520, -500, -120, -1, 0, 119, 120, 499, 500, 519, 520,
+                                   899, 900, 1021, 1023)])
     pairs = np.meshgrid(edges, edges)
     n = 300_000
     x = np.concatenate([pairs[0].ravel(), _random(rng, n, -1074, 1024), _random(rng, n, -30, 30)])
