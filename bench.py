@@ -176,13 +176,13 @@ ALGO = {"fp64_flops_per_subgrid_stage": 6565962.0, "bytes_per_subgrid_stage": 26
 # are taken on its 128^3 cut (4,096 sub-grids) and scaled by 8 (traffic
 # grows with the sub-grids processed).  None until captured for the current
 # kernel.
-# Sedov: the mean over the 42 (fused: 10) launches of one ncu launch list of
-# `--workload sedov --precision both --steps 3 --warmup 3`; polytrope: two
-# steps at 128^3.
-TRAFFIC_PER_LAUNCH = {"fp64_sedov": 1024.0e6 + 1050.5e6, "mixed_sedov": 131.0e6 + 48.5e6,
-                      "fused_sedov": 328.6e6 + 171.6e6,
+# Sedov: the mean over the 41 or 42 (fused: 10) launches of ncu launch lists of
+# `--workload sedov --steps 3 --warmup 3` (`--precision both`, fused: `mixed`);
+# polytrope: two steps at 128^3.
+TRAFFIC_PER_LAUNCH = {"fp64_sedov": 1026.5e6 + 1050.5e6, "mixed_sedov": 129.6e6 + 49.9e6,
+                      "fused_sedov": 328.6e6 + 172.5e6,
                       "fp64_polytrope": None, "mixed_polytrope": None,
-                      "fused_polytrope": 8 * (3002e6 + 2010e6)}
+                      "fused_polytrope": 8 * (2999e6 + 2023e6)}
 
 
 def algorithmic_work():
