@@ -283,15 +283,17 @@ static __device__ __noinline__ void line10_wild(const double* __restrict__ Q, in
   }
 }
 
-// 1 / sqrt(x) for x > 0 to about an ulp: the FP32 value y refined by one step of
-// Halley's third-order iteration, y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the
-// FP32 value's error of 2^-22 leaves 2^-63), five FP64 instructions.  Outside
-// FP32's normal range the library's function, in a call.
+// 1 / sqrt(x) for x > 0: the FP32 value y refined by one step of Halley's
+// third-order iteration, y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2 (the FP32
+// value's error of 2^-22 leaves 2^-64), five FP64 instructions.  y has 24 bits, so
+// y^2 is exact and e is rounded once: at most 0.501 ulp in all (4e6 values; the
+// library's function 0.508; with e from a rounded x y it was 0.997, rms 0.331
+// against 0.289).  Outside FP32's normal range the library's function, in a call.
 static __device__ __noinline__ double rsqrt_call(double x) { return rsqrt(x); }
 __device__ __forceinline__ double rsqrt64(double x) {
   if ((unsigned)__double2hiint(x) - 0x38100000u >= 0x0fd00000u) return rsqrt_call(x);
   const double y = widen(rsqrtf(narrow(x)));
-  const double e = fma(-rmul(x, y), y, 1.0);
+  const double e = fma(-x, rmul(y, y), 1.0);
   return fma(rmul(e, y), fma(0.375, e, 0.5), y);
 }
 
