@@ -20,7 +20,7 @@
 // FP64 staging buffer would not fit beside the FP32 primitives of two CTAs.
 //
 // What bounds it: the latency of a row's chain at 12 warps per SM (two tiles
-// in 150 us: issue slots 53 %, FMA pipe 41 %, ALU 38 %, FP64 pipe 26 % of the
+// in 146 us: issue slots 57 %, FMA pipe 41 %, ALU 45 %, FP64 pipe 27 % of the
 // cycles).  Of 1.83 ms for 4,096 sub-grids the sweep is 1.24 (measured with it
 // left out), the load and the finish about 0.19 each.  Two threads per row
 // (24 warps at 80 registers) take 2.34 ms, one line at a time instead of two
